@@ -317,40 +317,55 @@ __device__ __forceinline__ void warp_append(bool pred, int val, int *cnt, int *b
     if (pred) buf[base + __popc(mask & ((1u << lane) - 1u))] = val;
 }
 
-// Bounded grid barrier for a cooperative (co-resident) grid: one arrival
-// atomic per CTA on a counter; the last arrival resets it and releases the
-// next generation, which the other CTAs poll.  (Measured on GB300 with 152
-// CTAs: 2.4 us per barrier, against 3.0 us for per-CTA arrival flags polled
-// by one CTA.)  Every wait gives up after kWaitNs and sets ST_WAIT; returns
-// false when any CTA gave up (the kernel must then return).
+// A control word that was last written before the grid barrier the thread has
+// just passed (list sizes, flags): a plain load, which may be served by L1.
+// The barrier's acquire makes those writes visible to every thread of the CTA
+// and drops what L1 held before.  All 24 warps of an SM then share one L2
+// request; with ld.cg each of the grid's 3,648 warps sent its own to the one
+// L2 slice that holds the word.
+template <class T>
+__device__ __forceinline__ T lctl(const T *p) {
+    static_assert(sizeof(T) == 4 || sizeof(T) == 8, "control words");
+    T v;
+    if constexpr (sizeof(T) == 4) asm volatile("ld.global.b32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    else asm volatile("ld.global.b64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+    return v;
+}
+
+// Bounded grid barrier for a cooperative (co-resident) grid.  One word holds
+// the generation (high 16 bits) and the arrivals: the arrival's atomic
+// returns the generation to wait on, and the last CTA to arrive starts the
+// next generation with zero arrivals.  The CTA's earlier writes are released
+// by the arrival and the others' acquired by the poll, so no separate fence
+// stands on the path.  Every wait gives up after kWaitNs and sets ST_WAIT;
+// returns false when this CTA gave up or saw that another one did (the kernel
+// must then return; a CTA that had already passed sees the flag at its next
+// barrier, which can no longer complete).
 __device__ __forceinline__ bool grid_sync(Ctl *C) {
     __shared__ int ok;
     __syncthreads();
     if (threadIdx.x == 0) {
-        // one word holds the generation and the arrivals: the arrival's
-        // atomic returns the generation to wait on, and the last CTA to
-        // arrive starts the next generation with zero arrivals
-        __threadfence();
-        const unsigned old = atomicAdd(&C->bar_word, 1u);
+        int good = 1;
+        unsigned old;
+        asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(old) : "l"(&C->bar_word) : "memory");
         if ((old & 0xffffu) == gridDim.x - 1) {
-            __threadfence();
-            atomicAdd(&C->bar_word, 0x10000u - gridDim.x);
+            asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(&C->bar_word), "r"(0x10000u - gridDim.x)
+                         : "memory");
         } else {
-            const unsigned long long t0 = gtimer();
-            unsigned spins = 0;
-            while (((ld_acquire(&C->bar_word) ^ old) & 0xffff0000u) == 0) {
-                if ((++spins & 31u) == 0) {
-                    if (__ldcg(&C->status) & ST_WAIT) break;
-                    if (gtimer() - t0 > kWaitNs) {
+            unsigned long long t0 = 0;
+            for (unsigned spins = 1; ((ld_acquire(&C->bar_word) ^ old) & 0xffff0000u) == 0; ++spins) {
+                if ((spins & 63u) == 0) {
+                    if (t0 == 0) t0 = gtimer();
+                    if (__ldcg(&C->status) & ST_WAIT) good = 0;
+                    else if (gtimer() - t0 > kWaitNs) {
                         atomicOr(&C->status, ST_WAIT);
-                        break;
+                        good = 0;
                     }
+                    if (!good) break;
                 }
-                __nanosleep(20);
             }
         }
-        __threadfence();
-        ok = (__ldcg(&C->status) & ST_WAIT) == 0;
+        ok = good;
     }
     __syncthreads();
     return ok;
@@ -1548,8 +1563,8 @@ __device__ __forceinline__ bool vertex_ok(const Job &J, Ctl *C, int u, int n) {
         if (gtid == 0) {                                                      \
             const unsigned long long now_ = gtimer();                         \
             const long long dt_ = (long long)(now_ - tprev);                  \
-            ST[bucket] += dt_;                                                \
-            ST[S_BARRIERS] += 1;                                              \
+            s_stat[bucket] += dt_;                                            \
+            s_stat[S_BARRIERS] += 1;                                          \
             if (TR) {                                                         \
                 const int k_ = C->trace_n++;                                  \
                 if (k_ < G.trace_cap)                                         \
@@ -1566,7 +1581,7 @@ __device__ __forceinline__ bool vertex_ok(const Job &J, Ctl *C, int u, int n) {
         if (gtid == 0) {                                                      \
             const unsigned long long now_ = gtimer();                         \
             const long long dt_ = (long long)(now_ - tprev);                  \
-            ST[bucket] += dt_;                                                \
+            s_stat[bucket] += dt_;                                            \
             if (TR) {                                                         \
                 const int k_ = C->trace_n++;                                  \
                 if (k_ < G.trace_cap)                                         \
@@ -1605,33 +1620,37 @@ __global__ void __launch_bounds__(kBlock, 1) k_solve(DevGraph G, Job J) {
 
     // A sticky error (iteration cap, barrier wait) invalidates the state
     // until the next mf_solve, which clears it before launching.
-    if (__ldcg(&C->status) & ST_STICKY) return;
-    const unsigned stamp_base = __ldcg(&C->stamp_base) + 1u;
+    if (lctl(&C->status) & ST_STICKY) return;
+    const unsigned stamp_base = lctl(&C->stamp_base) + 1u;
     // JOB_AUTO: the policy kernel launched just before chose repair or
     // recompute and KERNELCYCLES
     int kind = J.kind, kc = J.kc, jmode = J.mode;
     bool pp_pick = true;   // a fixed job of a push-pull graph repairs by push-pull
     if (kind == JOB_AUTO) {
-        kind = lcg(&C->pol_kind);
-        kc = lcg(&C->pol_kc);
-        jmode = lcg(&C->pol_mode);
+        kind = lctl(&C->pol_kind);
+        kc = lctl(&C->pol_kc);
+        jmode = lctl(&C->pol_mode);
         pp_pick = jmode == MF_MODE_PUSH_PULL;
         if (pp_pick) jmode = MF_MODE_DATA_DRIVEN;   // the plain loop of push-pull's stage 2
     }
-    if (kind == JOB_REFRESH && lcg(&C->heights_exact)) return;
+    if (kind == JOB_REFRESH && lctl(&C->heights_exact)) return;
     const bool batch_job = kind == JOB_REPAIR || kind == JOB_RECOMPUTE;
-    const int kb = J.k_dev ? lcg(J.k_dev) : J.k;          // batch entries
-    const unsigned seq = __ldcg(&C->bseq) + 1u;           // this batch's stamp
+    const int kb = J.k_dev ? lctl(J.k_dev) : J.k;          // batch entries
+    const unsigned seq = lctl(&C->bseq) + 1u;           // this batch's stamp
+    // CTA 0's thread 0 keeps its counts and phase times in shared memory: a
+    // read-modify-write of the global words after every barrier kept CTA 0's
+    // first warp, and with it the whole grid, waiting for two L2 round trips
+    __shared__ long long s_stat[S_COUNT_MAX];
     if (gtid == 0) {
-        for (int i = 0; i < S_COUNT; ++i) ST[i] = 0;
-        ST[S_BATCH] = batch_job ? kb : 0;
+        for (int i = 0; i < S_COUNT; ++i) ST[i] = s_stat[i] = 0;
+        s_stat[S_BATCH] = batch_job ? kb : 0;
         C->t_start = gtimer();
         if (TR) C->trace_n = 0;
     }
 
     // Dynamic Push-Pull (Alg. 8) needs the exact cut of the previous state:
     // T = {h < n} can reach a sink, S = {h >= n} cannot
-    const bool pp = PP && J.pp && pp_pick && kind == JOB_REPAIR && G.part && lcg(&C->cut_exact);
+    const bool pp = PP && J.pp && pp_pick && kind == JOB_REPAIR && G.part && lctl(&C->cut_exact);
     if (pp)
         for (long long v0 = gtid; v0 < n; v0 += 4 * gthreads) {   // four heights in flight per thread
             int hv[4];
@@ -1663,9 +1682,10 @@ __global__ void __launch_bounds__(kBlock, 1) k_solve(DevGraph G, Job J) {
             if (bad) atomicOr(&C->batch_err, 1);
         }
         MF_SYNC(S_T_BATCH);
-        if (lcg(&C->batch_err)) {
+        if (lctl(&C->batch_err)) {
             grid_sync(C);
             if (gtid == 0) {
+                for (int i = 0; i < S_COUNT; ++i) ST[i] = s_stat[i];
                 atomicOr(&C->status, ST_EINVAL);
                 C->batch_err = 0;
                 C->bseq = seq;
@@ -1703,7 +1723,7 @@ __global__ void __launch_bounds__(kBlock, 1) k_solve(DevGraph G, Job J) {
         // leave that cut saturated and its capacity unchanged, so the flow
         // value stays the same and the state stays terminal (Sec. 4: only
         // changes on the cut's arcs can change the maximum).
-        fast = kind == JOB_REPAIR && lcg(&C->cut_exact) && !lcg(&C->inc_block);
+        fast = kind == JOB_REPAIR && lctl(&C->cut_exact) && !lctl(&C->inc_block);
         if (kind == JOB_REPAIR && !fast) {
             // flow above the new capacity goes back: the tail keeps it as
             // excess, the head becomes deficient (Alg. 5, lines 4-11; the
@@ -1878,7 +1898,7 @@ __global__ void __launch_bounds__(kBlock, 1) k_solve(DevGraph G, Job J) {
             if (lane == 0 && dsum) add_ll(&C->dacc[par], dsum);
             if (lane == 0 && rdeg) add_ll(&C->asum[0], rdeg);
         }
-        MF_SYNC_T(S_T_RESET, 0, 0, lcg(&C->qcnt[0]));
+        MF_SYNC_T(S_T_RESET, 0, 0, lctl(&C->qcnt[0]));
         // the flags of the next iteration: their last readers (the previous
         // iteration's exit test) are all past this barrier
         if (gtid == 0) C->ri_moved[par ^ 1] = 0;
@@ -1891,9 +1911,9 @@ __global__ void __launch_bounds__(kBlock, 1) k_solve(DevGraph G, Job J) {
         bool bottom_up = false;
         long long arcs_seen = 0;
         for (;;) {
-            const int cur = lcg(&C->qcnt[L % 3]);
+            const int cur = lctl(&C->qcnt[L % 3]);
             if (cur == 0) break;
-            const long long mf = lcg(&C->asum[L % 3]);
+            const long long mf = lctl(&C->asum[L % 3]);
             arcs_seen += mf;
             const bool dual = PP && stage == 1;   // push-pull: backward on T, forward on S
             // (the dual search of push-pull takes a smaller vertex share: its
@@ -2003,8 +2023,8 @@ __global__ void __launch_bounds__(kBlock, 1) k_solve(DevGraph G, Job J) {
                     }
                 }
                 MF_SYNC_T(S_T_BFS, L, 5, cur);
-                L = lcg(&C->solo_L);
-                arcs_seen = lcg(&C->solo_seen);
+                L = lctl(&C->solo_L);
+                arcs_seen = lctl(&C->solo_seen);
                 continue;
             }
             const int *F = (L & 1) ? G.qb1 : G.qb0;
@@ -2016,7 +2036,7 @@ __global__ void __launch_bounds__(kBlock, 1) k_solve(DevGraph G, Job J) {
                 C->qcnt[(L + 2) % 3] = 0;
                 C->ccnt[(L + 1) % 3] = 0;
                 C->asum[(L + 2) % 3] = 0;
-                if (bottom_up) ST[S_BU_LEVELS] += 1;
+                if (bottom_up) s_stat[S_BU_LEVELS] += 1;
             }
             Front FR{ncnt, NF, asum, 0x7fffffff, nullptr, s_bfs + (threadIdx.x >> 5) * kWq, 0, 0, wmark0};
             if (bottom_up) {
@@ -2055,7 +2075,7 @@ __global__ void __launch_bounds__(kBlock, 1) k_solve(DevGraph G, Job J) {
             }
             front_flush(G, FR, dual, K);
             MF_SYNC_T(S_T_BFS, L, bottom_up ? 2 : 0, cur);
-            const int nch = lcg(ccnt);
+            const int nch = lctl(ccnt);
             if (nch > 0) {
                 if (bottom_up) {
                     for (int c = gwarp; c < nch; c += nwarps) bfs_bottom_up_item(G, lcg(&G.cb[c]), dual, L, FR, K);
@@ -2098,11 +2118,11 @@ __global__ void __launch_bounds__(kBlock, 1) k_solve(DevGraph G, Job J) {
             }
             ++L;
         }
-        if (gtid == 0) ST[S_LEVELS] += L;
+        if (gtid == 0) s_stat[S_LEVELS] += L;
 
         // termination: no active vertex under the fresh BFS heights
-        const int nw = lcg(&C->wcnt);
-        const int nh = lcg(&C->hcnt);
+        const int nw = lctl(&C->wcnt);
+        const int nh = lctl(&C->hcnt);
         if (nw == 0 && nh == 0) {
             if (stage == 1) {
                 // Alg. 8: what neither search reached -- overflowing vertices
@@ -2120,7 +2140,7 @@ __global__ void __launch_bounds__(kBlock, 1) k_solve(DevGraph G, Job J) {
             if (gtid == 0) atomicOr(&C->status, ST_ITERS);
             break;
         }
-        if (lcg(&C->abort_loop)) {   // written before the height-init barrier
+        if (lctl(&C->abort_loop)) {   // written before the height-init barrier
             if (gtid == 0) atomicOr(&C->status, ST_TIME);
             break;
         }
@@ -2165,7 +2185,7 @@ __global__ void __launch_bounds__(kBlock, 1) k_solve(DevGraph G, Job J) {
                 }
                 C->hub_act[0] = C->hub_act[1] = 0;
                 C->hlc[0] = C->hlc[1] = 0;
-                ST[S_WL] += nhp;
+                s_stat[S_WL] += nhp;
             }
             // the data-driven and push-pull modes run PushRelabel from the
             // activation queue; the topology-driven mode in rounds
@@ -2207,11 +2227,11 @@ __global__ void __launch_bounds__(kBlock, 1) k_solve(DevGraph G, Job J) {
                 // first H3 (a later pass's first cycle has an H1 barrier)
                 if (pass > 0 && gtid == 0)
                     C->aq_head = C->aq_tail = C->aq_done = C->aq_over = C->aq_maxgen = C->aq_fin = 0;
-                const int nhc = lcg(&C->hccnt);
+                const int nhc = lctl(&C->hccnt);
                 const int hub_min = PP ? kMinHubCyclesPP : kMinHubCycles;
                 const int hub_cycles = kc > hub_min ? kc : hub_min;
                 for (int c = 0; c < hub_cycles; ++c) {
-                    if (gtid == 0) ST[S_HUB_CYCLES] += 1;
+                    if (gtid == 0) s_stat[S_HUB_CYCLES] += 1;
                     const bool fresh = c == 0 && pass == 0;   // H1 decided by the BFS heights
                     // H1: lowest residual neighbour of every unfinished hub; the
                     // warp that completes a hub's last item takes the hub's
@@ -2220,7 +2240,7 @@ __global__ void __launch_bounds__(kBlock, 1) k_solve(DevGraph G, Job J) {
                     // the cycle's items: all hub items in cycle 0, afterwards the
                     // items of the hubs still active after the previous cycle
                     const int2 *items = c == 0 ? G.hcl : ((c - 1) & 1 ? G.hlv1 : G.hlv0);
-                    const int nitems = c == 0 ? nhc : lcg(&C->hlc[(c - 1) & 1]);
+                    const int nitems = c == 0 ? nhc : lctl(&C->hlc[(c - 1) & 1]);
                     for (int w = fresh ? nitems : gwarp; w < nitems; w += nwarps) {
                         const int2 item = lcg(&items[w]);
                         const int i = item.x;
@@ -2359,17 +2379,17 @@ __global__ void __launch_bounds__(kBlock, 1) k_solve(DevGraph G, Job J) {
                             for (int q = lane; q < nit; q += 32) next_items[pos + q] = make_int2(i, beg + q * kPrChunk);
                         }
                     }
-                    MF_SYNC_T(S_T_HUB, c, 3, lcg(&C->hub_act[c & 1]));
+                    MF_SYNC_T(S_T_HUB, c, 3, lctl(&C->hub_act[c & 1]));
                     if (gtid == 0 && fresh) C->hccnt = 0;
-                    if (lcg(&C->hub_act[c & 1]) == 0) {
+                    if (lctl(&C->hub_act[c & 1]) == 0) {
                         pass_hubs_clean = true;
                         break;
                     }
                 }
             }
             bool pass_rounds_clean = true;
-            int cnt = lcg(&C->wcnt);
-            const int qtail0 = qmode ? lcg(&C->aq_tail) : 0;   // queued by the hub cycles
+            int cnt = lctl(&C->wcnt);
+            const int qtail0 = qmode ? lctl(&C->aq_tail) : 0;   // queued by the hub cycles
             if (qmode && cnt + qtail0 > 0) {
                 // PushRelabel from the activation queue, without rounds: the
                 // worklist entries (generation 0) are dealt to the warps by
@@ -2436,11 +2456,11 @@ __global__ void __launch_bounds__(kBlock, 1) k_solve(DevGraph G, Job J) {
                         if (d == n0 + ld_acquire_s32(&C->aq_tail)) atomicExch(&C->aq_fin, 1);
                     }
                 }
-                MF_SYNC_T(S_T_PRW, 0, 0, cnt + lcg(&C->aq_tail));
-                pass_rounds_clean = lcg(&C->aq_over) == 0;
+                MF_SYNC_T(S_T_PRW, 0, 0, cnt + lctl(&C->aq_tail));
+                pass_rounds_clean = lctl(&C->aq_over) == 0;
                 if (gtid == 0) {
-                    ST[S_ROUNDS] += lcg(&C->aq_maxgen) + 1;
-                    ST[S_WL] += cnt + lcg(&C->aq_tail);
+                    s_stat[S_ROUNDS] += lctl(&C->aq_maxgen) + 1;
+                    s_stat[S_WL] += cnt + lctl(&C->aq_tail);
                 }
                 // (the counters are zeroed for the next pass after its set-up
                 // barrier, when every thread has read them)
@@ -2452,8 +2472,8 @@ __global__ void __launch_bounds__(kBlock, 1) k_solve(DevGraph G, Job J) {
                     const ActList AL{&C->acnt[(rd + 1) % 3], nlist, snext++, rstamp_it, pcnt, AL0.hlist, hstamp};
                     if (gtid == 0) {
                         C->acnt[(rd + 2) % 3] = 0;
-                        ST[S_ROUNDS] += 1;
-                        ST[S_WL] += cnt;
+                        s_stat[S_ROUNDS] += 1;
+                        s_stat[S_WL] += cnt;
                     }
                     if (jmode == MF_MODE_TOPOLOGY) {
                         // topology-driven (Sec. 5.2): every round visits every
@@ -2489,7 +2509,7 @@ __global__ void __launch_bounds__(kBlock, 1) k_solve(DevGraph G, Job J) {
                             push_relabel_warp(G, lcg(&list[i]), kc, AL, stg, K);
                     }
                     MF_SYNC_T(S_T_PRW, rd, 0, cnt);
-                    cnt = lcg(AL.cnt);
+                    cnt = lctl(AL.cnt);
                     list = nlist;
                     if (cnt == 0) pass_rounds_clean = true;
                     if (cnt == 0 || rd + 1 >= max_rounds || (rd + 1 >= kMaxRounds && cnt > nwarps)) break;
@@ -2497,7 +2517,7 @@ __global__ void __launch_bounds__(kBlock, 1) k_solve(DevGraph G, Job J) {
             }
             hubs_clean = pass_hubs_clean;
             rounds_clean = pass_rounds_clean;
-            pend = lcg(pcnt);   // every append to it came before the pass's last barrier
+            pend = lctl(pcnt);   // every append to it came before the pass's last barrier
             // another pass only for a few re-activated hubs: a large set of
             // them is better served after a global relabel
             if (pend == 0 || pend > (PP ? kPassHubsPP : kPassHubs) || !pass_hubs_clean || !pass_rounds_clean)
@@ -2509,7 +2529,7 @@ __global__ void __launch_bounds__(kBlock, 1) k_solve(DevGraph G, Job J) {
         // (push-pull: only arcs within the vertex's part; the pull side uses
         // the h- form, Algorithm 7)
         const unsigned char *ptc = stage ? G.part : nullptr;
-        const int nrl = lcg(&C->rlcnt);
+        const int nrl = lctl(&C->rlcnt);
         for (int i = gwarp; i < nrl; i += nwarps) {
             const int u = bcast_ld(&G.rl[i]);
             if (!vertex_ok(J, C, u, n)) continue;   // warp-uniform
@@ -2519,7 +2539,7 @@ __global__ void __launch_bounds__(kBlock, 1) k_solve(DevGraph G, Job J) {
             else
                 remove_invalid_warp_t<false>(G, u, &C->ri_moved[par], ptc, side, K);
         }
-        const int nri = lcg(&C->rhcnt);
+        const int nri = lctl(&C->rhcnt);
         for (int w = gwarp; w < nri; w += nwarps) {
             const int2 item = lcg(&G.hri[w]);
             const int u = __shfl_sync(kFull, item.x, 0);
@@ -2552,7 +2572,7 @@ __global__ void __launch_bounds__(kBlock, 1) k_solve(DevGraph G, Job J) {
         // vertices, and RemoveInvalidEdges found none), so each vertex with
         // excess sits at height >= n and cannot reach a sink: the preflow is
         // maximum without another BFS.  The value needs the current deficits.
-        const int busy = (rounds_clean ? 0 : 1) | (hubs_clean ? 0 : 2) | (lcg(&C->ri_moved[par]) ? 4 : 0) |
+        const int busy = (rounds_clean ? 0 : 1) | (hubs_clean ? 0 : 2) | (lctl(&C->ri_moved[par]) ? 4 : 0) |
                          (pend > 0 ? 8 : 0);
         if (gtid == 0 && TR && C->trace_n - 1 < G.trace_cap) TR[C->trace_n - 1].mode = (short)busy;
         if (!J.exact_exit && kind != JOB_REFRESH && stage == 0 && busy == 0) {
@@ -2615,9 +2635,11 @@ __global__ void __launch_bounds__(kBlock, 1) k_solve(DevGraph G, Job J) {
 
     // ---- result and statistics -------------------------------------------
     if (gtid == 0) {
+        for (int i = 0; i < S_COUNT; ++i)
+            if (s_stat[i]) add_ll(&ST[i], s_stat[i]);
         // dacc: deficits at the last height init, or recounted at a clean
         // exit and after a push-pull repair
-        if (!fast) C->flow = lcg(&G.e[t]) + lcg(&C->dacc[(early || pp_ran) ? (it & 1) ^ 1 : it & 1]);
+        if (!fast) C->flow = lcg(&G.e[t]) + lctl(&C->dacc[(early || pp_ran) ? (it & 1) ^ 1 : it & 1]);
         if (kind != JOB_REFRESH) {
             C->iters = fast ? 0 : early ? it + 1 : it;
             C->exit_kind = fast ? EXIT_NO_CUT_CHANGE : early ? EXIT_CLEAN : pp_ran ? EXIT_PUSH_PULL : EXIT_BFS;
