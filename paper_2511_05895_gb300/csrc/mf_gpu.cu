@@ -72,9 +72,19 @@ enum JobKind { JOB_SOLVE = 0, JOB_REPAIR = 1, JOB_RECOMPUTE = 2, JOB_AUTO = 3, J
 // How the last solve/repair ended (mf_stats.exit_kind)
 enum ExitKind { EXIT_BFS = 0, EXIT_CLEAN = 1, EXIT_NO_CUT_CHANGE = 2, EXIT_PUSH_PULL = 3 };
 
-// Fewest PushRelabel activation rounds per loop iteration, and the fewest
+// Most PushRelabel rounds of the topology-driven mode per loop iteration
+// (more on deep graphs), and the fewest
 // cooperative cycles the high-degree vertices get per iteration (see k_solve).
 constexpr int kMaxRounds = 16;
+// Share of the last BFS's time that the activation queue gets (see k_solve).
+// Measured per batch for 1/2, 1, 2 and for the earlier bound of max(16, BFS
+// levels) generations: 1000-vertex graph 109, 126, 156, 127 us; unit
+// assignment graph of 2^18 + 2^18 vertices 1.43, 1.26, 1.40, 1.60 ms; 1023 x
+// 769 grid 1.37, 1.38, 1.75, 1.52 ms; 2048^2 grid (push-pull) 3.04, 2.69,
+// 2.76, 3.16 ms; RMAT-20 static solve 3.18, 3.20, 3.40, 3.18 ms.
+constexpr unsigned kQueueShareNum = 3, kQueueShareDen = 4;
+constexpr int kMinGen = 8;         // activation generations served whatever the time
+constexpr int kMaxGen = 1 << 30;   // generations fit the queue's 32-bit field
 constexpr int kMinHubCycles = 4;
 // The push-pull instance gives its hubs more cycles per pass: there a hub
 // left active costs another dual search of the whole graph (measured on
@@ -259,9 +269,11 @@ __device__ __forceinline__ unsigned long long ld_acquire_u64(const unsigned long
     return v;
 }
 
-__device__ __forceinline__ void st_release_u64(unsigned long long *p, unsigned long long v) {
-    asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+__device__ __forceinline__ void st_relaxed_u64(unsigned long long *p, unsigned long long v) {
+    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
+
+__device__ __forceinline__ void fence_acq_rel() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
 
 __device__ __forceinline__ unsigned long long gtimer() {
     unsigned long long t;
@@ -378,7 +390,7 @@ __device__ __forceinline__ bool grid_sync(Ctl *C) {
 // iteration cost ≈ 10 us per iteration: 3,648 atomics on each of 9 words.
 struct Counters {
     unsigned bfs_arcs = 0, bfs_verts = 0, pr_arcs = 0, push = 0, relabel = 0, ri_arcs = 0,
-             ri_moves = 0, clamped = 0, resat = 0;
+             ri_moves = 0, clamped = 0, resat = 0, visits = 0;
 };
 
 constexpr int kIlp = 4;    // arcs in flight per lane in PushRelabel and RemoveInvalidEdges
@@ -439,7 +451,6 @@ struct Front {
     int *stage;     // this warp's kWq shared ints, or nullptr
     int sn;         // staged entries (warp-uniform)
     long long ds;   // arc total not yet added (warp-uniform)
-    unsigned mark;  // activation stamp given to the worklist entries (queued from the start)
 };
 
 // Publish the staged entries and do their bookkeeping: each joins the global
@@ -479,7 +490,6 @@ __device__ __forceinline__ void front_flush_entries(const DevGraph &G, Front &F,
             K.bfs_verts += ok[j];
             hub[j] = act && deg[j] > kHubDeg;
             small[j] = act && !hub[j];
-            if (small[j]) G.astamp[v[j]] = F.mark;
         }
         warp_append_n(small, v, &G.ctl->wcnt, G.wl);
         warp_append_n(hub, v, &G.ctl->hcnt, G.hl);
@@ -552,7 +562,6 @@ __device__ __forceinline__ void bfs_discovered_n(const DevGraph &G, const bool (
         const bool act = disc[j] && (((fwd >> j) & 1u) ? ev[j] < 0 : ev[j] > 0);
         hub[j] = act && deg[j] > kHubDeg;
         small[j] = act && !hub[j];
-        if (small[j]) G.astamp[v[j]] = F.mark;
     }
     ds = warp_sum(ds);
     if ((threadIdx.x & 31) == 0 && ds) add_ll(F.asum, ds);
@@ -799,29 +808,36 @@ __device__ __forceinline__ long long pull_arc(const DevGraph &G, int a, int b, i
     return (long long)atomicAdd(reinterpret_cast<unsigned long long *>(&G.e[v]), (unsigned long long)(-(long long)d));
 }
 
-// Where the vertices that a push makes active go: the list of the next
-// activation round (see the PushRelabel phase of k_solve).  A vertex enters
-// one list at most once, by the stamp of that list.
+// Where the vertices that a push makes active go.
+//
+// Worklist vertices (degree <= kHubDeg), in the data-driven and push-pull
+// modes: the activation queue, with generation gen.  The sign of the excess
+// says who holds a vertex: the one atomic that takes e(v) from <= 0 to > 0
+// (its returned old value tells) makes v active and hands it to the thread
+// that issued it, which queues v or goes on with it; every later push finds
+// e(v) > 0 and files nothing; and the warp that serves v lowers e(v) once, as
+// the last thing it does with v, after a fence.  So a vertex is queued or
+// served at most once at a time, with no mark to take and give back (the mark
+// cost two returning atomics and two fences per activation).  A pull mirrors
+// the signs.  In the topology-driven mode they are only counted: every round
+// finds the active vertices by itself.
+//
+// Hubs (degree > kHubDeg): the next pass's hub list, once, by its stamp.
 struct ActList {
-    int *cnt;
-    int *list;
-    unsigned stamp;
-    unsigned rstamp;   // stamp of this loop iteration's relabel list
-    int *hcnt;         // the next pass's hub list (high-degree vertices a push
-    int *hlist;        //   turned active), its size and its stamp
+    int *hcnt, *hlist;          // the next pass's hub list, its size and its stamp
     unsigned hstamp;
-    // queue mode (the PushRelabel phases of the data-driven and push-pull
-    // modes): activated vertices go to the activation queue with generation
-    // gen instead of to list; stamp then marks "queued or being processed"
-    unsigned long long *aq;   // or nullptr: round lists
-    int qc, gen, gen_cap;
+    unsigned long long *aq;     // activation queue, or nullptr: count only
+    int qc, gen, gen_cap;       // its capacity; generation of what is filed, and the first one not queued
+    const volatile unsigned long long *deadline;   // shared: when the phase ends (globaltimer)
     Ctl *C;
+    int count;                  // filed without a queue (warp-uniform)
 };
 
 // Enqueue the lanes' flagged vertices of N slots into the activation queue
 // with generation AL.gen (one reservation per warp); entries past the queue's
 // capacity are dropped, counted as finished and flagged (the iteration then
-// ends on another global relabel).  All 32 lanes call.
+// ends on another global relabel).  The caller has fenced what the entries'
+// servers must see.  All 32 lanes call.
 template <int N>
 __device__ __forceinline__ void aq_push_n(const ActList &AL, const bool (&pred)[N], const int (&val)[N]) {
     const int lane = threadIdx.x & 31;
@@ -843,34 +859,26 @@ __device__ __forceinline__ void aq_push_n(const ActList &AL, const bool (&pred)[
     for (int j = 0; j < N; ++j) {
         if (pred[j]) {
             const int pos = base + __popc(m[j] & below);
-            if (pos < AL.qc) st_release_u64(&AL.aq[pos], tag | (unsigned)(val[j] + 1));
+            if (pos < AL.qc) st_relaxed_u64(&AL.aq[pos], tag | (unsigned)(val[j] + 1));
             else ++over;
         }
         base += __popc(m[j]);
     }
-    over = (int)warp_sum((long long)over);
-    if (lane == 0) {
-        atomicMax(&AL.C->aq_maxgen, AL.gen);
-        if (over) {
+    if (base > AL.qc) {   // warp-uniform: base is now past the warp's last entry
+        over = (int)warp_sum((long long)over);
+        if (lane == 0) {
             atomicAdd(&AL.C->aq_done, over);
             atomicExch(&AL.C->aq_over, 1);
         }
     }
-}
-
-// A vertex whose height PushRelabel raised joins the relabel list of the loop
-// iteration once: only relabelled vertices can own arcs that RemoveInvalidEdges
-// must saturate (the others keep their BFS height, which no residual arc can
-// make steep).  One thread calls.
-__device__ __forceinline__ void note_relabel(const DevGraph &G, int u, unsigned rstamp) {
-    if (atomicExch(&G.rstamp[u], rstamp) != rstamp) G.rl[atomicAdd(&G.ctl->rlcnt, 1)] = u;
+    if (lane == 0) atomicMax(&AL.C->aq_maxgen, AL.gen);
 }
 
 // Single-thread enqueue of v (as aq_push_n).
 __device__ __forceinline__ void aq_push_one(const ActList &AL, int v) {
     const int pos = atomicAdd(&AL.C->aq_tail, 1);
     if (pos < AL.qc) {
-        st_release_u64(&AL.aq[pos], ((unsigned long long)(unsigned)AL.gen << 32) | (unsigned)(v + 1));
+        st_relaxed_u64(&AL.aq[pos], ((unsigned long long)(unsigned)AL.gen << 32) | (unsigned)(v + 1));
     } else {
         atomicAdd(&AL.C->aq_done, 1);
         atomicExch(&AL.C->aq_over, 1);
@@ -878,44 +886,65 @@ __device__ __forceinline__ void aq_push_one(const ActList &AL, int v) {
     atomicMax(&AL.C->aq_maxgen, AL.gen);
 }
 
-// File the vertices that moves turned active (add: worklist vertices, degree
-// <= kHubDeg; add_hub: hubs; neither s nor t): each joins the next activation
-// round's list -- in queue mode the activation queue -- or the next pass's
-// hub list, once, by the list's stamp.  In queue mode a vertex is marked
-// from its enqueue until the warp that processes it has finished, and that
-// warp clears the mark before it reads the vertex's excess a last time: with
-// a fence between the excess atomic and the mark here, and between the clear
-// and the read there, at least one side sees the other, so a vertex that a
-// push turns active while it is being processed is queued again exactly once
-// and no activation is lost.  Past the generation cap a vertex is left
+// File hubs that moves turned active.  All 32 lanes call.
+template <int N>
+__device__ __forceinline__ void file_hubs(const DevGraph &G, bool (&add_hub)[N], const int (&v)[N],
+                                          const ActList &AL) {
+    bool any = false;
+#pragma unroll
+    for (int j = 0; j < N; ++j) any |= add_hub[j];
+    if (!__any_sync(kFull, any)) return;
+#pragma unroll
+    for (int j = 0; j < N; ++j)
+        if (add_hub[j]) add_hub[j] = atomicExch(&G.astamp[v[j]], AL.hstamp) != AL.hstamp;
+    warp_append_n(add_hub, v, AL.hcnt, AL.hlist);
+}
+
+// File the vertices that moves turned active (add: worklist vertices; add_hub:
+// hubs; neither s nor t).  Past the generation cap a worklist vertex is left
 // active, unqueued, and the phase is flagged.  All 32 lanes call.
 template <int N>
 __device__ __forceinline__ void file_activations(const DevGraph &G, bool (&add)[N], bool (&add_hub)[N],
-                                                 const int (&v)[N], const ActList &AL) {
+                                                 const int (&v)[N], ActList &AL) {
+    file_hubs(G, add_hub, v, AL);
     bool any = false;
 #pragma unroll
-    for (int j = 0; j < N; ++j) any |= add[j] || add_hub[j];
+    for (int j = 0; j < N; ++j) any |= add[j];
     if (!__any_sync(kFull, any)) return;
-    if (AL.aq) {
-        if (AL.gen >= AL.gen_cap) {
-            bool capped = false;
+    if (!AL.aq) {
 #pragma unroll
-            for (int j = 0; j < N; ++j) {
-                capped |= add[j];
-                add[j] = false;
-            }
-            if (__any_sync(kFull, capped) && (threadIdx.x & 31) == 0) atomicExch(&AL.C->aq_over, 1);
-        }
-        __threadfence();
+        for (int j = 0; j < N; ++j) AL.count += __popc(__ballot_sync(kFull, add[j]));
+        return;
     }
-#pragma unroll
-    for (int j = 0; j < N; ++j) {
-        if (add[j]) add[j] = atomicExch(&G.astamp[v[j]], AL.stamp) != AL.stamp;
-        if (add_hub[j]) add_hub[j] = atomicExch(&G.astamp[v[j]], AL.hstamp) != AL.hstamp;
+    if (AL.gen >= AL.gen_cap) {
+        if ((threadIdx.x & 31) == 0) atomicExch(&AL.C->aq_over, 1);
+        return;
     }
-    if (AL.aq) aq_push_n(AL, add, v);
-    else warp_append_n(add, v, AL.cnt, AL.list);
-    warp_append_n(add_hub, v, AL.hcnt, AL.hlist);
+    __syncwarp();
+    fence_acq_rel();
+    aq_push_n(AL, add, v);
+}
+
+// The vertices a warp has relabelled, staged one per lane: they join the loop
+// iteration's relabel list 32 at a time, each once (rstamp).  Only relabelled
+// vertices can own arcs that RemoveInvalidEdges must saturate (the others
+// keep their BFS height, which no residual arc can make steep).
+struct Relabelled {
+    int u = 0, cnt = 0;   // lane k's vertex; staged vertices (warp-uniform)
+    unsigned stamp = 0;
+};
+
+__device__ __forceinline__ void relabelled_flush(const DevGraph &G, Relabelled &R) {
+    const int lane = threadIdx.x & 31;
+    bool add = lane < R.cnt;
+    if (add) add = atomicExch(&G.rstamp[R.u], R.stamp) != R.stamp;
+    warp_append(add, R.u, &G.ctl->rlcnt, G.rl);
+    R.cnt = 0;
+}
+
+__device__ __forceinline__ void note_relabel(const DevGraph &G, int u, Relabelled &R) {
+    if ((threadIdx.x & 31) == R.cnt) R.u = u;
+    if (++R.cnt == 32) relabelled_flush(G, R);
 }
 
 // One round of a warp's arc scan: lane i holds arcs a0 + 32 j + i (j < kIlp)
@@ -983,34 +1012,18 @@ __device__ __forceinline__ long long move_arc(const DevGraph &G, int a, int b, i
     return PULL ? pull_arc(G, a, b, v, d) : push_arc(G, a, b, v, d);
 }
 
-// The amounts of one round at height hh, in arc order (round slot j, then
-// lane), as consecutive Alg. 2 steps would move them: min(rem, c_f) each
-// until rem is used up; tot receives the round's residual at height hh.
-__device__ __forceinline__ void round_amounts(const ArcRound &R, int hh, long long rem, int (&d)[kIlp],
-                                              long long &tot) {
-    tot = 0;
-#pragma unroll
-    for (int j = 0; j < kIlp; ++j) {
-        const int ra = (R.ra[j] > 0 && R.hv[j] == hh) ? R.ra[j] : 0;
-        const long long incl = warp_incl_scan(ra) + tot;
-        const long long dj = rem - (incl - ra);
-        d[j] = dj < 0 ? 0 : (dj > ra ? ra : (int)dj);
-        tot = __shfl_sync(kFull, incl, 31);
-    }
-}
-
 // The moves of one round (d[j] > 0: d[j] units along slot j of R, a round
 // loaded with its reverse arcs), and the filing of the vertices they turn
 // active: a push that raised e(v) above 0 (a pull that lowered it below 0)
-// makes v active, and v (not s or t) joins the next activation round when its
-// degree is <= kHubDeg, else the hub list of the next PushRelabel pass.  The
+// makes v active, and v (not s or t) is filed (ActList) as a worklist vertex
+// when its degree is <= kHubDeg, else as a hub.  The
 // heads' degrees load beside the move atomics, so the filing waits once for
 // both; v's height is the one the scan read (a push only goes below h(u) <
 // n).  Each list gets one reservation per warp.  Returns this lane's total
 // moved.  All 32 lanes call.
 template <bool PULL>
 __device__ __forceinline__ long long move_round(const DevGraph &G, int a0, const int (&d)[kIlp], const ArcRound &R,
-                                                const ActList &AL, Counters &K) {
+                                                ActList &AL, Counters &K) {
     const int lane = threadIdx.x & 31;
     long long old[kIlp], sent = 0;
     int deg[kIlp];
@@ -1086,13 +1099,13 @@ __device__ __forceinline__ void stage_wait() {
 // Heights of the heads of the staged residual arcs in [a0, a1): sh[i] = h of
 // the head, or INT_MAX for no residual arc (out of range, zero residual, or,
 // with a partition array pt, a head in another part: its residual is zeroed
-// in sr).  Returns this lane's lowest (height, arc - a0) key.
-__device__ __forceinline__ unsigned long long stage_heights(const DevGraph &G, const int *sv, int *sr, int *sh,
+// in sr).  Returns this lane's lowest height.
+__device__ __forceinline__ unsigned stage_heights(const DevGraph &G, const int *sv, int *sr, int *sh,
                                                             int a0, int a1, const unsigned char *pt,
                                                             unsigned char side) {
     const int lane = threadIdx.x & 31;
     const int base = a0 & ~3, cnt = a1 - base;
-    unsigned long long best = ~0ull;
+    unsigned best = INT_MAX;
     for (int i0 = lane; i0 < cnt; i0 += 32 * kGat) {
         int hv[kGat];
         bool res[kGat];
@@ -1113,10 +1126,7 @@ __device__ __forceinline__ unsigned long long stage_heights(const DevGraph &G, c
                 sr[i] = 0;
             }
             if (i < cnt) sh[i] = res[j] ? hv[j] : INT_MAX;
-            if (res[j]) {
-                const unsigned long long key = ((unsigned long long)(unsigned)hv[j] << 32) | (unsigned)(base + i - a0);
-                best = key < best ? key : best;
-            }
+            if (res[j]) best = min(best, (unsigned)hv[j]);
         }
     }
     __syncwarp();
@@ -1129,7 +1139,7 @@ __device__ __forceinline__ unsigned long long stage_heights(const DevGraph &G, c
 constexpr int kMv = 4;   // moves in flight per lane
 template <bool PULL, int N>
 __device__ __forceinline__ long long move_batch(const DevGraph &G, const int (&a)[N], const int (&b)[N],
-                                                const int (&v)[N], const int (&d)[N], const ActList &AL,
+                                                const int (&v)[N], const int (&d)[N], ActList &AL,
                                                 Counters &K) {
     long long old[N], sent = 0;
     int deg[N];
@@ -1162,7 +1172,7 @@ __device__ __forceinline__ long long move_batch(const DevGraph &G, const int (&a
 // once, kGat per lane in flight.  Returns the warp's total moved (all lanes).
 template <bool PULL>
 __device__ __forceinline__ long long stage_moves(const DevGraph &G, const int *sv, const int *sr, int *sh, int a0,
-                                                 int a1, int hh, long long rem, const ActList &AL, Counters &K) {
+                                                 int a1, int hh, long long rem, ActList &AL, Counters &K) {
     const int lane = threadIdx.x & 31;
     const int base = a0 & ~3, cnt = a1 - base;
     int iend = 0;
@@ -1197,139 +1207,285 @@ __device__ __forceinline__ long long stage_moves(const DevGraph &G, const int *s
     return warp_sum(sent);
 }
 
-// Algorithm 2 on vertex u by one warp, up to kc cycles.  A cycle scans u's
-// arcs once for the lowest residual neighbour height h^ (ties: lowest arc;
-// heights read once per cycle, Note 3 of Sec. 3).  If h(u) > h^ the cycle
-// performs the pushes that consecutive Alg. 2 steps would make to the arcs at
-// height h^ -- in arc order, min(e, c_f) each, until e(u) is used up --
-// (from the round the scan loaded when u has one round of arcs; vertices with
-// more reload the rounds that hold such an arc); otherwise it relabels u to
-// h^ + 1.  A vertex without residual arcs gets height n.  Only u's warp
-// lowers r(u, .) and e(u) and changes h(u) during a round; other warps only
-// raise r(u, .) and e(u), so every amount pushed is available, h(u) is read
-// once, and e(u) is re-read beside each cycle's arc loads.  With PULL the
-// same steps are Algorithm 6 (PullRelabel) on a deficient u: residual arcs
-// into u, pulls of min(-e, c_f) from the lowest of them.  Once its steps are
-// done u joins the iteration's relabel list if it was relabelled, and the
-// next round's list if still active.
-template <bool PULL>
-__device__ __forceinline__ void pr_finish_t(const DevGraph &G, int u, int hu, bool relabelled, const ActList &AL) {
-    if ((threadIdx.x & 31) == 0) {
-        if (relabelled) note_relabel(G, u, AL.rstamp);
-        if (AL.aq) {
-            atomicExch(&G.astamp[u], 0u);   // u leaves the queue before its excess is read (file_activations)
-            __threadfence();
-        }
-        const long long eu = lcg(&G.e[u]);
-        if (hu < G.n && (PULL ? eu < 0 : eu > 0)) {
-            if (AL.aq && AL.gen >= AL.gen_cap) {
-                atomicExch(&AL.C->aq_over, 1);
-            } else if (atomicExch(&G.astamp[u], AL.stamp) != AL.stamp) {
-                if (AL.aq) aq_push_one(AL, u);
-                else AL.list[atomicAdd(AL.cnt, 1)] = u;
-            }
-        }
-    }
-    __syncwarp();
-}
+// Minimum over the warp of a height (INT_MAX: none).
+__device__ __forceinline__ int warp_min_height(unsigned h) { return (int)__reduce_min_sync(kFull, h); }
 
-// The cycle's decision after the scan: returns the height to push to, or -1
-// after a relabel (hu updated, h(u) written), or -2 when u is done.
-__device__ __forceinline__ int pr_decide(const DevGraph &G, int u, unsigned long long best, long long eu, int &hu,
-                                         bool &relabelled, Counters &K) {
-    if (eu <= 0) return -2;
-    if (best == ~0ull) {
-        hu = G.n;
-        if ((threadIdx.x & 31) == 0) {
-            G.h[u] = G.n;
-            ++K.relabel;
-        }
-        relabelled = true;
-        return -2;
-    }
-    const int hh = (int)(best >> 32);
-    if (hu <= hh) {
-        hu = hh + 1;
-        if ((threadIdx.x & 31) == 0) {
-            G.h[u] = hu;
-            ++K.relabel;
-        }
-        relabelled = true;
-        return -1;
-    }
-    return hh;
-}
-
-// u with one round of arcs (<= 32 kIlp)
+// Algorithm 2 on a vertex u of degree > 32 kIlp (<= kHubDeg) by one warp, up
+// to kc steps, the arcs staged in the warp's shared memory (heads once,
+// residuals and heights before every push).  A step scans u's arcs for the
+// lowest residual neighbour height h^; if h(u) > h^ it performs the pushes
+// that consecutive Alg. 2 steps would make to the arcs at height h^ -- in arc
+// order, min(e, c_f) each, until e(u) is used up -- else it relabels u to
+// h^ + 1 (the next step pushes along the arcs just scanned).  A vertex
+// without residual arcs gets height n.  Only u's warp lowers r(u, .) and e(u)
+// and changes h(u) during the phase; other warps only raise r(u, .) and e(u),
+// so every amount pushed is available.  e(u) is lowered once, at the end
+// (ActList).  With PULL the same steps are Algorithm 6 (PullRelabel) on a
+// deficient u: residual arcs into u, pulls of min(-e, c_f) from the lowest of
+// them.  Returns whether u is still active (all lanes).
 template <bool PULL>
-__device__ __forceinline__ void push_relabel_small_t(const DevGraph &G, int u, int beg, int end, int kc,
-                                                  const ActList &AL, const unsigned char *pt, unsigned char side,
-                                                  Counters &K) {
-    const int lane = threadIdx.x & 31;
-    int hu = bcast_ld(&G.h[u]);
-    bool relabelled = false;
-    for (int c = 0; c < kc && hu < G.n; ++c) {
-        const long long eu = bcast_ld(&G.e[u]);
-        ArcRound R;
-        load_round_t<PULL, true>(G, beg, end, R, pt, side);
-        K.pr_arcs += round_arcs(beg, end);
-        const unsigned long long best = warp_min(round_min_key(R, beg, beg));
-        const int hh = pr_decide(G, u, best, PULL ? -eu : eu, hu, relabelled, K);
-        if (hh == -2) break;
-        if (hh == -1) continue;
-        int d[kIlp];
-        long long tot;
-        round_amounts(R, hh, PULL ? -eu : eu, d, tot);
-        const long long sent = warp_sum(move_round<PULL>(G, beg, d, R, AL, K));
-        if (lane == 0 && sent) add_ll(&G.e[u], PULL ? sent : -sent);
-        __syncwarp();
-    }
-    pr_finish_t<PULL>(G, u, hu, relabelled, AL);
-}
-
-// u with more than one round of arcs (<= kHubDeg): the arcs are staged in
-// the warp's shared memory (heads once, residuals and heights every cycle),
-// and the pushes go along the staged arcs at height h^ in arc order, 32 arcs
-// a step.
-template <bool PULL>
-__device__ __forceinline__ void push_relabel_staged_t(const DevGraph &G, int u, int beg, int end, int kc,
-                                                      const ActList &AL, const unsigned char *pt,
-                                                      unsigned char side, int *stg, Counters &K) {
+__device__ __forceinline__ bool visit_staged_t(const DevGraph &G, int u, int beg, int end, int kc, ActList &AL,
+                                               const unsigned char *pt, unsigned char side, int *stg, Relabelled &RL,
+                                               Counters &K) {
     const int lane = threadIdx.x & 31;
     int *sv = stg, *sr = stg + kStgInts, *sh = stg + 2 * kStgInts;
     stage_copy(G.head, sv, beg, end, G.A, G.al16);
-    int hu = bcast_ld(&G.h[u]);
-    bool relabelled = false;
-    for (int c = 0; c < kc && hu < G.n; ++c) {
-        const long long eu = bcast_ld(&G.e[u]);
+    const int hu = bcast_ld(&G.h[u]);
+    int h = hu;
+    const long long e0 = bcast_ld(&G.e[u]);
+    const long long want = PULL ? -e0 : e0;
+    long long sent = 0;
+    for (int c = 0; c < kc && h < G.n && sent < want; ++c) {
         stage_copy(PULL ? G.rr : G.r, sr, beg, end, G.A, G.al16);
         stage_wait();
         K.pr_arcs += (end - beg + 31 - lane) / 32;
-        const unsigned long long best = warp_min(stage_heights(G, sv, sr, sh, beg, end, pt, side));
-        const int hh = pr_decide(G, u, best, PULL ? -eu : eu, hu, relabelled, K);
-        if (hh == -2) break;
-        if (hh == -1) continue;
-        const long long sent = stage_moves<PULL>(G, sv, sr, sh, beg, end, hh, PULL ? -eu : eu, AL, K);
-        if (lane == 0 && sent) add_ll(&G.e[u], PULL ? sent : -sent);
+        const int hh = warp_min_height(stage_heights(G, sv, sr, sh, beg, end, pt, side));
+        if (h <= hh) {
+            h = hh == INT_MAX ? G.n : hh + 1;
+            if (lane == 0) {
+                G.h[u] = h;
+                ++K.relabel;
+            }
+            if (hh == INT_MAX || ++c >= kc || h >= G.n) break;
+        }
+        sent += stage_moves<PULL>(G, sv, sr, sh, beg, end, hh, want - sent, AL, K);
         __syncwarp();
     }
-    pr_finish_t<PULL>(G, u, hu, relabelled, AL);
+    if (h != hu) note_relabel(G, u, RL);
+    bool active = sent < want;
+    if (sent) {
+        __syncwarp();
+        fence_acq_rel();   // the moves and h(u), before another warp may take u
+        if (lane == 0) {
+            const unsigned long long d = PULL ? (unsigned long long)sent : (unsigned long long)(-sent);
+            const long long now = (long long)(atomicAdd(reinterpret_cast<unsigned long long *>(&G.e[u]), d) + d);
+            active = PULL ? now < 0 : now > 0;
+        }
+        active = __shfl_sync(kFull, active, 0);
+    }
+    __syncwarp();
+    return active && h < G.n;
 }
 
+// Serve the active vertex u of generation AL.gen - 1 by one warp: up to kc
+// steps of Algorithm 2 (as visit_staged_t) on the residuals and heights of
+// one load of its arcs (<= 32 kIlp; larger vertices: visit_staged_t), which
+// the steps share -- heights only rise and residuals out of u only grow
+// meanwhile, so the moves stay within the residuals, and an arc that a stale
+// height made steep is RemoveInvalidEdges' to saturate, as with Alg. 2's own
+// unlocked reads.  All moves are issued together at the end.
+//
+// Then the warp goes on with one of the vertices its moves turned active,
+// whose arc range has come back beside the move atomics, and only the others
+// go to the queue: a lone excess travels along its path at four dependent
+// round trips per vertex (arcs; heads' heights; move atomics; fence), without
+// the queue's three (reservation, slot, poll) and the row lookup.  What the
+// excess of u became is looked at after the next vertex's first loads are
+// issued.  In the topology-driven mode (AL.aq null) activations are counted
+// and nothing is followed.  Past the deadline (globaltimer) no generation
+// from kMinGen on is served: what is still active stays so, and the phase is
+// flagged.
 template <bool PULL>
-__device__ __forceinline__ void push_relabel_warp_t(const DevGraph &G, int u, int kc, const ActList &AL,
-                                                    const unsigned char *pt, unsigned char side, int *stg,
-                                                    Counters &K) {
-    const int beg = __ldg(&G.row[u]), end = __ldg(&G.row[u + 1]);
-    if (end - beg <= 32 * kIlp)
-        push_relabel_small_t<PULL>(G, u, beg, end, kc, AL, pt, side, K);
-    else
-        push_relabel_staged_t<PULL>(G, u, beg, end, kc, AL, pt, side, stg, K);
+__device__ __forceinline__ void visit_chain_t(const DevGraph &G, int u, int kc, ActList &AL, const unsigned char *pt,
+                                              unsigned char side, int *stg, Relabelled &RL, Counters &K) {
+    const int lane = threadIdx.x & 31;
+    int beg = __ldg(&G.row[u]), end = __ldg(&G.row[u + 1]);
+    const int gen0 = AL.gen;
+    int pu = -1;            // the vertex served before, if it may still be active:
+    long long pleft = 0;    // its excess after the visit (lane 0)
+    for (;;) {
+        if (lane == 0) ++K.visits;
+        const int deg = end - beg;
+        if (deg > 32 * kIlp) {
+            if (pu >= 0 && lane == 0 && (PULL ? pleft < 0 : pleft > 0)) {
+                --AL.gen;
+                aq_push_one(AL, pu);
+                ++AL.gen;
+            }
+            pu = -1;
+            __syncwarp();
+            const bool active = visit_staged_t<PULL>(G, u, beg, end, kc, AL, pt, side, stg, RL, K);
+            if (!active) break;
+            if (!AL.aq) {
+                ++AL.count;
+            } else if (lane == 0) {
+                if (AL.gen >= AL.gen_cap) atomicExch(&AL.C->aq_over, 1);
+                else aq_push_one(AL, u);
+            }
+            break;
+        }
+        int ra[kIlp], v[kIlp], hv[kIlp], rb[kIlp], d[kIlp];
+        long long eu = lane == 0 ? lcg(&G.e[u]) : 0;
+        int hu = lane == 0 ? lcg(&G.h[u]) : 0;
+#pragma unroll
+        for (int j = 0; j < kIlp; ++j) {
+            const int a = beg + 32 * j + lane;
+            ra[j] = a < end ? lcg(PULL ? &G.rr[a] : &G.r[a]) : 0;
+            v[j] = a < end ? __ldg(&G.head[a]) : 0;
+            d[j] = 0;
+            K.pr_arcs += a < end;
+        }
+        if (pu >= 0 && lane == 0 && (PULL ? pleft < 0 : pleft > 0)) {
+            --AL.gen;
+            aq_push_one(AL, pu);
+            ++AL.gen;
+        }
+        pu = -1;
+        eu = __shfl_sync(kFull, eu, 0);
+        hu = __shfl_sync(kFull, hu, 0);
+#pragma unroll
+        for (int j = 0; j < kIlp; ++j) {
+            const int a = beg + 32 * j + lane;
+            // (INT_MAX: not an arc to move along.  Arcs that a neighbour's push
+            // may make residual during the visit are kept where they cost no
+            // further round of loads)
+            const bool in = ra[j] > 0 || (deg <= 32 && a < end);
+            hv[j] = in ? lcg(&G.h[v[j]]) : INT_MAX;
+            rb[j] = in ? __ldg(&G.rev[a]) : 0;
+            if (pt && in && pt[v[j]] != side) hv[j] = INT_MAX;   // another part's arc counts as absent
+        }
+        const long long want = PULL ? -eu : eu;
+        long long rem = want;
+        int h = hu;
+        for (int c = 0; c < kc && rem > 0 && h < G.n; ++c) {
+            if (c > 0) {
+                // the heads' heights again, and the residuals beside them: two
+                // neighbours that both act on heights read before the other's
+                // relabel push the same excess back and forth (one read per
+                // visit: 30 -> 500-4,000 invalid arcs and 2-20x the iterations
+                // on grids)
+#pragma unroll
+                for (int j = 0; j < kIlp; ++j) {
+                    if (hv[j] == INT_MAX) continue;
+                    const int a = beg + 32 * j + lane;
+                    ra[j] = lcg(PULL ? &G.rr[a] : &G.r[a]);
+                    hv[j] = lcg(&G.h[v[j]]);
+                }
+            }
+            unsigned lo = INT_MAX;
+#pragma unroll
+            for (int j = 0; j < kIlp; ++j)
+                if (ra[j] > d[j]) lo = min(lo, (unsigned)hv[j]);
+            const int hh = warp_min_height(lo);
+            if (h <= hh) {
+                h = hh == INT_MAX ? G.n : hh + 1;
+                if (lane == 0) ++K.relabel;
+                continue;
+            }
+            // the moves at height hh, in arc order (slot j, then lane), until
+            // the excess is used up; sums saturate at 2^31 - 1, the most that
+            // one step moves
+            const unsigned most = rem > INT_MAX ? INT_MAX : (unsigned)rem;
+            unsigned left = most;
+#pragma unroll
+            for (int j = 0; j < kIlp; ++j) {
+                const unsigned x = (ra[j] > d[j] && hv[j] == hh) ? (unsigned)(ra[j] - d[j]) : 0u;
+                if (32 * j >= deg || !__any_sync(kFull, x > 0)) continue;   // warp-uniform
+                unsigned incl = x;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const unsigned y = __shfl_up_sync(kFull, incl, o);
+                    if (lane >= o) incl = min(incl + y, (unsigned)INT_MAX);
+                }
+                unsigned excl = __shfl_up_sync(kFull, incl, 1);
+                if (lane == 0) excl = 0;
+                d[j] += excl >= left ? 0 : (int)min(x, left - excl);
+                left -= min(__shfl_sync(kFull, incl, 31), left);
+            }
+            rem -= most - left;
+        }
+        if (h != hu) {
+            if (lane == 0) G.h[u] = h;
+            note_relabel(G, u, RL);
+        }
+        if (rem == want) {   // nothing moved: u keeps its excess
+            if (h >= G.n || rem <= 0) break;
+            if (!AL.aq) {
+                ++AL.count;
+            } else if (lane == 0) {
+                if (AL.gen >= AL.gen_cap) atomicExch(&AL.C->aq_over, 1);
+                else aq_push_one(AL, u);
+            }
+            break;
+        }
+        long long old[kIlp];
+        int vb[kIlp], ve[kIlp];
+#pragma unroll
+        for (int j = 0; j < kIlp; ++j) {
+            old[j] = 0;
+            vb[j] = ve[j] = 0;
+            if (d[j] > 0) {
+                old[j] = move_arc<PULL>(G, beg + 32 * j + lane, rb[j], v[j], d[j]);
+                vb[j] = __ldg(&G.row[v[j]]);
+                ve[j] = __ldg(&G.row[v[j] + 1]);
+                ++K.push;
+            }
+        }
+        bool add[kIlp], add_hub[kIlp];
+        int nu = -1, nb = 0, ne = 0;
+        unsigned tot = 0;
+#pragma unroll
+        for (int j = 0; j < kIlp; ++j) {
+            const bool turned = PULL ? (old[j] >= 0 && old[j] - d[j] < 0) : (old[j] <= 0 && old[j] + d[j] > 0);
+            const bool cand = d[j] > 0 && turned && v[j] != G.s && v[j] != G.t;
+            add[j] = cand && ve[j] - vb[j] <= kHubDeg;
+            add_hub[j] = cand && !add[j];
+            tot |= __ballot_sync(kFull, add[j]);
+        }
+        file_hubs(G, add_hub, v, AL);
+        __syncwarp();
+        fence_acq_rel();   // the moves and h(u), before another warp may take u or a head
+        if (lane == 0) {
+            const long long sent = want - rem;
+            const unsigned long long x = PULL ? (unsigned long long)sent : (unsigned long long)(-sent);
+            pleft = (long long)(atomicAdd(reinterpret_cast<unsigned long long *>(&G.e[u]), x) + x);
+        }
+        const bool maybe = h < G.n;   // u may still be active
+        if (!AL.aq) {
+#pragma unroll
+            for (int j = 0; j < kIlp; ++j) AL.count += __popc(__ballot_sync(kFull, add[j]));
+            AL.count += __shfl_sync(kFull, maybe && (PULL ? pleft < 0 : pleft > 0), 0);
+            break;
+        }
+        if (AL.gen >= kMinGen && (AL.gen >= AL.gen_cap || __any_sync(kFull, gtimer() > *AL.deadline))) {
+            const bool self = __shfl_sync(kFull, maybe && (PULL ? pleft < 0 : pleft > 0), 0);
+            if ((tot || self) && lane == 0) atomicExch(&AL.C->aq_over, 1);
+            break;
+        }
+        // the first of the activated heads is served next by this warp
+#pragma unroll
+        for (int j = 0; j < kIlp; ++j) {
+            const unsigned m = __ballot_sync(kFull, add[j]);
+            if (nu < 0 && m) {
+                const int src = __ffs(m) - 1;
+                nu = __shfl_sync(kFull, v[j], src);
+                nb = __shfl_sync(kFull, vb[j], src);
+                ne = __shfl_sync(kFull, ve[j], src);
+                if (lane == src) add[j] = false;
+            }
+        }
+        if (nu >= 0) {
+            aq_push_n(AL, add, v);
+            if (maybe) pu = u;
+        } else {
+            // no head: u itself, if it is still active
+            if (!__shfl_sync(kFull, maybe && (PULL ? pleft < 0 : pleft > 0), 0)) break;
+            nu = u;
+            nb = beg;
+            ne = end;
+        }
+        u = nu;
+        beg = nb;
+        end = ne;
+        ++AL.gen;
+    }
+    __syncwarp();
+    if (AL.aq && lane == 0 && AL.gen > gen0) atomicMax(&AL.C->aq_maxgen, AL.gen - 1);
 }
 
-__device__ __forceinline__ void push_relabel_warp(const DevGraph &G, int u, int kc, const ActList &AL, int *stg,
-                                                  Counters &K) {
-    push_relabel_warp_t<false>(G, u, kc, AL, nullptr, 0, stg, K);
+__device__ __forceinline__ void visit_chain(const DevGraph &G, int u, int kc, ActList &AL, int *stg, Relabelled &RL,
+                                            Counters &K) {
+    visit_chain_t<false>(G, u, kc, AL, nullptr, 0, stg, RL, K);
 }
 
 // Algorithm 3 over the arcs [a0, a1) of vertex u (height hu) by one warp:
@@ -1397,7 +1553,7 @@ __device__ __forceinline__ unsigned long long hub_scan_item(const DevGraph &G, i
 // (*rem) with one atomic.  Returns the amount this warp moved (all lanes).
 template <bool PULL>
 __device__ __forceinline__ long long hub_move_item(const DevGraph &G, int a0, int a1, int hh, long long *rem,
-                                                   const ActList &AL, const unsigned char *pt, unsigned char side,
+                                                   ActList &AL, const unsigned char *pt, unsigned char side,
                                                    bool skip_done, Counters &K) {
     const int lane = threadIdx.x & 31;
     long long sent = 0;
@@ -1437,12 +1593,12 @@ __device__ __forceinline__ long long hub_move_item(const DevGraph &G, int a0, in
 // Add the warp's counters to the statistics st and clear them.  All 32 lanes
 // call.
 __device__ __forceinline__ void flush_counters(Counters &K, long long *st) {
-    const unsigned vals[9] = {K.bfs_verts, K.bfs_arcs, K.pr_arcs, K.push, K.relabel, K.ri_arcs, K.ri_moves,
-                              K.clamped, K.resat};
-    const int idx[9] = {S_BFS_VERTS, S_BFS_ARCS, S_PR_ARCS, S_PUSH, S_RELABEL, S_RI_ARCS, S_RI_MOVES, S_CLAMPED,
-                        S_RESAT};
+    const unsigned vals[10] = {K.bfs_verts, K.bfs_arcs, K.pr_arcs, K.push, K.relabel, K.ri_arcs, K.ri_moves,
+                               K.clamped, K.resat, K.visits};
+    const int idx[10] = {S_BFS_VERTS, S_BFS_ARCS, S_PR_ARCS, S_PUSH, S_RELABEL, S_RI_ARCS, S_RI_MOVES, S_CLAMPED,
+                         S_RESAT, S_WL};
 #pragma unroll
-    for (int i = 0; i < 9; ++i) {
+    for (int i = 0; i < 10; ++i) {
         const long long v = warp_sum((long long)vals[i]);
         if ((threadIdx.x & 31) == 0 && v) add_ll(&st[idx[i]], v);
     }
@@ -1453,18 +1609,18 @@ __device__ __forceinline__ void flush_counters(Counters &K, long long *st) {
 // first: one global atomic per statistic and CTA instead of one per warp.
 // Every thread of the CTA calls.
 __device__ __forceinline__ void flush_counters_cta(Counters &K, long long *st) {
-    __shared__ unsigned long long s_sum[9];
-    if (threadIdx.x < 9) s_sum[threadIdx.x] = 0;
+    __shared__ unsigned long long s_sum[10];
+    if (threadIdx.x < 10) s_sum[threadIdx.x] = 0;
     __syncthreads();
-    const unsigned vals[9] = {K.bfs_verts, K.bfs_arcs, K.pr_arcs, K.push, K.relabel, K.ri_arcs, K.ri_moves,
-                              K.clamped, K.resat};
+    const unsigned vals[10] = {K.bfs_verts, K.bfs_arcs, K.pr_arcs, K.push, K.relabel, K.ri_arcs, K.ri_moves,
+                               K.clamped, K.resat, K.visits};
 #pragma unroll
-    for (int i = 0; i < 9; ++i) {
+    for (int i = 0; i < 10; ++i) {
         const long long v = warp_sum((long long)vals[i]);
         if ((threadIdx.x & 31) == 0 && v) atomicAdd(&s_sum[i], (unsigned long long)v);
     }
     __syncthreads();
-    if (threadIdx.x < 9 && s_sum[threadIdx.x]) {
+    if (threadIdx.x < 10 && s_sum[threadIdx.x]) {
         int slot;
         switch (threadIdx.x) {
             case 0: slot = S_BFS_VERTS; break;
@@ -1475,7 +1631,8 @@ __device__ __forceinline__ void flush_counters_cta(Counters &K, long long *st) {
             case 5: slot = S_RI_ARCS; break;
             case 6: slot = S_RI_MOVES; break;
             case 7: slot = S_CLAMPED; break;
-            default: slot = S_RESAT; break;
+            case 8: slot = S_RESAT; break;
+            default: slot = S_WL; break;
         }
         add_ll(&st[slot], (long long)s_sum[threadIdx.x]);
     }
@@ -1612,6 +1769,10 @@ __global__ void __launch_bounds__(kBlock, 1) k_solve(DevGraph G, Job J) {
     extern __shared__ __align__(16) int s_dyn[];
     int *const s_bfs = s_dyn;
     int *const stg = s_dyn + (threadIdx.x >> 5) * kStgWarp;
+    __shared__ volatile unsigned long long s_deadline;           // end of the queue phase (globaltimer)
+    __shared__ unsigned long long s_bfs_begin, s_bfs_end;   // the last BFS, as thread 0 saw it
+    __shared__ int s_fin;   // the queue phase has ended (see the activation queue)
+    if (threadIdx.x == 0) s_fin = 0;
     static_assert(2 * kSoloCap * 4 <= kDynSmem, "the shared frontiers exceed the dynamic shared memory");
     static_assert(kWq * (kBlock / 32) <= 2 * kSoloCap, "frontier stages exceed the shared frontier");
     static_assert(kWq >= 32 * kIlpB, "a stage holds one round of arcs");
@@ -1832,9 +1993,6 @@ __global__ void __launch_bounds__(kBlock, 1) k_solve(DevGraph G, Job J) {
     unsigned snext = stamp_base;   // next unused activation stamp
     for (it = 0; !fast; ++it) {
         const int par = (int)(it & 1);
-        // the stamp of the first PushRelabel pass's queue: the BFS gives it to
-        // the worklist entries it files (queued from the start)
-        const unsigned wmark0 = snext++;
         // height init: t and deficient vertices are sinks (height 0), all
         // others n; the sinks form BFS level 0.
         if (gtid == 0) {
@@ -1903,6 +2061,7 @@ __global__ void __launch_bounds__(kBlock, 1) k_solve(DevGraph G, Job J) {
         // iteration's exit test) are all past this barrier
         if (gtid == 0) C->ri_moved[par ^ 1] = 0;
 
+        if (threadIdx.x == 0) s_bfs_begin = gtimer();
         // backward BFS from the sinks over residual arcs (global relabel),
         // level-synchronous and direction-optimising: top-down from the
         // frontier while it is small, bottom-up from the unvisited vertices
@@ -1950,7 +2109,7 @@ __global__ void __launch_bounds__(kBlock, 1) k_solve(DevGraph G, Job J) {
                     for (;;) {
                         int *ccs = &C->ccnt[Ls % 3];
                         int *spill = (Ls & 1) ? G.qb0 : G.qb1;   // positions >= kSoloCap of the next frontier
-                        Front SF{&s_cnt[b ^ 1], s_front[b ^ 1], &s_arcs[b ^ 1], kSoloCap, spill, nullptr, 0, 0, wmark0};
+                        Front SF{&s_cnt[b ^ 1], s_front[b ^ 1], &s_arcs[b ^ 1], kSoloCap, spill, nullptr, 0, 0};
                         int gs = 32;   // frontier vertices per warp: fewer when they do not fill the warps
                         while (gs > 1 && (gs >> 1) * (kBlock / 32) >= cs) gs >>= 1;
                         for (int grp = cw; grp * gs < cs; grp += kBlock / 32) {
@@ -2038,7 +2197,7 @@ __global__ void __launch_bounds__(kBlock, 1) k_solve(DevGraph G, Job J) {
                 C->asum[(L + 2) % 3] = 0;
                 if (bottom_up) s_stat[S_BU_LEVELS] += 1;
             }
-            Front FR{ncnt, NF, asum, 0x7fffffff, nullptr, s_bfs + (threadIdx.x >> 5) * kWq, 0, 0, wmark0};
+            Front FR{ncnt, NF, asum, 0x7fffffff, nullptr, s_bfs + (threadIdx.x >> 5) * kWq, 0, 0};
             if (bottom_up) {
                 // groups of 32 consecutive vertex ids (warp w: groups w, w + W, ...)
                 const int groups = (n + 31) / 32;
@@ -2120,6 +2279,7 @@ __global__ void __launch_bounds__(kBlock, 1) k_solve(DevGraph G, Job J) {
         }
         if (gtid == 0) s_stat[S_LEVELS] += L;
 
+        if (threadIdx.x == 0) s_bfs_end = gtimer();
         // termination: no active vertex under the fresh BFS heights
         const int nw = lctl(&C->wcnt);
         const int nh = lctl(&C->hcnt);
@@ -2154,6 +2314,8 @@ __global__ void __launch_bounds__(kBlock, 1) k_solve(DevGraph G, Job J) {
         // ever processed by two warps at once.  High-degree vertices that a
         // pass turns active again form the hub list of the next pass.
         const unsigned rstamp_it = snext++;   // relabel-list stamp of this iteration
+        Relabelled RL;
+        RL.stamp = rstamp_it;
         if (gtid == 0) {
             C->qcnt[0] = 0;
             C->asum[0] = 0;
@@ -2161,16 +2323,15 @@ __global__ void __launch_bounds__(kBlock, 1) k_solve(DevGraph G, Job J) {
         bool rounds_clean = true;   // the last activation round left no active vertex
         bool hubs_clean = true;     // the last hub cycle left no hub active
         int pend = 0;               // hubs that the last pass turned active
-        // Rounds per pass: kMaxRounds, and past that, while the list holds at
+        // Rounds per pass (topology-driven mode): kMaxRounds, and past that, while the list holds at
         // most one vertex per warp, as many as the BFS just run had levels --
         // such a round costs about what a BFS level costs, so on deep graphs
         // (grids) finishing a few active vertices by rounds is cheaper than
         // another global relabel.
-        const int max_rounds = L > kMaxRounds ? L : kMaxRounds;
+const int max_rounds = L > kMaxRounds ? L : kMaxRounds;
         for (int pass = 0; pass < (PP ? kMaxPassesPP : kMaxPasses); ++pass) {
             const int *HL = (pass & 1) ? G.hl2 : G.hl;
             const int nhp = pass == 0 ? nh : pend;
-            const unsigned wstamp = pass == 0 ? wmark0 : snext++;   // this pass's round-0 list / queue
             const unsigned hstamp = snext++;   // the next pass's hub list
             int *const pcnt = &C->phc[(pass + 1) & 1];
             // pass 0 appends to phc[1] and starts its rounds on the counters
@@ -2190,8 +2351,7 @@ __global__ void __launch_bounds__(kBlock, 1) k_solve(DevGraph G, Job J) {
             // the data-driven and push-pull modes run PushRelabel from the
             // activation queue; the topology-driven mode in rounds
             const bool qmode = jmode != MF_MODE_TOPOLOGY && G.aq != nullptr;
-            const ActList AL0{&C->wcnt, G.wl,   wstamp,     rstamp_it, pcnt, (pass & 1) ? G.hl : G.hl2,
-                              hstamp,   qmode ? G.aq : nullptr, G.qc, 0, max_rounds, C};
+            ActList AL{pcnt, (pass & 1) ? G.hl : G.hl2, hstamp, qmode ? G.aq : nullptr, G.qc, 0, kMaxGen, &s_deadline, C, 0};
             bool pass_hubs_clean = true;
             if (nhp > 0) {
                 pass_hubs_clean = false;
@@ -2349,11 +2509,11 @@ __global__ void __launch_bounds__(kBlock, 1) k_solve(DevGraph G, Job J) {
                         if (fresh || lcg(reinterpret_cast<const int *>(&G.hikey[w])) == hh) {
                             const unsigned char *ptc = stage == 1 ? G.part : nullptr;
                             if (pull) {
-                                const long long got = hub_move_item<true>(G, item.y, a1, hh, &G.hrem[i], AL0, ptc,
+                                const long long got = hub_move_item<true>(G, item.y, a1, hh, &G.hrem[i], AL, ptc,
                                                                           side, stage != 1, K);
                                 if (lane == 0 && got) add_ll(&G.e[u], got);
                             } else {
-                                const long long sent = hub_move_item<false>(G, item.y, a1, hh, &G.hrem[i], AL0,
+                                const long long sent = hub_move_item<false>(G, item.y, a1, hh, &G.hrem[i], AL,
                                                                             ptc, side, stage != 1, K);
                                 if (lane == 0 && sent) add_ll(&G.e[u], -sent);
                             }
@@ -2379,6 +2539,8 @@ __global__ void __launch_bounds__(kBlock, 1) k_solve(DevGraph G, Job J) {
                             for (int q = lane; q < nit; q += 32) next_items[pos + q] = make_int2(i, beg + q * kPrChunk);
                         }
                     }
+                    if (AL.count && lane == 0) atomicAdd(&C->wcnt, AL.count);   // (topology-driven mode)
+                    AL.count = 0;
                     MF_SYNC_T(S_T_HUB, c, 3, lctl(&C->hub_act[c & 1]));
                     if (gtid == 0 && fresh) C->hccnt = 0;
                     if (lctl(&C->hub_act[c & 1]) == 0) {
@@ -2394,25 +2556,35 @@ __global__ void __launch_bounds__(kBlock, 1) k_solve(DevGraph G, Job J) {
                 // PushRelabel from the activation queue, without rounds: the
                 // worklist entries (generation 0) are dealt to the warps by
                 // stride, then each warp takes a ticket for the next queued
-                // entry and waits for it; a vertex that a push turns active is
-                // queued at once with the next generation and taken by the next
-                // free warp, so a slow vertex holds up only the vertices it
-                // activates.  The phase ends when every queued entry has been
-                // processed (the warp whose completion makes the count of
-                // processed entries equal to the count of queued ones raises
-                // aq_fin).  Generations stand for the activation rounds: none
-                // past max_rounds is queued.  One grid barrier at the end.
+                // entry and waits for it; of the vertices that a visit turns
+                // active the warp serves one itself (visit_chain_t) and queues
+                // the others at once with the next generation, for the next
+                // free warps.  The phase ends when every queued entry has been
+                // processed: a warp counts what it has finished when it finds
+                // no entry ready, and the one that makes the counts equal
+                // raises aq_fin.  One warp per CTA polls that word and tells
+                // the others in shared memory.  One grid barrier at the end.
+                //
+                // How long it goes on: what another global relabel costs is
+                // known, the BFS has just been timed, so the queue gets
+                // kQueueShare of that time and then leaves what is still active
+                // to the next iteration (neither side can then cost much more
+                // than the better choice would have).  Generations below
+                // kMinGen are served in any case, so every iteration makes
+                // progress.
                 const int n0 = cnt;
+                if (threadIdx.x == 0) s_deadline = gtimer() + (s_bfs_end - s_bfs_begin) * kQueueShareNum / kQueueShareDen;
+                __syncthreads();
+                int ndone = 0;   // entries finished and not yet counted (warp-uniform)
                 for (int i = gwarp;; i += nwarps) {
                     int u = -1, gen = 0;
                     if (i < n0) {
                         u = bcast_ld(&G.wl[i]);
                     } else {
-                        int q = 0;
                         unsigned long long slot = 0;
                         if (lane == 0) {
-                            q = atomicAdd(&C->aq_head, 1);
-                            const unsigned long long t0 = gtimer();
+                            const int q = atomicAdd(&C->aq_head, 1);
+                            unsigned long long t0 = 0;
                             unsigned ns = 32;
                             for (int k = 0;; ++k) {
                                 if (q < G.qc) {
@@ -2422,95 +2594,96 @@ __global__ void __launch_bounds__(kBlock, 1) k_solve(DevGraph G, Job J) {
                                         break;
                                     }
                                 }
-                                if ((k & 3) == 3 && ld_acquire_s32(&C->aq_fin)) break;
-                                if (gtimer() - t0 > kWaitNs) {
-                                    atomicOr(&C->status, ST_WAIT);
+                                if (ndone) {
+                                    // the finished entries' own enqueues, and (by the acquire)
+                                    // those of every entry counted before them, precede the
+                                    // tail read
+                                    int d;
+                                    asm volatile("atom.acq_rel.gpu.global.add.s32 %0, [%1], %2;"
+                                                 : "=r"(d) : "l"(&C->aq_done), "r"(ndone) : "memory");
+                                    if (d + ndone == n0 + ld_acquire_s32(&C->aq_tail)) atomicExch(&C->aq_fin, 1);
+                                    ndone = 0;
+                                }
+                                if (threadIdx.x == 0) {
+                                    if (ld_acquire_s32(&C->aq_fin)) {
+                                        *(volatile int *)&s_fin = 1;
+                                        break;
+                                    }
+                                } else if (*(volatile int *)&s_fin) {
                                     break;
                                 }
+                                if ((k & 15) == 15) {
+                                    if (t0 == 0) t0 = gtimer();
+                                    if (gtimer() - t0 > kWaitNs) {
+                                        atomicOr(&C->status, ST_WAIT);
+                                        *(volatile int *)&s_fin = 1;
+                                        break;
+                                    }
+                                }
                                 __nanosleep(ns);
-                                ns = ns < 1024 ? 2 * ns : ns;
+                                ns = ns < 256 ? 2 * ns : ns;
                             }
                         }
+                        ndone = __shfl_sync(kFull, ndone, 0);
                         slot = __shfl_sync(kFull, slot, 0);
                         if (!slot) break;   // every entry processed (or a wait gave up)
                         u = (int)(slot & 0xffffffffu) - 1;
                         gen = (int)(slot >> 32);
                     }
-                    const ActList AL{nullptr, nullptr, wstamp, rstamp_it, pcnt, AL0.hlist, hstamp,
-                                     G.aq,    G.qc,    gen + 1, max_rounds, C};
+                    AL.gen = gen + 1;
                     if (!vertex_ok(J, C, u, n)) {
                         // skipped; still counted as processed below
+                    } else if (gen >= kMinGen && __any_sync(kFull, gtimer() > s_deadline)) {
+                        if (lane == 0) C->aq_over = 1;   // left active
                     } else if (stage == 1) {
                         const unsigned char side = G.part[u];
                         if (side == kPartS)
-                            push_relabel_warp_t<true>(G, u, kc, AL, G.part, side, stg, K);
+                            visit_chain_t<true>(G, u, kc, AL, G.part, side, stg, RL, K);
                         else
-                            push_relabel_warp_t<false>(G, u, kc, AL, G.part, side, stg, K);
+                            visit_chain_t<false>(G, u, kc, AL, G.part, side, stg, RL, K);
                     } else {
-                        push_relabel_warp(G, u, kc, AL, stg, K);
+                        visit_chain(G, u, kc, AL, stg, RL, K);
                     }
-                    if (lane == 0) {
-                        // this entry's own enqueues, and (by the acquire) those
-                        // of every entry counted before it, precede the tail read
-                        const int d = arrive_acq_rel(&C->aq_done) + 1;
-                        if (d == n0 + ld_acquire_s32(&C->aq_tail)) atomicExch(&C->aq_fin, 1);
-                    }
+                    ++ndone;
                 }
+                if (RL.cnt) relabelled_flush(G, RL);
                 MF_SYNC_T(S_T_PRW, 0, 0, cnt + lctl(&C->aq_tail));
+                if (lctl(&C->status) & ST_WAIT) return;   // a wait gave up: the queue's state is undefined
+                if (threadIdx.x == 0) s_fin = 0;
                 pass_rounds_clean = lctl(&C->aq_over) == 0;
-                if (gtid == 0) {
-                    s_stat[S_ROUNDS] += lctl(&C->aq_maxgen) + 1;
-                    s_stat[S_WL] += cnt + lctl(&C->aq_tail);
-                }
+                if (gtid == 0) s_stat[S_ROUNDS] += lctl(&C->aq_maxgen) + 1;
                 // (the counters are zeroed for the next pass after its set-up
                 // barrier, when every thread has read them)
             } else if (!qmode && (cnt > 0 || (pass == 0 && jmode == MF_MODE_TOPOLOGY))) {
                 pass_rounds_clean = false;
-                const int *list = G.wl;
                 for (int rd = 0;; ++rd) {
-                    int *nlist = (rd & 1) ? G.qb0 : G.qb1;
-                    const ActList AL{&C->acnt[(rd + 1) % 3], nlist, snext++, rstamp_it, pcnt, AL0.hlist, hstamp};
+                    // topology-driven (Sec. 5.2): every round visits every
+                    // vertex id and serves the active ones, each warp 32 ids
+                    // at a time (no worklist: the counts only tell whether
+                    // another round has work)
+                    int *const ncnt = &C->acnt[(rd + 1) % 3];
                     if (gtid == 0) {
                         C->acnt[(rd + 2) % 3] = 0;
                         s_stat[S_ROUNDS] += 1;
-                        s_stat[S_WL] += cnt;
                     }
-                    if (jmode == MF_MODE_TOPOLOGY) {
-                        // topology-driven (Sec. 5.2): every round visits every
-                        // vertex id and serves the active ones, each warp 32 ids
-                        // at a time (no worklist: the round lists only tell
-                        // whether another round has work)
-                        for (int grp = gwarp; grp * 32 < n; grp += nwarps) {
-                            const int base = grp * 32;
-                            const int v = base + lane;
-                            bool act = false;
-                            if (v < n && v != s && v != t && __ldg(&G.row[v + 1]) - __ldg(&G.row[v]) <= kHubDeg)
-                                act = lcg(&G.h[v]) < n && lcg(&G.e[v]) > 0;
-                            unsigned mask = __ballot_sync(kFull, act);
-                            while (mask) {
-                                const int j = __ffs(mask) - 1;
-                                mask &= mask - 1u;
-                                push_relabel_warp(G, base + j, kc, AL, stg, K);
-                            }
+                    for (int grp = gwarp; grp * 32 < n; grp += nwarps) {
+                        const int base = grp * 32;
+                        const int v = base + lane;
+                        bool act = false;
+                        if (v < n && v != s && v != t && __ldg(&G.row[v + 1]) - __ldg(&G.row[v]) <= kHubDeg)
+                            act = lcg(&G.h[v]) < n && lcg(&G.e[v]) > 0;
+                        unsigned mask = __ballot_sync(kFull, act);
+                        while (mask) {
+                            const int j = __ffs(mask) - 1;
+                            mask &= mask - 1u;
+                            visit_chain(G, base + j, kc, AL, stg, RL, K);
                         }
-                    } else if (stage == 1) {
-                        // push-pull: push on T (h+), pull on S (h-), each side
-                        // only over arcs within it
-                        for (int i = gwarp; i < cnt; i += nwarps) {
-                            const int u = lcg(&list[i]);
-                            const unsigned char side = G.part[u];
-                            if (side == kPartS)
-                                push_relabel_warp_t<true>(G, u, kc, AL, G.part, side, stg, K);
-                            else
-                                push_relabel_warp_t<false>(G, u, kc, AL, G.part, side, stg, K);
-                        }
-                    } else {
-                        for (int i = gwarp; i < cnt; i += nwarps)
-                            push_relabel_warp(G, lcg(&list[i]), kc, AL, stg, K);
                     }
+                    if (RL.cnt) relabelled_flush(G, RL);
+                    if (AL.count && lane == 0) atomicAdd(ncnt, AL.count);
+                    AL.count = 0;
                     MF_SYNC_T(S_T_PRW, rd, 0, cnt);
-                    cnt = lctl(AL.cnt);
-                    list = nlist;
+                    cnt = lctl(ncnt);
                     if (cnt == 0) pass_rounds_clean = true;
                     if (cnt == 0 || rd + 1 >= max_rounds || (rd + 1 >= kMaxRounds && cnt > nwarps)) break;
                 }
