@@ -101,6 +101,12 @@ constexpr int kMaxPassesPP = 4;
 // CTA 0 alone, with the frontiers in shared memory
 constexpr long long kSoloArcs = 8192;
 constexpr int kSoloCap = 4096;
+// Above this many hubs the cycles file no activations and one pass over all
+// vertices finds the active ones (7-10 us on 2^20 vertices); filing made every
+// pushing item wait for its atomics, a stamp, a fence and a queue reservation
+// (measured on RMAT-20 100k batches with ~2,000 hubs: 38 -> 29 us per push
+// phase).  A few hubs are better off filing.
+constexpr int kDeferHubs = 128;
 constexpr int kPassHubs = 32;   // most re-activated hubs a further pass takes
 constexpr int kPassHubsPP = 64;
 
@@ -124,9 +130,9 @@ struct Ctl {
     unsigned bseq;        // sequence number of the last batch (duplicate-id stamps)
     int wcnt;             // (z) active worklist size (vertices of degree <= kHubDeg)
     int hcnt;             // (z) active hub list size (degree > kHubDeg)
-    int hccnt;            // (z) hub work items
-    int hub_act[2];       // (z) hubs still active in the current hub cycle
-    int hlc[2];           // (z) live hub items for the next cycle, double-buffered
+    int hub_live[2];      // (z) hubs and items of a hub cycle's list, by cycle parity
+    int hub_items[2];     // (z)
+    int hub_act[2];       // (z) hubs still active after a short list's pushes, by cycle parity
     int pad0;
     long long dacc[2];    // (z) sum of deficits at the last height init
     long long iters;
@@ -154,15 +160,19 @@ struct Ctl {
     long long solo_seen;  // frontier arcs counted up to that level
     long long st[S_COUNT_MAX];  // statistics, see enum Stat
     long long st_aux[S_COUNT_MAX];  // where a JOB_REFRESH counts, keeping st intact
-    // the activation queue of a PushRelabel phase (see k_solve): consumer
-    // tickets, producer reservations and finished entries, each on its own
-    // 128-byte line (every warp of the grid polls or bumps them)
-    alignas(128) int aq_head;   // (z)
-    alignas(128) int aq_tail;   // (z)
-    alignas(128) int aq_done;   // (z)
-    alignas(128) int aq_over;   // (z) an active vertex was left out (generation cap, full queue)
-    int aq_maxgen;              // (z) highest generation enqueued
-    alignas(128) int aq_fin;    // (z) every queued entry has been processed
+    // the activation queue of a PushRelabel phase (see k_solve), one set per
+    // pass parity: consumer tickets, producer reservations and finished
+    // entries, each on its own 128-byte line (every warp of the grid polls or
+    // bumps them)
+    struct Queue {
+        alignas(128) int head;   // (z)
+        alignas(128) int tail;   // (z)
+        alignas(128) int done;   // (z)
+        alignas(128) int over;   // (z) an active vertex was left out (time, full queue)
+        int maxgen;              // (z) highest generation enqueued
+        alignas(128) int fin;    // (z) every queued entry has been processed
+        __device__ void clear() { head = tail = done = over = maxgen = fin = 0; }
+    } q[2];
     long long chk_where;        // first failed debug check: kind << 40 | index (kept until mf_solve)
 };
 
@@ -194,14 +204,13 @@ struct DevGraph {
     unsigned *stamp;
     int *qb0, *qb1, *wl;
     int2 *cb;
-    int *hl, *hmode;          // active hubs; per-hub cycle state
+    int *hl;                  // active hubs
     int *hl2;                 // hub list of odd PushRelabel passes
     int2 *hri;                // RemoveInvalidEdges items of relabelled hubs (vertex, first arc)
-    int *hnit, *hdone;        // per-hub work items, and items finished in the cycle
-    int2 *hcl;                // hub work items (hub index, first arc)
-    int2 *hlv0, *hlv1;        // items of the hubs still active, per cycle (double buffer)
-    unsigned *hikey;          // lowest residual-neighbour height per item of the current cycle
-    unsigned long long *hkey; // per-hub lowest (height, arc) key
+    int *hlist0, *hlist1;     // hubs of a cycle's list (indices into hl or hl2), by cycle parity
+    int4 *hit0, *hit1;        // their work items (HubItem), by cycle parity
+    int *hikey;               // lowest residual-neighbour height per item of the current cycle
+    int *hkey;                // per hub, by cycle parity (two each)
     long long *hrem;          // per-hub excess left to push in the current cycle
     TraceRec *trace;          // per-barrier trace records, or null
     int trace_cap;
@@ -238,6 +247,12 @@ struct Job {
 __device__ __forceinline__ int lcg(const int *p) { return __ldcg(p); }
 __device__ __forceinline__ long long lcg(const long long *p) { return __ldcg(p); }
 __device__ __forceinline__ int2 lcg(const int2 *p) { return __ldcg(p); }
+
+// The height of a vertex in a phase that does not depend on heights written
+// during it (see the callers): a plain load, which L1 may serve.
+__device__ __forceinline__ int lheight(const int *p) {
+    return __ldca(p);
+}
 
 __device__ __forceinline__ void add_ll(long long *p, long long v) {
     atomicAdd(reinterpret_cast<unsigned long long *>(p), static_cast<unsigned long long>(v));
@@ -604,7 +619,7 @@ __device__ __forceinline__ void bfs_visit_n(const DevGraph &G, const int (&a)[kI
         K.bfs_arcs += ok[j];
     }
 #pragma unroll
-    for (int j = 0; j < kIlpB; ++j) hv[j] = (rin[j] > 0 && v[j] != G.s) ? lcg(&G.h[v[j]]) : -1;
+    for (int j = 0; j < kIlpB; ++j) hv[j] = (rin[j] > 0 && v[j] != G.s) ? lheight(&G.h[v[j]]) : -1;
 #pragma unroll
     for (int j = 0; j < kIlpB; ++j) disc[j] = hv[j] == n && atomicCAS(&G.h[v[j]], n, L + 1) == n;
     bfs_discovered_n(G, disc, v, fwd, dual, F, K);
@@ -730,7 +745,7 @@ __device__ __forceinline__ void bfs_bottom_up_group(const DevGraph &G, int base,
             unsigned hit = 0;
 #pragma unroll
             for (int jj = 0; jj < kIlpB; ++jj)
-                if (ra[jj] > 0 && lcg(&G.h[w[jj]]) == L &&
+                if (ra[jj] > 0 && lheight(&G.h[w[jj]]) == L &&
                     (!dual || G.part[w[jj]] == (((pull_lanes >> own[jj]) & 1u) ? kPartS : kPartT)))
                     hit |= 1u << own[jj];
             found |= __reduce_or_sync(kFull, hit);
@@ -765,7 +780,7 @@ __device__ __forceinline__ void bfs_bottom_up_item(const DevGraph &G, int2 item,
             bool mine = false;
 #pragma unroll
             for (int j = 0; j < kIlpB; ++j)
-                mine |= R.ra[j] > 0 && lcg(&G.h[R.w[j]]) == L && (!dual || G.part[R.w[j]] == side);
+                mine |= R.ra[j] > 0 && lheight(&G.h[R.w[j]]) == L && (!dual || G.part[R.w[j]] == side);
             hit = __any_sync(kFull, mine);
         }
         if (hit && lane == 0) disc = atomicCAS(&G.h[v], G.n, L + 1) == G.n;
@@ -809,6 +824,15 @@ __device__ __forceinline__ long long pull_arc(const DevGraph &G, int a, int b, i
     return (long long)atomicAdd(reinterpret_cast<unsigned long long *>(&G.e[v]), (unsigned long long)(-(long long)d));
 }
 
+// debug_checks: record a failed check (the first one's kind and index) and
+// make the state invalid until the next mf_solve; the caller skips the
+// access.  Kinds: 1 list entry out of range, 2 excess != net inflow, 3
+// residual pair or mirror inconsistent.
+__device__ __forceinline__ void check_fail(Ctl *C, int kind, long long where) {
+    if ((atomicOr(&C->status, ST_CHECK) & ST_CHECK) == 0)
+        C->chk_where = ((long long)kind << 40) | (where & 0xffffffffffll);
+}
+
 // Where the vertices that a push makes active go.
 //
 // Worklist vertices (degree <= kHubDeg), in the data-driven and push-pull
@@ -830,8 +854,9 @@ struct ActList {
     unsigned long long *aq;     // activation queue, or nullptr: count only
     int qc, gen, gen_cap;       // its capacity; generation of what is filed, and the first one not queued
     const volatile unsigned long long *deadline;   // shared: when the phase ends (globaltimer)
-    Ctl *C;
+    Ctl::Queue *Q;
     int count;                  // filed without a queue (warp-uniform)
+    bool defer;                 // hub cycles: file nothing, a scan finds the active vertices
 };
 
 // Enqueue the lanes' flagged vertices of N slots into the activation queue
@@ -852,7 +877,7 @@ __device__ __forceinline__ void aq_push_n(const ActList &AL, const bool (&pred)[
     }
     if (tot == 0) return;
     int base = 0;
-    if (lane == 0) base = atomicAdd(&AL.C->aq_tail, tot);
+    if (lane == 0) base = atomicAdd(&AL.Q->tail, tot);
     base = __shfl_sync(kFull, base, 0);
     int over = 0;
     const unsigned long long tag = (unsigned long long)(unsigned)AL.gen << 32;
@@ -868,23 +893,23 @@ __device__ __forceinline__ void aq_push_n(const ActList &AL, const bool (&pred)[
     if (base > AL.qc) {   // warp-uniform: base is now past the warp's last entry
         over = (int)warp_sum((long long)over);
         if (lane == 0) {
-            atomicAdd(&AL.C->aq_done, over);
-            atomicExch(&AL.C->aq_over, 1);
+            atomicAdd(&AL.Q->done, over);
+            atomicExch(&AL.Q->over, 1);
         }
     }
-    if (lane == 0) atomicMax(&AL.C->aq_maxgen, AL.gen);
+    if (lane == 0) atomicMax(&AL.Q->maxgen, AL.gen);
 }
 
 // Single-thread enqueue of v (as aq_push_n).
 __device__ __forceinline__ void aq_push_one(const ActList &AL, int v) {
-    const int pos = atomicAdd(&AL.C->aq_tail, 1);
+    const int pos = atomicAdd(&AL.Q->tail, 1);
     if (pos < AL.qc) {
         st_relaxed_u64(&AL.aq[pos], ((unsigned long long)(unsigned)AL.gen << 32) | (unsigned)(v + 1));
     } else {
-        atomicAdd(&AL.C->aq_done, 1);
-        atomicExch(&AL.C->aq_over, 1);
+        atomicAdd(&AL.Q->done, 1);
+        atomicExch(&AL.Q->over, 1);
     }
-    atomicMax(&AL.C->aq_maxgen, AL.gen);
+    atomicMax(&AL.Q->maxgen, AL.gen);
 }
 
 // File hubs that moves turned active.  All 32 lanes call.
@@ -918,7 +943,7 @@ __device__ __forceinline__ void file_activations(const DevGraph &G, bool (&add)[
         return;
     }
     if (AL.gen >= AL.gen_cap) {
-        if ((threadIdx.x & 31) == 0) atomicExch(&AL.C->aq_over, 1);
+        if ((threadIdx.x & 31) == 0) atomicExch(&AL.Q->over, 1);
         return;
     }
     __syncwarp();
@@ -978,7 +1003,7 @@ __device__ __forceinline__ void load_round_t(const DevGraph &G, int a0, int end,
     }
 #pragma unroll
     for (int j = 0; j < kIlp; ++j) {
-        R.hv[j] = R.ra[j] > 0 ? lcg(&G.h[R.v[j]]) : 0;
+        R.hv[j] = R.ra[j] > 0 ? lheight(&G.h[R.v[j]]) : 0;
         R.rb[j] = (REV && R.ra[j] > 0) ? __ldg(&G.rev[a0 + 32 * j + lane]) : 0;
     }
 }
@@ -991,64 +1016,11 @@ __device__ __forceinline__ int round_arcs(int a0, int end) {
     return c;
 }
 
-// Lowest (height, arc offset from beg) key over the residual arcs of a round.
-__device__ __forceinline__ unsigned long long round_min_key(const ArcRound &R, int a0, int beg) {
-    const int lane = threadIdx.x & 31;
-    unsigned long long best = ~0ull;
-#pragma unroll
-    for (int j = 0; j < kIlp; ++j) {
-        if (R.ra[j] > 0) {
-            const unsigned long long key =
-                ((unsigned long long)(unsigned)R.hv[j] << 32) | (unsigned)(a0 + 32 * j + lane - beg);
-            best = key < best ? key : best;
-        }
-    }
-    return best;
-}
-
 // The amount moved along arc a (u -> v, reverse b) in one step: a push or a
 // pull.
 template <bool PULL>
 __device__ __forceinline__ long long move_arc(const DevGraph &G, int a, int b, int v, int d) {
     return PULL ? pull_arc(G, a, b, v, d) : push_arc(G, a, b, v, d);
-}
-
-// The moves of one round (d[j] > 0: d[j] units along slot j of R, a round
-// loaded with its reverse arcs), and the filing of the vertices they turn
-// active: a push that raised e(v) above 0 (a pull that lowered it below 0)
-// makes v active, and v (not s or t) is filed (ActList) as a worklist vertex
-// when its degree is <= kHubDeg, else as a hub.  The
-// heads' degrees load beside the move atomics, so the filing waits once for
-// both; v's height is the one the scan read (a push only goes below h(u) <
-// n).  Each list gets one reservation per warp.  Returns this lane's total
-// moved.  All 32 lanes call.
-template <bool PULL>
-__device__ __forceinline__ long long move_round(const DevGraph &G, int a0, const int (&d)[kIlp], const ArcRound &R,
-                                                ActList &AL, Counters &K) {
-    const int lane = threadIdx.x & 31;
-    long long old[kIlp], sent = 0;
-    int deg[kIlp];
-#pragma unroll
-    for (int j = 0; j < kIlp; ++j) {
-        old[j] = 0;
-        deg[j] = 0;
-        if (d[j] > 0) {
-            old[j] = move_arc<PULL>(G, a0 + 32 * j + lane, R.rb[j], R.v[j], d[j]);
-            deg[j] = __ldg(&G.row[R.v[j] + 1]) - __ldg(&G.row[R.v[j]]);
-            sent += d[j];
-            ++K.push;
-        }
-    }
-    bool add[kIlp], add_hub[kIlp];
-#pragma unroll
-    for (int j = 0; j < kIlp; ++j) {
-        const bool turned = PULL ? (old[j] >= 0 && old[j] - d[j] < 0) : (old[j] <= 0 && old[j] + d[j] > 0);
-        const bool cand = d[j] > 0 && turned && R.v[j] != G.s && R.v[j] != G.t;
-        add[j] = cand && deg[j] <= kHubDeg;
-        add_hub[j] = cand && deg[j] > kHubDeg;
-    }
-    file_activations(G, add, add_hub, R.v, AL);
-    return sent;
 }
 
 // ------------------------------------------------ staged arc ranges --
@@ -1310,7 +1282,7 @@ __device__ __forceinline__ void visit_chain_t(const DevGraph &G, int u, int kc, 
             if (!AL.aq) {
                 ++AL.count;
             } else if (lane == 0) {
-                if (AL.gen >= AL.gen_cap) atomicExch(&AL.C->aq_over, 1);
+                if (AL.gen >= AL.gen_cap) atomicExch(&AL.Q->over, 1);
                 else aq_push_one(AL, u);
             }
             break;
@@ -1404,7 +1376,7 @@ __device__ __forceinline__ void visit_chain_t(const DevGraph &G, int u, int kc, 
             if (!AL.aq) {
                 ++AL.count;
             } else if (lane == 0) {
-                if (AL.gen >= AL.gen_cap) atomicExch(&AL.C->aq_over, 1);
+                if (AL.gen >= AL.gen_cap) atomicExch(&AL.Q->over, 1);
                 else aq_push_one(AL, u);
             }
             break;
@@ -1450,7 +1422,7 @@ __device__ __forceinline__ void visit_chain_t(const DevGraph &G, int u, int kc, 
         }
         if (AL.gen >= kMinGen && (AL.gen >= AL.gen_cap || __any_sync(kFull, gtimer() > *AL.deadline))) {
             const bool self = __shfl_sync(kFull, maybe && (PULL ? pleft < 0 : pleft > 0), 0);
-            if ((tot || self) && lane == 0) atomicExch(&AL.C->aq_over, 1);
+            if ((tot || self) && lane == 0) atomicExch(&AL.Q->over, 1);
             break;
         }
         // the first of the activated heads is served next by this warp
@@ -1481,7 +1453,7 @@ __device__ __forceinline__ void visit_chain_t(const DevGraph &G, int u, int kc, 
         ++AL.gen;
     }
     __syncwarp();
-    if (AL.aq && lane == 0 && AL.gen > gen0) atomicMax(&AL.C->aq_maxgen, AL.gen - 1);
+    if (AL.aq && lane == 0 && AL.gen > gen0) atomicMax(&AL.Q->maxgen, AL.gen - 1);
 }
 
 __device__ __forceinline__ void visit_chain(const DevGraph &G, int u, int kc, ActList &AL, int *stg, Relabelled &RL,
@@ -1531,64 +1503,318 @@ __device__ __forceinline__ void remove_invalid_warp_t(const DevGraph &G, int u, 
     }
 }
 
-// Hub cycle helpers (the cooperative PushRelabel of high-degree vertices).
-// H1 scan of one kPrChunk-arc item [a0, a1) of hub u (first arc beg): the
-// lowest (height, arc) key over its residual arcs (PULL: arcs into u).
-template <bool PULL>
-__device__ __forceinline__ unsigned long long hub_scan_item(const DevGraph &G, int a0, int a1, int beg,
-                                                            const unsigned char *pt, unsigned char side,
-                                                            Counters &K) {
-    unsigned long long best = ~0ull;
-    for (; a0 < a1; a0 += 32 * kIlp) {
-        ArcRound R;
-        load_round_t<PULL, false>(G, a0, a1, R, pt, side);
-        K.pr_arcs += round_arcs(a0, a1);
-        const unsigned long long k = round_min_key(R, a0, beg);
-        best = k < best ? k : best;
-    }
-    return best;
+// ------------------------------------------------- cooperative hubs --
+// Hubs run PushRelabel over the whole grid in kPrChunk-arc items, in cycles
+// of three phases (hub_list, hub_lowest, hub_push) between grid barriers.  An item's
+// heads and residuals are copied to the warp's shared memory by cp.async one
+// item ahead, and what the item needs of its hub is loaded two and one items
+// ahead, so that an item waits only for the heights of its heads (kHubArcs
+// per lane in flight) and for its share of the hub's excess.  What is decided
+// per hub is decided one hub per lane over the grid: with the last item's warp
+// deciding (arrival counters), a few warps took several decisions of five round
+// trips each while the rest of the grid waited (38 % of the warps' time busy).
+// Bound by the random reads of the heights (~140-240 G/s from L2 measured on
+// hub-heavy index sets; 9.5M arcs a scan).  RMAT-20 100k, per phase: scan 15.6
+// -> 9.9 us, pushes 31.9 -> 22.7 us; the static solve's scan 23.6 -> 13.1,
+// pushes 38.8 -> 27.5 us.
+constexpr int kHubArcs = kPrChunk / 32;    // arcs per lane of an item
+constexpr int kHubBuf = kPrChunk + 8;      // ints per array of a staged item
+static_assert(4 * kHubBuf <= kStgWarp, "two staged hub items per warp");
+
+// x: index in the hub list, y, z: arcs, w: the hub, sign bit: on the pull side
+// of a push-pull repair
+using HubItem = int4;
+__device__ __forceinline__ int hub_of(const HubItem &m) { return m.w & 0x7fffffff; }
+__device__ __forceinline__ bool hub_pull(const HubItem &m) { return m.w < 0; }
+__device__ __forceinline__ HubItem hub_item(const HubItem *items, int w, int nitems) {
+    return w < nitems ? __ldcg(&items[w]) : make_int4(0, 0, 0, 0);
 }
 
-// H3 of one item: moves along the item's residual arcs at height hh, in arc
-// order, each warp reserving its share of what the hub has left to move
-// (*rem) with one atomic.  Returns the amount this warp moved (all lanes).
-template <bool PULL>
-__device__ __forceinline__ long long hub_move_item(const DevGraph &G, int a0, int a1, int hh, long long *rem,
-                                                   ActList &AL, const unsigned char *pt, unsigned char side,
-                                                   bool skip_done, Counters &K) {
-    const int lane = threadIdx.x & 31;
-    long long sent = 0;
-    for (; a0 < a1; a0 += 32 * kIlp) {
-        // the hub's excess may already be reserved by the items before this
-        // one (not checked in the first push-pull stage, where scanning every
-        // item measured faster: its pushes spread over the hub's arcs)
-        if (skip_done && bcast_ld(rem) <= 0) break;
-        ArcRound R;
-        // (the arcs H1 scanned in this cycle: not counted again)
-        load_round_t<PULL, true>(G, a0, a1, R, pt, side);
-        int ra[kIlp];
-        long long incl[kIlp], tot = 0;
+__device__ __forceinline__ void hub_issue(const DevGraph &G, const HubItem &m, int *buf) {
+    stage_copy(G.head, buf, m.y, m.z, G.A, G.al16);
+    stage_copy(hub_pull(m) ? G.rr : G.r, buf + kHubBuf, m.y, m.z, G.A, G.al16);
+}
+
+// Heights of the heads of the staged item's residual arcs, lane i holding arcs
+// y + 32 j + i (INT_MAX: no residual arc, or, with a partition array, a head
+// in another part); returns the lane's lowest.
+__device__ __forceinline__ unsigned hub_heights(const DevGraph &G, const HubItem &m, const int *buf,
+                                                const unsigned char *pt, int (&hv)[kHubArcs]) {
+    const int at = (m.y & 3) + (threadIdx.x & 31), cnt = m.z - m.y - (threadIdx.x & 31);
+    const unsigned char side = hub_pull(m) ? kPartS : kPartT;
+    unsigned lo = INT_MAX;
 #pragma unroll
-        for (int j = 0; j < kIlp; ++j) {
-            ra[j] = (R.ra[j] > 0 && R.hv[j] == hh) ? R.ra[j] : 0;
-            incl[j] = warp_incl_scan(ra[j]) + tot;   // arc order: round j, then lane
-            tot = __shfl_sync(kFull, incl[j], 31);
-        }
-        if (tot == 0) continue;
-        long long old = 0;
-        if (lane == 0)
-            old = (long long)atomicAdd(reinterpret_cast<unsigned long long *>(rem), (unsigned long long)(-tot));
-        old = __shfl_sync(kFull, old, 0);
-        if (old <= 0) break;
-        int d[kIlp];
-#pragma unroll
-        for (int j = 0; j < kIlp; ++j) {
-            const long long dj = old - (incl[j] - ra[j]);
-            d[j] = dj < 0 ? 0 : (dj > ra[j] ? ra[j] : (int)dj);
-        }
-        sent += move_round<PULL>(G, a0, d, R, AL, K);
+    for (int j = 0; j < kHubArcs; ++j) {
+        const bool res = 32 * j < cnt && buf[kHubBuf + at + 32 * j] > 0;
+        const int v = res ? buf[at + 32 * j] : 0;
+        hv[j] = res ? lheight(&G.h[v]) : INT_MAX;
+        if (pt && res && pt[v] != side) hv[j] = INT_MAX;
     }
-    return warp_sum(sent);
+#pragma unroll
+    for (int j = 0; j < kHubArcs; ++j) lo = min(lo, (unsigned)hv[j]);
+    return lo;
+}
+
+// The item list of a cycle of parity par: the items of the hubs of the last
+// cycle's list (of HL, in the first cycle; cnt hubs) that are active now, kHubsPerWarp hubs per
+// warp, one per lane.  Sets what the cycle needs of each: hrem (the amount to
+// move) and hkey (by cycle parity: the lowest residual-neighbour height, to
+// be found; when the heights are those of the BFS just run (fresh), u's
+// lowest residual neighbour sits one level below it, and no scan is needed).
+// The hubs themselves are listed in hlist, by cycle parity.
+constexpr int kHubsPerWarp = 8;
+template <bool PP>
+__device__ __forceinline__ void hub_list(const DevGraph &G, const int *HL, int par, int cnt, bool first, bool fresh,
+                                         const unsigned char *pt, int gwarp, int nwarps, bool check) {
+    const int lane = threadIdx.x & 31;
+    HubItem *items = par ? G.hit1 : G.hit0;
+    const int *from = par ? G.hlist0 : G.hlist1;
+    int *to = par ? G.hlist1 : G.hlist0;
+    for (int k0 = gwarp * kHubsPerWarp; k0 < cnt; k0 += nwarps * kHubsPerWarp) {
+        const int k = k0 + lane;
+        int i = 0, u = 0, beg = 0, end = 0, tag = 0, h = G.n;
+        long long e = 0;
+        if (lane < kHubsPerWarp && k < cnt) {
+            i = first ? k : lcg(&from[k]);
+            u = lcg(&HL[i]);
+            if (check && (u < 0 || u >= G.n)) {
+                check_fail(G.ctl, 1, u);
+            } else {
+                beg = __ldg(&G.row[u]);
+                end = __ldg(&G.row[u + 1]);
+                h = lcg(&G.h[u]);
+                e = lcg(&G.e[u]);
+                tag = u;
+                if (PP && pt && pt[u] == kPartS) {
+                    tag |= (int)0x80000000u;
+                    e = -e;
+                }
+            }
+        }
+        const bool live = h < G.n && e > 0;
+        const unsigned m = __ballot_sync(kFull, live);
+        if (!m) continue;
+        const int nit = live ? (end - beg + kPrChunk - 1) / kPrChunk : 0;
+        const int incl = (int)warp_incl_scan(nit);
+        int pos = 0, base = 0;
+        if (lane == 0) base = atomicAdd(&G.ctl->hub_live[par], __popc(m));
+        if (lane == 31) pos = atomicAdd(&G.ctl->hub_items[par], incl);
+        base = __shfl_sync(kFull, base, 0);
+        pos = __shfl_sync(kFull, pos, 31) + incl - nit;
+        if (live) {
+            to[base + __popc(m & ((1u << lane) - 1u))] = i;
+            G.hrem[i] = e;
+            G.hkey[2 * i + par] = fresh ? h - 1 : INT_MAX;
+            G.hkey[2 * i + (par ^ 1)] = nit;   // items still to push (hub_push)
+        }
+        for (unsigned r = m; r; r &= r - 1u) {   // the items, all lanes a hub
+            const int src = __ffs(r) - 1;
+            const int n1 = __shfl_sync(kFull, nit, src), p1 = __shfl_sync(kFull, pos, src);
+            const int i1 = __shfl_sync(kFull, i, src), t1 = __shfl_sync(kFull, tag, src);
+            const int b1 = __shfl_sync(kFull, beg, src), e1 = __shfl_sync(kFull, end, src);
+            for (int q = lane; q < n1; q += 32)
+                items[p1 + q] = make_int4(i1, b1 + q * kPrChunk, min(b1 + (q + 1) * kPrChunk, e1), t1);
+        }
+    }
+}
+
+// The lowest residual neighbour of every listed hub (hkey) and item (hikey).
+// No push or relabel runs meanwhile.
+__device__ __forceinline__ void hub_lowest(const DevGraph &G, int nitems, int par, int gwarp, int nwarps, int *stg,
+                                           const unsigned char *pt, Counters &K) {
+    const int lane = threadIdx.x & 31;
+    const HubItem *items = par ? G.hit1 : G.hit0;
+    HubItem cur = hub_item(items, gwarp, nitems), nxt = hub_item(items, gwarp + nwarps, nitems);
+    if (gwarp < nitems) hub_issue(G, cur, stg);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    int b = 0;
+    for (int w = gwarp; w < nitems; w += nwarps) {
+        if (w + nwarps < nitems) hub_issue(G, nxt, stg + (b ^ 1) * 2 * kHubBuf);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        const HubItem nn = hub_item(items, w + 2 * nwarps, nitems);
+        asm volatile("cp.async.wait_group 1;" ::: "memory");
+        __syncwarp();
+        int hv[kHubArcs];
+        unsigned lo = hub_heights(G, cur, stg + b * 2 * kHubBuf, pt, hv);
+        K.pr_arcs += (cur.z - cur.y + 31 - lane) >> 5;
+        lo = __reduce_min_sync(kFull, lo);
+        if (lane == 0) {
+            G.hikey[w] = (int)lo;
+            if (lo < INT_MAX) atomicMin(&G.hkey[2 * cur.x + par], (int)lo);
+        }
+        __syncwarp();   // every lane is done with the item's buffer
+        cur = nxt;
+        nxt = nn;
+        b ^= 1;
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+}
+
+// The decisions of the listed hubs after hub_lowest: a hub that is not above
+// its lowest residual neighbour is relabelled to one above it (to n without
+// one); its pushes follow in the same cycle (a rescan in the next cycle cost a
+// cycle per relabel).  Its items join the iteration's RemoveInvalidEdges list
+// once.  One hub per lane.
+__device__ __forceinline__ void hub_relabel(const DevGraph &G, const int *HL, int par, int cnt, unsigned rstamp,
+                                            int gwarp, int nwarps, Counters &K) {
+    const int lane = threadIdx.x & 31;
+    const int *list = par ? G.hlist1 : G.hlist0;
+    for (int k0 = gwarp * kHubsPerWarp; k0 < cnt; k0 += nwarps * kHubsPerWarp) {
+        const int k = k0 + lane;
+        int u = 0, beg = 0, nit = 0;
+        if (lane < kHubsPerWarp && k < cnt) {
+            const int i = lcg(&list[k]);
+            u = lcg(&HL[i]);
+            const int hh = lcg(&G.hkey[2 * i + par]), hu = lcg(&G.h[u]);
+            if (hu <= hh) {
+                G.h[u] = hh == INT_MAX ? G.n : hh + 1;
+                ++K.relabel;
+                if (atomicExch(&G.rstamp[u], rstamp) != rstamp) {
+                    beg = __ldg(&G.row[u]);
+                    nit = (__ldg(&G.row[u + 1]) - beg + kPrChunk - 1) / kPrChunk;
+                }
+            }
+        }
+        const unsigned m = __ballot_sync(kFull, nit > 0);
+        if (!m) continue;
+        const int incl = (int)warp_incl_scan(nit);
+        int pos = 0;
+        if (lane == 31) pos = atomicAdd(&G.ctl->rhcnt, incl);
+        pos = __shfl_sync(kFull, pos, 31) + incl - nit;
+        for (unsigned r = m; r; r &= r - 1u) {
+            const int src = __ffs(r) - 1;
+            const int n1 = __shfl_sync(kFull, nit, src), p1 = __shfl_sync(kFull, pos, src);
+            const int u1 = __shfl_sync(kFull, u, src), b1 = __shfl_sync(kFull, beg, src);
+            for (int q = lane; q < n1; q += 32) G.hri[p1 + q] = make_int2(u1, b1 + q * kPrChunk);
+        }
+    }
+}
+
+// Moves along the lowest arcs of the listed hubs, each warp reserving its
+// share of the hub's excess with one atomic.  With AL.defer the vertices made
+// active are not filed: the moves are reductions that nothing waits for, and
+// a scan finds the active vertices afterwards (k_solve).  Otherwise the list is
+// short and the warp that finishes a hub's last item looks whether the hub is
+// still active (hub_act): mostly none is, and the next cycle's list phase need
+// not run.  (The count-down is relaxed: an excess read too early reads too
+// high, which only costs that phase.)
+__device__ __forceinline__ void hub_push(const DevGraph &G, int nitems, int par, bool fresh, int gwarp, int nwarps,
+                                         int *stg, const unsigned char *pt, ActList &AL, Counters &K) {
+    const int lane = threadIdx.x & 31;
+    const HubItem *items = par ? G.hit1 : G.hit0;
+    // the height that item m (number w) pushes at, or -1: its hub has no
+    // neighbour below n - 1 or nothing left to move, or no arc at its height here
+    auto push_height = [&](const HubItem &m, int w) {
+        if (w >= nitems) return -1;
+        const int hh = lcg(&G.hkey[2 * m.x + par]);
+        const int key = fresh ? hh : lcg(&G.hikey[w]);
+        const long long rem = lcg(&G.hrem[m.x]);
+        return __shfl_sync(kFull, hh < G.n - 1 && key == hh && rem > 0 ? hh : -1, 0);
+    };
+    HubItem cur = hub_item(items, gwarp, nitems), nxt = hub_item(items, gwarp + nwarps, nitems);
+    int hh = push_height(cur, gwarp);
+    if (hh >= 0) hub_issue(G, cur, stg);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    int hn = push_height(nxt, gwarp + nwarps);
+    int b = 0;
+    for (int w = gwarp; w < nitems; w += nwarps) {
+        if (hn >= 0) hub_issue(G, nxt, stg + (b ^ 1) * 2 * kHubBuf);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        const HubItem nn = hub_item(items, w + 2 * nwarps, nitems);
+        if (hh >= 0) {
+            asm volatile("cp.async.wait_group 1;" ::: "memory");
+            __syncwarp();
+            const int *buf = stg + b * 2 * kHubBuf;
+            const int at = (cur.y & 3) + lane;
+            int hv[kHubArcs], d[kHubArcs], rb[kHubArcs];
+            hub_heights(G, cur, buf, pt, hv);
+            if (fresh) K.pr_arcs += (cur.z - cur.y + 31 - lane) >> 5;   // (else counted by the scan)
+            // d: the exclusive prefix of the item's residual at height hh, in
+            // arc order; sums saturate at 2^31 - 1, the most an item moves
+            unsigned tot = 0;
+#pragma unroll
+            for (int j = 0; j < kHubArcs; ++j) {
+                const unsigned x = hv[j] == hh ? (unsigned)buf[kHubBuf + at + 32 * j] : 0u;
+                rb[j] = x ? __ldg(&G.rev[cur.y + 32 * j + lane]) : 0;
+                d[j] = (int)tot;
+                if (!__any_sync(kFull, x > 0)) continue;   // warp-uniform
+                unsigned incl = x;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const unsigned y = __shfl_up_sync(kFull, incl, o);
+                    if (lane >= o) incl = min(incl + y, (unsigned)INT_MAX);
+                }
+                unsigned excl = __shfl_up_sync(kFull, incl, 1);
+                if (lane == 0) excl = 0;
+                d[j] = (int)min(tot + excl, (unsigned)INT_MAX);
+                tot = min(tot + __shfl_sync(kFull, incl, 31), (unsigned)INT_MAX);
+            }
+            long long got = 0;
+            if (tot) {
+                if (lane == 0)
+                    got = (long long)atomicAdd(reinterpret_cast<unsigned long long *>(&G.hrem[cur.x]),
+                                               (unsigned long long)(-(long long)tot));
+                got = __shfl_sync(kFull, got, 0);
+            }
+            if (got > 0) {   // warp-uniform
+                const unsigned most = got > (long long)tot ? tot : (unsigned)got;
+                const bool pull = hub_pull(cur);
+                long long sent = 0;
+#pragma unroll
+                for (int half = 0; half < kHubArcs; half += 4) {
+                    bool add[4], add_hub[4];
+                    int v[4];
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        const int j = half + q;
+                        add[q] = add_hub[q] = false;
+                        v[q] = 0;
+                        const unsigned x = hv[j] == hh ? (unsigned)buf[kHubBuf + at + 32 * j] : 0u;
+                        const unsigned m = (unsigned)d[j] >= most ? 0u : min(x, most - (unsigned)d[j]);
+                        if (m == 0) continue;
+                        const int a = cur.y + 32 * j + lane;
+                        v[q] = buf[at + 32 * j];
+                        ++K.push;
+                        sent += m;
+                        // a push moves along a, a pull along its reverse
+                        const int x0 = pull ? rb[j] : a, x1 = pull ? a : rb[j];
+                        atomicSub(&G.r[x0], (int)m);
+                        atomicSub(&G.rr[x1], (int)m);
+                        atomicAdd(&G.r[x1], (int)m);
+                        atomicAdd(&G.rr[x0], (int)m);
+                        if (AL.defer || v[q] == G.t || v[q] == G.s) {
+                            add_ll(&G.e[v[q]], pull ? -(long long)m : (long long)m);
+                        } else {
+                            const unsigned long long s = pull ? (unsigned long long)(-(long long)m) : m;
+                            const long long old =
+                                (long long)atomicAdd(reinterpret_cast<unsigned long long *>(&G.e[v[q]]), s);
+                            const bool turned =
+                                pull ? old >= 0 && old < (long long)m : old <= 0 && -old < (long long)m;
+                            const int deg = __ldg(&G.row[v[q] + 1]) - __ldg(&G.row[v[q]]);
+                            add[q] = turned && deg <= kHubDeg;
+                            add_hub[q] = turned && deg > kHubDeg;
+                        }
+                    }
+                    if (!AL.defer) file_activations(G, add, add_hub, v, AL);
+                }
+                sent = warp_sum(sent);
+                if (lane == 0) add_ll(&G.e[hub_of(cur)], pull ? sent : -sent);
+            }
+            __syncwarp();   // every lane is done with the item's buffer
+        }
+        if (!AL.defer && lane == 0 && atomicSub(&G.hkey[2 * cur.x + (par ^ 1)], 1) == 1) {
+            const int u = hub_of(cur);
+            const long long eu = lcg(&G.e[u]);
+            if (lcg(&G.h[u]) < G.n && (hub_pull(cur) ? eu < 0 : eu > 0)) atomicAdd(&G.ctl->hub_act[par], 1);
+        }
+        __syncwarp();
+        cur = nxt;
+        nxt = nn;
+        hh = hn;
+        hn = push_height(nxt, w + 2 * nwarps);
+        b ^= 1;
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
 }
 
 // Add the warp's counters to the statistics st and clear them.  All 32 lanes
@@ -1687,19 +1913,10 @@ __device__ __forceinline__ void bfs_visit_staged(const DevGraph &G, const int *s
         K.bfs_arcs += ok[j];
     }
 #pragma unroll
-    for (int j = 0; j < kIlpB; ++j) hv[j] = (rin[j] > 0 && v[j] != G.s) ? lcg(&G.h[v[j]]) : -1;
+    for (int j = 0; j < kIlpB; ++j) hv[j] = (rin[j] > 0 && v[j] != G.s) ? lheight(&G.h[v[j]]) : -1;
 #pragma unroll
     for (int j = 0; j < kIlpB; ++j) disc[j] = hv[j] == n && atomicCAS(&G.h[v[j]], n, L + 1) == n;
     bfs_discovered_n(G, disc, v, fwd, dual, F, K);
-}
-
-// debug_checks: record a failed check (the first one's kind and index) and
-// make the state invalid until the next mf_solve; the caller skips the
-// access.  Kinds: 1 list entry out of range, 2 excess != net inflow, 3
-// residual pair or mirror inconsistent.
-__device__ __forceinline__ void check_fail(Ctl *C, int kind, long long where) {
-    if ((atomicOr(&C->status, ST_CHECK) & ST_CHECK) == 0)
-        C->chk_where = ((long long)kind << 40) | (where & 0xffffffffffll);
 }
 
 // A vertex id read from a list or queue, checked when debug_checks is on.
@@ -2039,7 +2256,8 @@ __global__ void __launch_bounds__(kBlock, 1) k_solve(DevGraph G, Job J) {
         // height init: t and deficient vertices are sinks (height 0), all
         // others n; the sinks form BFS level 0.
         if (gtid == 0) {
-            C->aq_head = C->aq_tail = C->aq_done = C->aq_over = C->aq_maxgen = C->aq_fin = 0;
+            C->q[0].clear();
+            C->q[1].clear();
             C->qcnt[1] = 0;
             C->qcnt[2] = 0;
             C->ccnt[0] = 0;
@@ -2050,9 +2268,8 @@ __global__ void __launch_bounds__(kBlock, 1) k_solve(DevGraph G, Job J) {
             C->phc[1] = 0;
             C->wcnt = 0;
             C->hcnt = 0;
-            C->hccnt = 0;
+            C->hub_live[0] = C->hub_live[1] = C->hub_items[0] = C->hub_items[1] = 0;
             C->hub_act[0] = C->hub_act[1] = 0;
-            C->hlc[0] = C->hlc[1] = 0;
             C->dacc[par ^ 1] = 0;
             if (gtimer() - C->t_start > J.time_limit_ns) C->abort_loop = 1;
         }
@@ -2372,6 +2589,7 @@ __global__ void __launch_bounds__(kBlock, 1) k_solve(DevGraph G, Job J) {
         // (grids) finishing a few active vertices by rounds is cheaper than
         // another global relabel.
 const int max_rounds = L > kMaxRounds ? L : kMaxRounds;
+        int hub_no = 0;             // hub cycles' lists built in this iteration
         for (int pass = 0; pass < (PP ? kMaxPassesPP : kMaxPasses); ++pass) {
             const int *HL = (pass & 1) ? G.hl2 : G.hl;
             const int nhp = pass == 0 ? nh : pend;
@@ -2379,222 +2597,109 @@ const int max_rounds = L > kMaxRounds ? L : kMaxRounds;
             int *const pcnt = &C->phc[(pass + 1) & 1];
             // pass 0 appends to phc[1] and starts its rounds on the counters
             // zeroed at the iteration's start; a later pass always has hubs,
-            // so its set-up barrier comes before any use of what is zeroed
-            // here (the previous pass's rounds ended with an empty list)
+            // so the barrier of its first list comes before any use of what is
+            // zeroed here (the previous pass's rounds ended with an empty list)
             if (gtid == 0) {
                 if (pass > 0) {
                     *pcnt = 0;
                     C->wcnt = 0;
                     C->acnt[0] = C->acnt[1] = C->acnt[2] = 0;
                 }
-                C->hub_act[0] = C->hub_act[1] = 0;
-                C->hlc[0] = C->hlc[1] = 0;
                 s_stat[S_WL] += nhp;
             }
             // the data-driven and push-pull modes run PushRelabel from the
             // activation queue; the topology-driven mode in rounds
             const bool qmode = jmode != MF_MODE_TOPOLOGY && G.aq != nullptr;
-            ActList AL{pcnt, (pass & 1) ? G.hl : G.hl2, hstamp, qmode ? G.aq : nullptr, G.qc, 0, kMaxGen, &s_deadline, C, 0};
+            ActList AL{pcnt, (pass & 1) ? G.hl : G.hl2, hstamp, qmode ? G.aq : nullptr, G.qc, 0, kMaxGen, &s_deadline,
+                       &C->q[pass & 1], 0, nhp > kDeferHubs};
             bool pass_hubs_clean = true;
             if (nhp > 0) {
                 pass_hubs_clean = false;
-                for (int i = gwarp; i < nhp; i += nwarps) {
-                    const int u = bcast_ld(&HL[i]);
-                    if (!vertex_ok(J, C, u, n)) continue;   // warp-uniform
-                    const int beg = __ldg(&G.row[u]);
-                    const int nc = (__ldg(&G.row[u + 1]) - beg + kPrChunk - 1) / kPrChunk;
-                    int pos = 0;
-                    if (lane == 0) {
-                        pos = atomicAdd(&C->hccnt, nc);
-                        G.hkey[i] = ~0ull;
-                        G.hnit[i] = nc;
-                        G.hdone[i] = 0;
-                        if (pass == 0) {
-                            // right after the BFS a reached vertex's lowest
-                            // residual neighbour sits exactly one level below
-                            // it, so the first cycle's decision needs no scan:
-                            // push to the arcs at height h(u) - 1
-                            const long long eu = lcg(&G.e[u]);
-                            G.hmode[i] = lcg(&G.h[u]);
-                            G.hrem[i] = eu < 0 ? -eu : eu;
-                        } else {
-                            G.hmode[i] = 0;
-                        }
-                    }
-                    pos = __shfl_sync(kFull, pos, 0);
-                    for (int c = lane; c < nc; c += 32) G.hcl[pos + c] = make_int2(i, beg + c * kPrChunk);
-                }
-                MF_SYNC_T(S_T_HUB, -1, 0, nhp);
-                // a later pass's queue: the previous pass's counters have been
-                // read (before this barrier), and nothing is queued before the
-                // first H3 (a later pass's first cycle has an H1 barrier)
-                if (pass > 0 && gtid == 0)
-                    C->aq_head = C->aq_tail = C->aq_done = C->aq_over = C->aq_maxgen = C->aq_fin = 0;
-                const int nhc = lctl(&C->hccnt);
                 const int hub_min = PP ? kMinHubCyclesPP : kMinHubCycles;
                 const int hub_cycles = kc > hub_min ? kc : hub_min;
-                for (int c = 0; c < hub_cycles; ++c) {
-                    if (gtid == 0) s_stat[S_HUB_CYCLES] += 1;
-                    const bool fresh = c == 0 && pass == 0;   // H1 decided by the BFS heights
-                    // H1: lowest residual neighbour of every unfinished hub; the
-                    // warp that completes a hub's last item takes the hub's
-                    // decision (push at the lowest height, after a relabel when
-                    // the hub is not above it; or finish)
-                    // the cycle's items: all hub items in cycle 0, afterwards the
-                    // items of the hubs still active after the previous cycle
-                    const int2 *items = c == 0 ? G.hcl : ((c - 1) & 1 ? G.hlv1 : G.hlv0);
-                    const int nitems = c == 0 ? nhc : lctl(&C->hlc[(c - 1) & 1]);
-                    for (int w = fresh ? nitems : gwarp; w < nitems; w += nwarps) {
-                        const int2 item = lcg(&items[w]);
-                        const int i = item.x;
-                        if (lcg(&G.hmode[i]) < 0) continue;
-                        const int u = lcg(&HL[i]);
-                        const int beg = __ldg(&G.row[u]);
-                        const int a1 = min(item.y + kPrChunk, __ldg(&G.row[u + 1]));
-                        // no push or relabel runs during H1, so every item of a hub
-                        // sees the same e(u), h(u): the items of a hub that is no
-                        // longer active skip the scan and only arrive
-                        // (a hub of the pull side of a push-pull repair is
-                        // active when deficient and scans its arcs in)
-                        const unsigned char side = stage == 1 ? G.part[u] : kPartT;
-                        const bool pull = PP && side == kPartS;
-                        const long long eu0 = lcg(&G.e[u]);
-                        const bool live = (pull ? eu0 < 0 : eu0 > 0) && lcg(&G.h[u]) < n;
-                        const unsigned char *ptc = stage == 1 ? G.part : nullptr;
-                        unsigned long long best = ~0ull;
-                        if (live)
-                            best = pull ? hub_scan_item<true>(G, item.y, a1, beg, ptc, side, K)
-                                        : hub_scan_item<false>(G, item.y, a1, beg, ptc, side, K);
-                        best = warp_min(best);
-                        bool relabelled = false;
-                        if (lane == 0) {
-                            G.hikey[w] = (unsigned)(best >> 32);   // lowest height in this item
-                            if (best != ~0ull) atomicMin(&G.hkey[i], best);
-                            if (arrive_acq_rel(&G.hdone[i]) == lcg(&G.hnit[i]) - 1) {
-                                const int hu = lcg(&G.h[u]);
-                                const long long eu = pull ? -lcg(&G.e[u]) : lcg(&G.e[u]);   // amount to move
-                                const unsigned long long key = __ldcg(&G.hkey[i]);
-                                G.hkey[i] = ~0ull;
-                                G.hdone[i] = 0;
-                                int mode;
-                                if (hu >= n || eu <= 0) {
-                                    mode = -1;
-                                } else if (key == ~0ull) {
-                                    G.h[u] = n;
-                                    ++K.relabel;
-                                    relabelled = true;
-                                    mode = -1;
-                                } else {
-                                    const int hh = (int)(key >> 32);
-                                    // push to the arcs at height hh, after
-                                    // relabelling u to hh + 1 if it is not
-                                    // above them (the same cycle's H3 pushes:
-                                    // a relabel followed by a rescan in the
-                                    // next cycle cost a cycle per relabel)
-                                    if (hu <= hh) {
-                                        G.h[u] = hh + 1;
-                                        ++K.relabel;
-                                        relabelled = true;
-                                    }
-                                    if (hh + 1 < n) {
-                                        mode = hh + 1;
-                                        G.hrem[i] = eu;
-                                    } else {
-                                        mode = -1;
-                                    }
-                                }
-                                G.hmode[i] = mode;
-                                // (a pushing hub is counted, and listed for the
-                                // next cycle, by its last H3 item if it is still
-                                // active after its pushes)
-                                // a relabelled hub's items join the iteration's
-                                // RemoveInvalidEdges list once
-                                if (relabelled && atomicExch(&G.rstamp[u], rstamp_it) == rstamp_it)
-                                    relabelled = false;
-                            }
-                        }
-                        // the deciding warp lists a newly relabelled hub's items
-                        // for RemoveInvalidEdges
-                        relabelled = __shfl_sync(kFull, relabelled, 0);
-                        if (relabelled) {
-                            const int nit = lcg(&G.hnit[i]);
-                            int rpos = 0;
-                            if (lane == 0) rpos = atomicAdd(&C->rhcnt, nit);
-                            rpos = __shfl_sync(kFull, rpos, 0);
-                            for (int q = lane; q < nit; q += 32) G.hri[rpos + q] = make_int2(u, beg + q * kPrChunk);
-                        }
-                    }
-                    if (!fresh) MF_SYNC_T(S_T_HUB, c, 1, nitems);
-                    // hub_act[(c+1)&1] was last read by the exit test of cycle c-1,
-                    // which every thread has passed once it is past the H1 barrier;
-                    // likewise the item count of the set-up, read before H1 (with
-                    // no H1 barrier, it is zeroed after the H3 barrier instead)
+                const unsigned char *const ptc = stage == 1 ? G.part : nullptr;
+                int nlive = nhp;   // hubs of the cycle's list
+                for (int c = 0;; ++c, ++hub_no) {
+                    const int par = hub_no & 1;
+                    const bool fresh = c == 0 && pass == 0;   // the BFS heights decide the first cycle
+                    // the next list's counters: every thread has read them
+                    // before the last cycle's pushes
                     if (gtid == 0) {
-                        C->hub_act[(c + 1) & 1] = 0;
-                        if (c == 0 && !fresh) C->hccnt = 0;
+                        C->hub_live[par ^ 1] = C->hub_items[par ^ 1] = 0;
+                        // the worklist that the scan below builds replaces the
+                        // BFS's (whose length only matters without active hubs)
+                        if (AL.defer && c == 0) C->wcnt = 0;
                     }
-                    // H3: pushes along the lowest arcs; each warp reserves its share
-                    // of the hub's excess with one atomic
-                    // hlc[(c+1)&1] counted the list of cycle c-1, read before H1
-                    if (gtid == 0) C->hlc[(c + 1) & 1] = 0;
-                    for (int w = gwarp; w < nitems; w += nwarps) {
-                        const int2 item = lcg(&items[w]);
-                        const int i = item.x;
-                        const int mode = lcg(&G.hmode[i]);
-                        if (mode <= 0) continue;
-                        const int hh = mode - 1;
-                        const int u = lcg(&HL[i]);
-                        const int beg = __ldg(&G.row[u]);
-                        const int a1 = min(item.y + kPrChunk, __ldg(&G.row[u + 1]));
-                        const unsigned char side = stage == 1 ? G.part[u] : kPartT;
-                        const bool pull = PP && side == kPartS;
-                        // (hikey: the item's lowest height, found by H1; else no arc at h^ here)
-                        if (fresh || lcg(reinterpret_cast<const int *>(&G.hikey[w])) == hh) {
-                            const unsigned char *ptc = stage == 1 ? G.part : nullptr;
-                            if (pull) {
-                                const long long got = hub_move_item<true>(G, item.y, a1, hh, &G.hrem[i], AL, ptc,
-                                                                          side, stage != 1, K);
-                                if (lane == 0 && got) add_ll(&G.e[u], got);
-                            } else {
-                                const long long sent = hub_move_item<false>(G, item.y, a1, hh, &G.hrem[i], AL,
-                                                                            ptc, side, stage != 1, K);
-                                if (lane == 0 && sent) add_ll(&G.e[u], -sent);
-                            }
-                        }
-                        // the hub's last item to finish sees e(u) after all of
-                        // its pushes: a hub still active takes its items into
-                        // the next cycle's list
-                        int pos = -1;
-                        const int nit = lcg(&G.hnit[i]);
-                        if (lane == 0) {
-                            if (arrive_acq_rel(&G.hdone[i]) == nit - 1) {
-                                G.hdone[i] = 0;
-                                const long long eu = lcg(&G.e[u]);
-                                if (lcg(&G.h[u]) < n && (pull ? eu < 0 : eu > 0)) {
-                                    atomicAdd(&C->hub_act[c & 1], 1);
-                                    pos = atomicAdd(&C->hlc[c & 1], nit);
-                                }
-                            }
-                        }
-                        pos = __shfl_sync(kFull, pos, 0);
-                        if (pos >= 0) {
-                            int2 *next_items = c & 1 ? G.hlv1 : G.hlv0;
-                            for (int q = lane; q < nit; q += 32) next_items[pos + q] = make_int2(i, beg + q * kPrChunk);
-                        }
-                    }
-                    if (AL.count && lane == 0) atomicAdd(&C->wcnt, AL.count);   // (topology-driven mode)
-                    AL.count = 0;
-                    MF_SYNC_T(S_T_HUB, c, 3, lctl(&C->hub_act[c & 1]));
-                    if (gtid == 0 && fresh) C->hccnt = 0;
-                    if (lctl(&C->hub_act[c & 1]) == 0) {
-                        pass_hubs_clean = true;
+                    hub_list<PP>(G, HL, par, nlive, c == 0, fresh, ptc, gwarp, nwarps, J.debug != 0);
+                    MF_SYNC_T(S_T_HUB, c, 0, nlive);
+                    // the next pass's queue counters: every thread has read what
+                    // the pass before this one left there
+                    if (gtid == 0 && c == 0 && pass > 0) C->q[(pass + 1) & 1].clear();
+                    nlive = lctl(&C->hub_live[par]);
+                    const int nitems = lctl(&C->hub_items[par]);
+                    if (nlive == 0) pass_hubs_clean = true;
+                    if (nlive == 0 || c >= hub_cycles) {
+                        ++hub_no;
                         break;
                     }
+                    if (gtid == 0) s_stat[S_HUB_CYCLES] += 1;
+                    if (!fresh) {
+                        hub_lowest(G, nitems, par, gwarp, nwarps, stg, ptc, K);
+                        MF_SYNC_T(S_T_HUB, c, 1, nitems);
+                    }
+                    if (gtid == 0) C->hub_act[par ^ 1] = 0;   // (read before this cycle's list phase)
+                    if (!fresh) hub_relabel(G, HL, par, nlive, rstamp_it, gwarp, nwarps, K);
+                    hub_push(G, nitems, par, fresh, gwarp, nwarps, stg, ptc, AL, K);
+                    if (AL.count && lane == 0) atomicAdd(&C->wcnt, AL.count);   // (topology-driven mode)
+                    AL.count = 0;
+                    MF_SYNC_T(S_T_HUB, c, 3, nitems);
+                    if (!AL.defer && lctl(&C->hub_act[par]) == 0) {
+                        pass_hubs_clean = true;
+                        ++hub_no;
+                        break;
+                    }
+                }
+                if (AL.defer) {
+                    // the active vertices, by one pass over all vertices: the
+                    // worklist anew, and the hubs (left active by the cycles, or
+                    // made active by another one) into the next pass's list
+                    constexpr int kSc = 4;   // vertices in flight per thread
+                    for (long long vb0 = (long long)gwarp * 32; vb0 < n; vb0 += kSc * gthreads) {
+                        int v[kSc], hs[kSc], deg[kSc];
+                        long long es[kSc];
+                        bool small[kSc], hub[kSc], any = false;
+#pragma unroll
+                        for (int j = 0; j < kSc; ++j) {
+                            const long long x = vb0 + j * gthreads + lane;
+                            v[j] = x < n ? (int)x : s;
+                            hs[j] = lcg(&G.h[v[j]]);
+                            es[j] = lcg(&G.e[v[j]]);
+                        }
+#pragma unroll
+                        for (int j = 0; j < kSc; ++j) {
+                            hub[j] = hs[j] < n && v[j] != s && v[j] != t &&
+                                     (stage == 1 && G.part[v[j]] == kPartS ? es[j] < 0 : es[j] > 0);
+                            any |= hub[j];
+                        }
+                        if (!__any_sync(kFull, any)) continue;
+#pragma unroll
+                        for (int j = 0; j < kSc; ++j)
+                            deg[j] = hub[j] ? __ldg(&G.row[v[j] + 1]) - __ldg(&G.row[v[j]]) : 0;
+#pragma unroll
+                        for (int j = 0; j < kSc; ++j) {
+                            small[j] = hub[j] && deg[j] <= kHubDeg;
+                            hub[j] = deg[j] > kHubDeg;
+                        }
+                        warp_append_n(small, v, &C->wcnt, G.wl);
+                        warp_append_n(hub, v, pcnt, AL.hlist);
+                    }
+                    MF_SYNC_T(S_T_HUB, hub_cycles, 2, lctl(&C->wcnt));
+                    pass_hubs_clean = true;   // (those left active are listed)
                 }
             }
             bool pass_rounds_clean = true;
             int cnt = lctl(&C->wcnt);
-            const int qtail0 = qmode ? lctl(&C->aq_tail) : 0;   // queued by the hub cycles
+            const int qtail0 = qmode ? lctl(&AL.Q->tail) : 0;   // queued by the hub cycles
             if (qmode && cnt + qtail0 > 0) {
                 // PushRelabel from the activation queue, without rounds: the
                 // worklist entries (generation 0) are dealt to the warps by
@@ -2626,7 +2731,7 @@ const int max_rounds = L > kMaxRounds ? L : kMaxRounds;
                     } else {
                         unsigned long long slot = 0;
                         if (lane == 0) {
-                            const int q = atomicAdd(&C->aq_head, 1);
+                            const int q = atomicAdd(&AL.Q->head, 1);
                             unsigned long long t0 = 0;
                             unsigned ns = 32;
                             for (int k = 0;; ++k) {
@@ -2643,12 +2748,12 @@ const int max_rounds = L > kMaxRounds ? L : kMaxRounds;
                                     // tail read
                                     int d;
                                     asm volatile("atom.acq_rel.gpu.global.add.s32 %0, [%1], %2;"
-                                                 : "=r"(d) : "l"(&C->aq_done), "r"(ndone) : "memory");
-                                    if (d + ndone == n0 + ld_acquire_s32(&C->aq_tail)) atomicExch(&C->aq_fin, 1);
+                                                 : "=r"(d) : "l"(&AL.Q->done), "r"(ndone) : "memory");
+                                    if (d + ndone == n0 + ld_acquire_s32(&AL.Q->tail)) atomicExch(&AL.Q->fin, 1);
                                     ndone = 0;
                                 }
                                 if (threadIdx.x == 0) {
-                                    if (ld_acquire_s32(&C->aq_fin)) {
+                                    if (ld_acquire_s32(&AL.Q->fin)) {
                                         *(volatile int *)&s_fin = 1;
                                         break;
                                     }
@@ -2677,7 +2782,7 @@ const int max_rounds = L > kMaxRounds ? L : kMaxRounds;
                     if (!vertex_ok(J, C, u, n)) {
                         // skipped; still counted as processed below
                     } else if (gen >= kMinGen && __any_sync(kFull, gtimer() > s_deadline)) {
-                        if (lane == 0) C->aq_over = 1;   // left active
+                        if (lane == 0) AL.Q->over = 1;   // left active
                     } else if (stage == 1) {
                         const unsigned char side = G.part[u];
                         if (side == kPartS)
@@ -2690,13 +2795,11 @@ const int max_rounds = L > kMaxRounds ? L : kMaxRounds;
                     ++ndone;
                 }
                 if (RL.cnt) relabelled_flush(G, RL);
-                MF_SYNC_T(S_T_PRW, 0, 0, cnt + lctl(&C->aq_tail));
+                MF_SYNC_T(S_T_PRW, 0, 0, cnt + lctl(&AL.Q->tail));
                 if (lctl(&C->status) & ST_WAIT) return;   // a wait gave up: the queue's state is undefined
                 if (threadIdx.x == 0) s_fin = 0;
-                pass_rounds_clean = lctl(&C->aq_over) == 0;
-                if (gtid == 0) s_stat[S_ROUNDS] += lctl(&C->aq_maxgen) + 1;
-                // (the counters are zeroed for the next pass after its set-up
-                // barrier, when every thread has read them)
+                pass_rounds_clean = lctl(&AL.Q->over) == 0;
+                if (gtid == 0) s_stat[S_ROUNDS] += lctl(&AL.Q->maxgen) + 1;
             } else if (!qmode && (cnt > 0 || (pass == 0 && jmode == MF_MODE_TOPOLOGY))) {
                 pass_rounds_clean = false;
                 for (int rd = 0;; ++rd) {
@@ -2871,12 +2974,12 @@ const int max_rounds = L > kMaxRounds ? L : kMaxRounds;
             C->qcnt[i] = C->ccnt[i] = 0;
             C->asum[i] = 0;
         }
-        C->wcnt = C->hcnt = C->hccnt = C->rlcnt = 0;
+        C->wcnt = C->hcnt = C->rlcnt = 0;
         C->acnt[0] = C->acnt[1] = C->acnt[2] = 0;
         C->stamp_base = snext;
         if (batch_job) C->bseq = seq;
-        C->hub_act[0] = C->hub_act[1] = 0;
-        C->hlc[0] = C->hlc[1] = 0;
+        C->hub_live[0] = C->hub_live[1] = C->hub_items[0] = C->hub_items[1] = 0;
+            C->hub_act[0] = C->hub_act[1] = 0;
         C->dacc[0] = C->dacc[1] = 0;
         C->batch_err = 0;
         C->abort_loop = 0;
@@ -3068,23 +3171,21 @@ struct NoAllocLayout {
     static constexpr size_t astamp = rl + align256(sizeof(int) * kNoAllocMaxN);
     static constexpr size_t rstamp = astamp + align256(sizeof(unsigned) * kNoAllocMaxN);
     static constexpr size_t cb = rstamp + align256(sizeof(unsigned) * kNoAllocMaxN);
-    static constexpr size_t hcl = cb + align256(sizeof(int2) * (kNoAllocMaxArcs / kChunk + kNoAllocMaxN));
-    static constexpr size_t hlv0 = hcl + align256(sizeof(int2) * (kNoAllocMaxArcs / kPrChunk + kNoAllocMaxHubs));
-    static constexpr size_t hlv1 = hlv0 + align256(sizeof(int2) * (kNoAllocMaxArcs / kPrChunk + kNoAllocMaxHubs));
-    static constexpr size_t hikey = hlv1 + align256(sizeof(int2) * (kNoAllocMaxArcs / kPrChunk + kNoAllocMaxHubs));
-    static constexpr size_t hl = hikey + align256(sizeof(unsigned) * (kNoAllocMaxArcs / kPrChunk + kNoAllocMaxHubs));
-    static constexpr size_t hmode = hl + align256(sizeof(int) * kNoAllocMaxHubs);
-    static constexpr size_t hnit = hmode + align256(sizeof(int) * kNoAllocMaxHubs);
-    static constexpr size_t hdone = hnit + align256(sizeof(int) * kNoAllocMaxHubs);
-    static constexpr size_t hkey = hdone + align256(sizeof(int) * kNoAllocMaxHubs);
-    static constexpr size_t hrem = hkey + align256(sizeof(unsigned long long) * kNoAllocMaxHubs);
+    static constexpr size_t hit0 = cb + align256(sizeof(int2) * (kNoAllocMaxArcs / kChunk + kNoAllocMaxN));
+    static constexpr size_t hit1 = hit0 + align256(sizeof(int4) * (kNoAllocMaxArcs / kPrChunk + kNoAllocMaxHubs));
+    static constexpr size_t hikey = hit1 + align256(sizeof(int4) * (kNoAllocMaxArcs / kPrChunk + kNoAllocMaxHubs));
+    static constexpr size_t hl = hikey + align256(sizeof(int) * (kNoAllocMaxArcs / kPrChunk + kNoAllocMaxHubs));
+    static constexpr size_t hlist0 = hl + align256(sizeof(int) * kNoAllocMaxHubs);
+    static constexpr size_t hlist1 = hlist0 + align256(sizeof(int) * kNoAllocMaxHubs);
+    static constexpr size_t hkey = hlist1 + align256(sizeof(int) * kNoAllocMaxHubs);
+    static constexpr size_t hrem = hkey + align256(2 * sizeof(int) * kNoAllocMaxHubs);
     static constexpr size_t hl2 = hrem + align256(sizeof(long long) * kNoAllocMaxHubs);
     static constexpr size_t hri = hl2 + align256(sizeof(int) * kNoAllocMaxHubs);
     static constexpr size_t aq = hri + align256(sizeof(int2) * (kNoAllocMaxArcs / kPrChunk + kNoAllocMaxHubs));
     static constexpr size_t total = aq + align256(sizeof(unsigned long long) * kNoAllocMaxN);
 };
 
-static_assert(NoAllocLayout::total == 14288384, "the header states the scratch size (14,288,384 bytes)");
+static_assert(NoAllocLayout::total == 14371072, "the header states the scratch size");
 static __device__ __align__(256) unsigned char g_noalloc_scratch[NoAllocLayout::total];
 
 }  // namespace mf
@@ -3185,6 +3286,13 @@ T *dnew(mf_graph *g, size_t count) {
         g->owned_bytes.push_back(count * sizeof(T));
     }
     return p;
+}
+
+// Hub items are read 16 bytes at a time; an allocator callback may return
+// blocks of any alignment.
+HubItem *dnew_hub_items(mf_graph *g, size_t count) {
+    const uintptr_t p = reinterpret_cast<uintptr_t>(dnew<HubItem>(g, count + 1));   // 0: failed, stays 0
+    return reinterpret_cast<HubItem *>((p + 15) & ~uintptr_t(15));
 }
 
 void dforget(mf_graph *g, void *p) {
@@ -3444,15 +3552,13 @@ int mf_create(int32_t n, int64_t m, const int64_t *row_ptr, const int32_t *col, 
     const size_t NH = size_t(std::max<int64_t>(H.hubs, 1));
     D.hl = dnew<int>(g, NH);
     D.hl2 = dnew<int>(g, NH);
-    D.hmode = dnew<int>(g, NH);
-    D.hkey = dnew<unsigned long long>(g, NH);
+    D.hkey = dnew<int>(g, 2 * NH);
     D.hrem = dnew<long long>(g, NH);
-    D.hnit = dnew<int>(g, NH);
-    D.hdone = dnew<int>(g, NH);
-    D.hcl = dnew<int2>(g, size_t(std::max<int64_t>(H.hub_chunk_items, 1)));
-    D.hlv0 = dnew<int2>(g, size_t(std::max<int64_t>(H.hub_chunk_items, 1)));
-    D.hlv1 = dnew<int2>(g, size_t(std::max<int64_t>(H.hub_chunk_items, 1)));
-    D.hikey = dnew<unsigned>(g, size_t(std::max<int64_t>(H.hub_chunk_items, 1)));
+    D.hlist0 = dnew<int>(g, NH);
+    D.hlist1 = dnew<int>(g, NH);
+    D.hit0 = dnew_hub_items(g, size_t(std::max<int64_t>(H.hub_chunk_items, 1)));
+    D.hit1 = dnew_hub_items(g, size_t(std::max<int64_t>(H.hub_chunk_items, 1)));
+    D.hikey = dnew<int>(g, size_t(std::max<int64_t>(H.hub_chunk_items, 1)));
     D.hri = dnew<int2>(g, size_t(std::max<int64_t>(H.hub_chunk_items, 1)));
     D.astamp = dnew<unsigned>(g, N);
     D.rstamp = dnew<unsigned>(g, N);
@@ -3467,8 +3573,8 @@ int mf_create(int32_t n, int64_t m, const int64_t *row_ptr, const int32_t *col, 
     auto al16 = [](const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; };
     D.al16 = al16(D.head) && al16(D.r) && al16(D.rr);
     if (!row || !head || !rev || !aoe || !est || !D.cap || !D.r || !D.rr || !D.h || !D.e || !D.cap_edge || !D.stamp ||
-        !D.qb0 || !D.qb1 || !D.wl || !D.cb || !D.ctl || !g->side_buf || !D.hl || !D.hmode || !D.hkey ||
-        !D.hrem || !D.hnit || !D.hdone || !D.hcl || !D.hlv0 || !D.hlv1 || !D.hikey || !D.hl2 || !D.hri || !D.astamp ||
+        !D.qb0 || !D.qb1 || !D.wl || !D.cb || !D.ctl || !g->side_buf || !D.hl || !D.hkey ||
+        !D.hrem || !D.hlist0 || !D.hlist1 || !D.hit0 || !D.hit1 || !D.hikey || !D.hl2 || !D.hri || !D.astamp ||
         !D.rstamp || !D.rl || !D.aq)
         return fail(MF_ENOMEM, "device allocation failed");
     auto up = [&](void *dst, const void *src, size_t bytes) {
@@ -3959,15 +4065,13 @@ int mf_solve_bicsr_noalloc(int32_t n, int64_t arcs, const int32_t *row, const in
     D.astamp = reinterpret_cast<unsigned *>(b + Lo::astamp);
     D.rstamp = reinterpret_cast<unsigned *>(b + Lo::rstamp);
     D.cb = reinterpret_cast<int2 *>(b + Lo::cb);
-    D.hcl = reinterpret_cast<int2 *>(b + Lo::hcl);
-    D.hlv0 = reinterpret_cast<int2 *>(b + Lo::hlv0);
-    D.hlv1 = reinterpret_cast<int2 *>(b + Lo::hlv1);
-    D.hikey = reinterpret_cast<unsigned *>(b + Lo::hikey);
+    D.hit0 = reinterpret_cast<int4 *>(b + Lo::hit0);
+    D.hit1 = reinterpret_cast<int4 *>(b + Lo::hit1);
+    D.hikey = reinterpret_cast<int *>(b + Lo::hikey);
     D.hl = reinterpret_cast<int *>(b + Lo::hl);
-    D.hmode = reinterpret_cast<int *>(b + Lo::hmode);
-    D.hnit = reinterpret_cast<int *>(b + Lo::hnit);
-    D.hdone = reinterpret_cast<int *>(b + Lo::hdone);
-    D.hkey = reinterpret_cast<unsigned long long *>(b + Lo::hkey);
+    D.hlist0 = reinterpret_cast<int *>(b + Lo::hlist0);
+    D.hlist1 = reinterpret_cast<int *>(b + Lo::hlist1);
+    D.hkey = reinterpret_cast<int *>(b + Lo::hkey);
     D.hrem = reinterpret_cast<long long *>(b + Lo::hrem);
     D.hl2 = reinterpret_cast<int *>(b + Lo::hl2);
     D.hri = reinterpret_cast<int2 *>(b + Lo::hri);
