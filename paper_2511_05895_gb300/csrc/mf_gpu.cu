@@ -1975,7 +1975,9 @@ __global__ void __launch_bounds__(kBlock, 1) k_solve(DevGraph G, Job J) {
     const int lane = threadIdx.x & 31;
     const long long gtid = (long long)blockIdx.x * kBlock + threadIdx.x;
     const long long gthreads = (long long)gridDim.x * kBlock;
-    const int gwarp = (int)(gtid >> 5);
+    // consecutive numbers on different SMs: neighbouring work items (the hubs'
+    // rows of a renumbered graph, the items of one hub) cost alike
+    const int gwarp = (int)((threadIdx.x >> 5) * gridDim.x + blockIdx.x);
     const int nwarps = (int)(gthreads >> 5);
     const int n = G.n, s = G.s, t = G.t;
     Counters K;
@@ -3143,9 +3145,17 @@ __global__ void __launch_bounds__(256) k_policy(DevGraph G, PolicyJob PJ) {
     }
 }
 
-__global__ void k_cut_side(const int *h, int n, unsigned char *side) {
+// at (or null for the identity): the place of each output element in the input
+__global__ void k_cut_side(const int *h, int n, const int *at, unsigned char *side) {
     for (long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (long long)gridDim.x * blockDim.x)
-        side[v] = h[v] >= n ? 1 : 0;
+        side[v] = h[at ? at[v] : v] >= n ? 1 : 0;
+}
+
+template <class T>
+__global__ void k_gather(T *dst, const T *src, const int *at, long long count) {
+    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < count;
+         i += (long long)gridDim.x * blockDim.x)
+        dst[i] = src[at[i]];
 }
 
 // ---------------------------------------------- allocation-free solve --
@@ -3215,6 +3225,13 @@ struct mf_graph {
     float *params = nullptr;   // policy network parameters on the device
     int max_deg = 0;
     cudaStream_t last = nullptr;
+    // a renumbered graph (mf_build.cpp): the resident arrays are in the
+    // library's own vertex ids, everything that crosses the C ABI in the
+    // input's (s, t above too)
+    std::vector<int32_t> ord, inv;   // input id of each vertex, and the inverse (empty: not renumbered)
+    int *d_inv = nullptr;            // inv on the device
+    std::vector<int32_t> ext_row, arc_at;   // the arcs in the input's order, made when first asked for
+    int *d_arc_at = nullptr;                // and on the device, where it fits
 };
 
 namespace {
@@ -3397,6 +3414,30 @@ int ensure_batch_capacity(mf_graph *g, int64_t k, cudaStream_t st) {
     return MF_OK;
 }
 
+int gather_blocks(const mf_graph *g, long long count) {
+    return int(std::max<long long>(1, std::min<long long>(g->sms * 8, (count + 255) / 256)));
+}
+
+// Fill ext_row / arc_at of a renumbered graph (and d_arc_at if device memory
+// allows; a caller that finds it null permutes on the host).
+int need_external_arcs(mf_graph *g) {
+    if (g->ord.empty() || !g->ext_row.empty()) return MF_OK;
+    try {
+        std::vector<int32_t> row(size_t(g->n) + 1), head(size_t(g->A)), ext_row(size_t(g->n) + 1), at(size_t(g->A));
+        MF_CUDA(cudaMemcpy(row.data(), g->dg.row, row.size() * 4, cudaMemcpyDeviceToHost));
+        if (g->A) MF_CUDA(cudaMemcpy(head.data(), g->dg.head, head.size() * 4, cudaMemcpyDeviceToHost));
+        external_arcs(g->n, row.data(), head.data(), g->ord.data(), g->inv.data(), ext_row.data(), at.data());
+        g->ext_row.swap(ext_row);
+        g->arc_at.swap(at);
+    } catch (const std::bad_alloc &) {
+        return set_err(MF_ENOMEM, "host allocation");
+    }
+    g->d_arc_at = dnew<int>(g, size_t(std::max<int64_t>(g->A, 1)));
+    if (g->d_arc_at && g->A)
+        MF_CUDA(cudaMemcpy(g->d_arc_at, g->arc_at.data(), size_t(g->A) * 4, cudaMemcpyHostToDevice));
+    return MF_OK;
+}
+
 // Make h the exact BFS heights of the current state (a no-op on the device
 // when they are exact already), on the graph's last stream.
 int refresh_heights(mf_graph *g) {
@@ -3416,8 +3457,9 @@ int status_to_code(mf_graph *g, const Ctl &c) {
         static const char *kinds[] = {"?", "list entry out of range", "excess differs from the net inflow",
                                       "residual pair or mirror inconsistent"};
         const long long kind = c.chk_where >> 40, where = c.chk_where & 0xffffffffffll;
+        const bool vertex = (kind == 1 || kind == 2) && where >= 0 && where < g->n && !g->ord.empty();
         return set_err(MF_ECHECK, std::string("debug check failed: ") + kinds[kind >= 1 && kind <= 3 ? kind : 0] +
-                                      " (index " + std::to_string(where) + ")");
+                                      " (index " + std::to_string(vertex ? (long long)g->ord[size_t(where)] : where) + ")");
     }
     if (c.status & ST_STICKY) {
         g->solved = false;
@@ -3467,7 +3509,7 @@ int mf_bicsr_host(int32_t n, int64_t m, const int64_t *row_ptr, const int32_t *c
                   int32_t *arc_cap, int32_t *arc_of_edge, int32_t *cap_limit) {
     if (!row_ptr || (m > 0 && (!col || !cap)) || !arcs) return set_err(MF_EINVAL, "null argument");
     HostBiCSR G;
-    int rc = build_bicsr(n, m, row_ptr, col, cap, s, t, &G);
+    int rc = build_bicsr(n, m, row_ptr, col, cap, s, t, false, &G);
     if (rc) return set_err(rc == 2 ? MF_ENOMEM : MF_EINVAL, "graph rejected by the Bi-CSR builder");
     *arcs = G.arcs;
     if (arc_row) for (int32_t u = 0; u <= n; ++u) arc_row[u] = G.row[size_t(u)];
@@ -3497,7 +3539,7 @@ int mf_create(int32_t n, int64_t m, const int64_t *row_ptr, const int32_t *col, 
         if ((rc = host_copy(cap, size_t(m), hcap, &pcap))) return rc;
     }
     HostBiCSR H;
-    rc = build_bicsr(n, m, prow, pcol, pcap, s, t, &H);
+    rc = build_bicsr(n, m, prow, pcol, pcap, s, t, true, &H);
     if (rc) return set_err(rc == 2 ? MF_ENOMEM : MF_EINVAL, "graph rejected by the Bi-CSR builder");
 
     mf_graph *g = new (std::nothrow) mf_graph();
@@ -3540,6 +3582,17 @@ int mf_create(int32_t n, int64_t m, const int64_t *row_ptr, const int32_t *col, 
     const size_t A = size_t(std::max<int64_t>(H.arcs, 1)), N = size_t(n), M = size_t(std::max<int64_t>(m, 1));
     DevGraph &D = g->dg;
     D.n = n; D.s = s; D.t = t; D.m = int(m); D.A = H.arcs; D.cap_limit = H.cap_limit;
+    if (!H.inv.empty()) {
+        D.s = H.inv[size_t(s)];
+        D.t = H.inv[size_t(t)];
+        try {
+            g->ord.assign(H.ord.begin(), H.ord.end());
+            g->inv.assign(H.inv.begin(), H.inv.end());
+        } catch (const std::bad_alloc &) {
+            return fail(MF_ENOMEM, "host allocation");
+        }
+        if (!(g->d_inv = dnew<int>(g, N))) return fail(MF_ENOMEM, "device allocation failed");
+    }
     int *row = dnew<int>(g, N + 1), *head = dnew<int>(g, A), *rev = dnew<int>(g, A), *aoe = dnew<int>(g, M);
     D.row = row; D.head = head; D.rev = rev; D.arc_of_edge = aoe;
     unsigned char *est = dnew<unsigned char>(g, M);
@@ -3580,17 +3633,10 @@ int mf_create(int32_t n, int64_t m, const int64_t *row_ptr, const int32_t *col, 
     auto up = [&](void *dst, const void *src, size_t bytes) {
         return bytes ? cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, st) : cudaSuccess;
     };
-    std::vector<int32_t> cap_edge(pcap, pcap + m);
-    // the policy's "edges out of s or into t" feature, one byte per edge (0
-    // for a self-loop, which has no arc)
-    std::vector<unsigned char> edge_st(size_t(std::max<int64_t>(m, 1)), 0);
-    for (int32_t u = 0; u < n; ++u)
-        for (int64_t i = prow[u]; i < prow[u + 1]; ++i)
-            edge_st[size_t(i)] = pcol[i] != u && (u == s || pcol[i] == t);
     if (up(row, H.row.data(), (N + 1) * 4) || up(head, H.head.data(), size_t(H.arcs) * 4) ||
         up(rev, H.rev.data(), size_t(H.arcs) * 4) || up(aoe, H.arc_of_edge.data(), size_t(m) * 4) ||
-        up(est, edge_st.data(), size_t(m)) ||
-        up(D.cap, H.cap.data(), size_t(H.arcs) * 4) || up(D.cap_edge, cap_edge.data(), size_t(m) * 4) ||
+        up(est, H.edge_st.data(), size_t(m)) || (g->d_inv && up(g->d_inv, H.inv.data(), N * 4)) ||
+        up(D.cap, H.cap.data(), size_t(H.arcs) * 4) || up(D.cap_edge, pcap, size_t(m) * 4) ||
         cudaMemsetAsync(D.stamp, 0, M * 4, st) || cudaMemsetAsync(D.ctl, 0, sizeof(Ctl), st) ||
         cudaMemsetAsync(D.aq, 0, size_t(D.qc) * 8, st) ||
         cudaMemsetAsync(D.e, 0, N * 8, st) || cudaMemsetAsync(D.h, 0, N * 4, st) ||
@@ -3799,7 +3845,7 @@ int mf_min_cut(mf_graph *g, uint8_t *side, int32_t flags) {
     unsigned char *dst = (flags & MF_DEVICE_PTRS) ? side : g->side_buf;
     int blocks = std::max(1, std::min(g->sms * 4, (g->n + 255) / 256));
     cudaGetLastError();   // an earlier, unrelated failure of this thread is not this launch's
-    k_cut_side<<<blocks, 256, 0, g->last>>>(g->dg.h, g->n, dst);
+    k_cut_side<<<blocks, 256, 0, g->last>>>(g->dg.h, g->n, g->d_inv, dst);
     MF_CUDA(cudaGetLastError());
     if (!(flags & MF_DEVICE_PTRS))
         MF_CUDA(cudaMemcpyAsync(side, g->side_buf, size_t(g->n), cudaMemcpyDeviceToHost, g->last));
@@ -3855,6 +3901,36 @@ int mf_export_graph(mf_graph *g, int64_t *arc_row, int32_t *head, int32_t *rev, 
     if (!g) return MF_EINVAL;
     MF_CUDA(cudaSetDevice(g->dev));
     MF_CUDA(cudaStreamSynchronize(g->last));
+    if (!g->ord.empty()) {
+        int rc = need_external_arcs(g);
+        if (rc) return rc;
+        if (arc_row) for (size_t i = 0; i < g->ext_row.size(); ++i) arc_row[i] = g->ext_row[i];
+        try {
+            std::vector<int32_t> tmp(size_t(g->A));
+            if (cap && g->A) {
+                MF_CUDA(cudaMemcpy(tmp.data(), g->dg.cap, tmp.size() * 4, cudaMemcpyDeviceToHost));
+                gather_i32(tmp.data(), g->arc_at.data(), g->A, false, cap);
+            }
+            if (head && g->A) {
+                MF_CUDA(cudaMemcpy(tmp.data(), g->dg.head, tmp.size() * 4, cudaMemcpyDeviceToHost));
+                gather_i32(tmp.data(), g->arc_at.data(), g->A, false, head);
+                gather_i32(g->ord.data(), head, g->A, false, tmp.data());
+                std::copy(tmp.begin(), tmp.end(), head);
+            }
+            if (rev && g->A) {
+                // the reverse arc's place in the input's order
+                std::vector<int32_t> place(size_t(g->A)), iota(size_t(g->A));
+                for (size_t i = 0; i < iota.size(); ++i) iota[i] = int32_t(i);
+                gather_i32(iota.data(), g->arc_at.data(), g->A, true, place.data());
+                MF_CUDA(cudaMemcpy(tmp.data(), g->dg.rev, tmp.size() * 4, cudaMemcpyDeviceToHost));
+                gather_i32(tmp.data(), g->arc_at.data(), g->A, false, iota.data());
+                gather_i32(place.data(), iota.data(), g->A, false, rev);
+            }
+        } catch (const std::bad_alloc &) {
+            return set_err(MF_ENOMEM, "host allocation");
+        }
+        return MF_OK;
+    }
     if (arc_row) {
         std::vector<int32_t> row(size_t(g->n) + 1);
         MF_CUDA(cudaMemcpy(row.data(), g->dg.row, row.size() * 4, cudaMemcpyDeviceToHost));
@@ -3874,6 +3950,55 @@ int mf_export_state(mf_graph *g, int32_t *r, int64_t *excess, int32_t *height, i
         if (rc) return rc;
     }
     cudaMemcpyKind kind = (flags & MF_DEVICE_PTRS) ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
+    if (!g->ord.empty()) {
+        // in the input's order: gathered on the device into the caller's device
+        // buffers, else (host buffers, or no room for arc_at) on the host
+        if (r) {
+            int rc = need_external_arcs(g);
+            if (rc) return rc;
+        }
+        try {
+            std::vector<int32_t> a, b;
+            auto out32 = [&](int32_t *dst, const int *src, const std::vector<int32_t> &at, const int *d_at) -> int {
+                const long long count = (long long)at.size();
+                if (!dst || count == 0) return MF_OK;
+                if ((flags & MF_DEVICE_PTRS) && d_at) {
+                    k_gather<<<gather_blocks(g, count), 256, 0, g->last>>>(dst, src, d_at, count);
+                    MF_CUDA(cudaGetLastError());
+                    return MF_OK;
+                }
+                a.resize(at.size());
+                MF_CUDA(cudaMemcpyAsync(a.data(), src, at.size() * 4, cudaMemcpyDeviceToHost, g->last));
+                MF_CUDA(cudaStreamSynchronize(g->last));
+                if (!(flags & MF_DEVICE_PTRS)) {
+                    gather_i32(a.data(), at.data(), count, false, dst);
+                    return MF_OK;
+                }
+                b.resize(at.size());
+                gather_i32(a.data(), at.data(), count, false, b.data());
+                MF_CUDA(cudaMemcpy(dst, b.data(), at.size() * 4, cudaMemcpyHostToDevice));
+                return MF_OK;
+            };
+            cudaGetLastError();   // an earlier, unrelated failure of this thread is not these launches'
+            int rc = out32(r, g->dg.r, g->arc_at, g->d_arc_at);
+            if (rc == MF_OK) rc = out32(height, g->dg.h, g->inv, g->d_inv);
+            if (rc) return rc;
+            if (excess && (flags & MF_DEVICE_PTRS)) {
+                k_gather<<<gather_blocks(g, g->n), 256, 0, g->last>>>(reinterpret_cast<long long *>(excess), g->dg.e,
+                                                                      g->d_inv, (long long)g->n);
+                MF_CUDA(cudaGetLastError());
+            } else if (excess) {
+                std::vector<int64_t> e(size_t(g->n));
+                MF_CUDA(cudaMemcpyAsync(e.data(), g->dg.e, e.size() * 8, cudaMemcpyDeviceToHost, g->last));
+                MF_CUDA(cudaStreamSynchronize(g->last));
+                for (int32_t v = 0; v < g->n; ++v) excess[v] = e[size_t(g->inv[size_t(v)])];
+            }
+        } catch (const std::bad_alloc &) {
+            return set_err(MF_ENOMEM, "host allocation");
+        }
+        MF_CUDA(cudaStreamSynchronize(g->last));
+        return MF_OK;
+    }
     if (r && g->A) MF_CUDA(cudaMemcpyAsync(r, g->dg.r, size_t(g->A) * 4, kind, g->last));
     if (excess) MF_CUDA(cudaMemcpyAsync(excess, g->dg.e, size_t(g->n) * 8, kind, g->last));
     if (height) MF_CUDA(cudaMemcpyAsync(height, g->dg.h, size_t(g->n) * 4, kind, g->last));
@@ -3886,9 +4011,33 @@ int mf_import_state(mf_graph *g, const int32_t *r, const int64_t *excess, const 
     MF_CUDA(cudaSetDevice(g->dev));
     cudaMemcpyKind kind = (flags & MF_DEVICE_PTRS) ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
     MF_CUDA(cudaStreamSynchronize(g->last));
-    if (g->A) MF_CUDA(cudaMemcpy(g->dg.r, r, size_t(g->A) * 4, kind));
-    MF_CUDA(cudaMemcpy(g->dg.e, excess, size_t(g->n) * 8, kind));
-    MF_CUDA(cudaMemcpy(g->dg.h, height, size_t(g->n) * 4, kind));
+    if (!g->ord.empty()) {
+        // given in the input's order: permuted on the host
+        int rc = need_external_arcs(g);
+        if (rc) return rc;
+        const cudaMemcpyKind in = (flags & MF_DEVICE_PTRS) ? cudaMemcpyDeviceToHost : cudaMemcpyHostToHost;
+        try {
+            std::vector<int32_t> a(size_t(std::max<int64_t>(g->A, g->n))), b(a.size());
+            std::vector<int64_t> x(size_t(g->n)), y(size_t(g->n));
+            if (g->A) {
+                MF_CUDA(cudaMemcpy(a.data(), r, size_t(g->A) * 4, in));
+                gather_i32(a.data(), g->arc_at.data(), g->A, true, b.data());
+                MF_CUDA(cudaMemcpy(g->dg.r, b.data(), size_t(g->A) * 4, cudaMemcpyHostToDevice));
+            }
+            MF_CUDA(cudaMemcpy(a.data(), height, size_t(g->n) * 4, in));
+            gather_i32(a.data(), g->inv.data(), g->n, true, b.data());
+            MF_CUDA(cudaMemcpy(g->dg.h, b.data(), size_t(g->n) * 4, cudaMemcpyHostToDevice));
+            MF_CUDA(cudaMemcpy(x.data(), excess, size_t(g->n) * 8, in));
+            for (int32_t v = 0; v < g->n; ++v) y[size_t(g->inv[size_t(v)])] = x[size_t(v)];
+            MF_CUDA(cudaMemcpy(g->dg.e, y.data(), size_t(g->n) * 8, cudaMemcpyHostToDevice));
+        } catch (const std::bad_alloc &) {
+            return set_err(MF_ENOMEM, "host allocation");
+        }
+    } else {
+        if (g->A) MF_CUDA(cudaMemcpy(g->dg.r, r, size_t(g->A) * 4, kind));
+        MF_CUDA(cudaMemcpy(g->dg.e, excess, size_t(g->n) * 8, kind));
+        MF_CUDA(cudaMemcpy(g->dg.h, height, size_t(g->n) * 4, kind));
+    }
     // rebuild the mirror rr[a] = r[rev[a]] on the host side of the copy
     std::vector<int32_t> hr(size_t(g->A)), hrev(size_t(g->A)), hrr(size_t(g->A));
     if (g->A) {
@@ -3900,9 +4049,10 @@ int mf_import_state(mf_graph *g, const int32_t *r, const int64_t *excess, const 
     // value of the imported state: e(t) plus the deficits (Alg. 4, final sum)
     std::vector<int64_t> he(size_t(g->n));
     MF_CUDA(cudaMemcpy(he.data(), g->dg.e, size_t(g->n) * 8, cudaMemcpyDeviceToHost));
-    long long flow = he[size_t(g->t)];
+    const int32_t ds = g->dg.s, dt = g->dg.t;
+    long long flow = he[size_t(dt)];
     for (int32_t v = 0; v < g->n; ++v)
-        if (v != g->s && v != g->t && he[size_t(v)] < 0) flow += he[size_t(v)];
+        if (v != ds && v != dt && he[size_t(v)] < 0) flow += he[size_t(v)];
     MF_CUDA(cudaMemset(g->dg.ctl, 0, sizeof(Ctl)));
     MF_CUDA(cudaMemset(g->dg.stamp, 0, size_t(std::max<int64_t>(g->m, 1)) * 4));
     MF_CUDA(cudaMemset(g->dg.astamp, 0, size_t(g->n) * 4));
