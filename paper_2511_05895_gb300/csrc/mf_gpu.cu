@@ -360,6 +360,20 @@ __device__ __forceinline__ T lctl(const T *p) {
     return v;
 }
 
+// Two counters in the CTA's shared memory that are zero at the start of every
+// phase (the grid barrier resets them).
+__device__ __forceinline__ int *cta_words() {
+    static __shared__ int w[2];
+    return w;
+}
+
+// The next of the CTA's work items, to one warp: 0, 1, ...  All 32 lanes call.
+__device__ __forceinline__ int cta_ticket(int *word) {
+    int k = 0;
+    if ((threadIdx.x & 31) == 0) k = atomicAdd(word, 1);
+    return __shfl_sync(kFull, k, 0);
+}
+
 // Bounded grid barrier for a cooperative (co-resident) grid.  One word holds
 // the generation (high 16 bits) and the arrivals: the arrival's atomic
 // returns the generation to wait on, and the last CTA to arrive starts the
@@ -394,6 +408,7 @@ __device__ __forceinline__ bool grid_sync(Ctl *C) {
             }
         }
         ok = good;
+        cta_words()[0] = cta_words()[1] = 0;
     }
     __syncthreads();
     return ok;
@@ -2806,27 +2821,42 @@ const int max_rounds = L > kMaxRounds ? L : kMaxRounds;
                 pass_rounds_clean = false;
                 for (int rd = 0;; ++rd) {
                     // topology-driven (Sec. 5.2): every round visits every
-                    // vertex id and serves the active ones, each warp 32 ids
-                    // at a time (no worklist: the counts only tell whether
-                    // another round has work)
+                    // vertex id and serves the active ones (no worklist is kept:
+                    // the counts only tell whether another round has work).  A
+                    // CTA first collects the active ones of its ids, groups of
+                    // 32 dealt over the CTAs, in its part of qb0, and its warps
+                    // then take them one by one: served in place, the active
+                    // ones of a group, often neighbours in id, waited for one
+                    // another (RMAT-18, renumbered: 62 -> 17 us a round).
                     int *const ncnt = &C->acnt[(rd + 1) % 3];
                     if (gtid == 0) {
                         C->acnt[(rd + 2) % 3] = 0;
                         s_stat[S_ROUNDS] += 1;
                     }
-                    for (int grp = gwarp; grp * 32 < n; grp += nwarps) {
-                        const int base = grp * 32;
-                        const int v = base + lane;
-                        bool act = false;
-                        if (v < n && v != s && v != t && __ldg(&G.row[v + 1]) - __ldg(&G.row[v]) <= kHubDeg)
-                            act = lcg(&G.h[v]) < n && lcg(&G.e[v]) > 0;
-                        unsigned mask = __ballot_sync(kFull, act);
-                        while (mask) {
-                            const int j = __ffs(mask) - 1;
-                            mask &= mask - 1u;
-                            visit_chain(G, base + j, kc, AL, stg, RL, K);
+                    const int groups = (n + 31) / 32, per = groups / (int)gridDim.x, more = groups % (int)gridDim.x;
+                    int *const mine = G.qb0 + 32 * ((int)blockIdx.x * per + min((int)blockIdx.x, more));
+                    int *const w = cta_words();
+                    constexpr int kTp = 2;   // groups in flight per warp
+                    for (int g0 = gwarp; g0 < groups; g0 += kTp * nwarps) {
+                        int hs[kTp], deg[kTp];
+                        long long es[kTp];
+#pragma unroll
+                        for (int j = 0; j < kTp; ++j) {
+                            const int v = min((g0 + j * nwarps) * 32 + lane, n - 1);
+                            hs[j] = lcg(&G.h[v]);
+                            es[j] = lcg(&G.e[v]);
+                            deg[j] = __ldg(&G.row[v + 1]) - __ldg(&G.row[v]);
+                        }
+#pragma unroll
+                        for (int j = 0; j < kTp; ++j) {
+                            const int v = (g0 + j * nwarps) * 32 + lane;
+                            warp_append(v < n && v != s && v != t && hs[j] < n && es[j] > 0 && deg[j] <= kHubDeg, v,
+                                        &w[0], mine);
                         }
                     }
+                    __syncthreads();
+                    for (int k = cta_ticket(&w[1]); k < w[0]; k = cta_ticket(&w[1]))
+                        visit_chain(G, bcast_ld(&mine[k]), kc, AL, stg, RL, K);
                     if (RL.cnt) relabelled_flush(G, RL);
                     if (AL.count && lane == 0) atomicAdd(ncnt, AL.count);
                     AL.count = 0;
@@ -3600,7 +3630,7 @@ int mf_create(int32_t n, int64_t m, const int64_t *row_ptr, const int32_t *col, 
     D.cap = dnew<int>(g, A); D.r = dnew<int>(g, A); D.rr = dnew<int>(g, A);
     D.h = dnew<int>(g, N); D.e = dnew<long long>(g, N);
     D.cap_edge = dnew<int>(g, M); D.stamp = dnew<unsigned>(g, M);
-    D.qb0 = dnew<int>(g, N); D.qb1 = dnew<int>(g, N); D.wl = dnew<int>(g, N);
+    D.qb0 = dnew<int>(g, N + 32); D.qb1 = dnew<int>(g, N); D.wl = dnew<int>(g, N);
     D.cb = dnew<int2>(g, size_t(std::max<int64_t>(H.chunk_items, 1)));
     const size_t NH = size_t(std::max<int64_t>(H.hubs, 1));
     D.hl = dnew<int>(g, NH);
