@@ -1934,6 +1934,240 @@ __device__ __forceinline__ void bfs_visit_staged(const DevGraph &G, const int *s
     bfs_discovered_n(G, disc, v, fwd, dual, F, K);
 }
 
+// --------------------------------------- BFS levels of a small frontier --
+// CTA 0 runs the levels of a small frontier alone, in step by __syncthreads
+// only, while the rest of the grid waits at one barrier: until the frontier
+// passes kSoloCap vertices or kSoloArcs arcs, the search would turn bottom-up,
+// or the frontier empties; it then hands the frontier back in the global
+// queue.  What bounds a level is its chain of round trips, so the frontier is
+// kept in shared memory as the list of its arcs (sign bit: searched forward,
+// on the pull side of a push-pull repair), written when a vertex is found: a
+// level takes four trips (heads and residuals; heights; the claiming CAS; rows
+// of what it found), three where few arcs make the height reads not worth
+// their trip.  Which of the found vertices are active is looked up afterwards,
+// for the whole run.  (Measured on grids, per level: frontier of vertices, rows
+// and excesses looked up and global lists reserved in every level 4.6-5.7 us,
+// now @@.)
+constexpr int kSoloWl = 12288;      // found vertices kept at most
+constexpr int kSoloBig = 128;       // frontier vertices of degree > kBigDeg: at most kSoloArcs / (kBigDeg + 1)
+constexpr int kSoloCas = 1024;      // arcs up to which every residual arc tries the CAS at once
+static_assert(kSoloArcs / (kBigDeg + 1) <= kSoloBig, "big vertices of a small frontier");
+static_assert(2 * kSoloArcs + 2 * kSoloCap + kSoloWl + 4 * kSoloBig <= kDynSmem / 4, "shared lists of a small frontier");
+
+struct SoloWords {
+    int nv[2], nbig[2];     // frontier vertices and big vertices, by level parity
+    int na[2];              // arcs of the others
+    unsigned arcs[2];       // all arcs (fewer than 2^31)
+    int nw;                 // vertices found before the current level, and kept
+};
+
+__device__ __forceinline__ void bfs_solo(const DevGraph &G, int L, int cur, long long arcs_seen, bool dual, int *smem,
+                                         long long *s_stat, unsigned long long &tprev, long long it, TraceRec *trace,
+                                         Counters &K) {
+    __shared__ SoloWords W;
+    Ctl *C = G.ctl;
+    const int n = G.n, tid = threadIdx.x, lane = tid & 31;
+    int *const sv[2] = {smem, smem + kSoloCap};
+    int *const sa[2] = {smem + 2 * kSoloCap, smem + 2 * kSoloCap + (int)kSoloArcs};
+    int *const swl = smem + 2 * kSoloCap + 2 * (int)kSoloArcs;
+    int2 *const sbig[2] = {reinterpret_cast<int2 *>(swl + kSoloWl), reinterpret_cast<int2 *>(swl + kSoloWl) + kSoloBig};
+
+    // The lanes' flagged vertices of kIlpB slots, rows [beg, end), join frontier
+    // q (positions from kSoloCap on go to spill); a sets the sign of their
+    // arcs.  One reservation per warp and counter.  All 32 lanes call.
+    auto add = [&](const bool (&ok)[kIlpB], const int (&v)[kIlpB], const int (&beg)[kIlpB], const int (&end)[kIlpB],
+                   const int (&a)[kIlpB], int q, int *spill, bool found) {
+        unsigned mine = 0;   // this lane's vertices (high half) and listed arcs (low half)
+        unsigned all = 0;
+#pragma unroll
+        for (int j = 0; j < kIlpB; ++j)
+            if (ok[j]) {
+                const int deg = end[j] - beg[j];
+                all += (unsigned)deg;
+                mine += 0x10000u + (deg <= kBigDeg ? (unsigned)deg : 0u);
+            }
+        all = __reduce_add_sync(kFull, all);
+        unsigned incl = mine;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned y = __shfl_up_sync(kFull, incl, o);
+            if (lane >= o) incl += y;
+        }
+        int pv = 0, pa = 0;
+        if (lane == 31) {
+            pv = atomicAdd(&W.nv[q], (int)(incl >> 16));
+            pa = atomicAdd(&W.na[q], (int)(incl & 0xffffu));
+            atomicAdd(&W.arcs[q], all);
+        }
+        pv = __shfl_sync(kFull, pv, 31) + (int)((incl - mine) >> 16);
+        pa = __shfl_sync(kFull, pa, 31) + (int)((incl - mine) & 0xffffu);
+#pragma unroll
+        for (int j = 0; j < kIlpB; ++j) {
+            if (!ok[j]) continue;
+            const int deg = end[j] - beg[j], sign = a[j] & (int)0x80000000u;
+            (pv < kSoloCap ? sv[q] : spill)[pv] = v[j];
+            if (found) swl[W.nw + pv] = v[j] | sign;
+            ++pv;
+            if (deg > kBigDeg) {
+                const int k = atomicAdd(&W.nbig[q], 1);
+                if (k < kSoloBig) sbig[q][k] = make_int2(beg[j] | sign, end[j]);
+            } else {
+                // (a frontier of more than kSoloArcs arcs is handed back: its
+                // list need not be whole)
+                if (pa + deg <= (int)kSoloArcs)
+                    for (int i = 0; i < deg; ++i) sa[q][pa + i] = (beg[j] + i) | sign;
+                pa += deg;
+            }
+        }
+    };
+    // kIlpB arcs per lane (ok[j]: arc a[j], sign set: searched forward)
+    auto visit = [&](const int (&a)[kIlpB], const bool (&ok)[kIlpB], bool cas, int Ls, int q, int *spill) {
+        int v[kIlpB], rin[kIlpB], beg[kIlpB], end[kIlpB];
+        bool disc[kIlpB];
+#pragma unroll
+        for (int j = 0; j < kIlpB; ++j) {
+            const int x = a[j] & 0x7fffffff;
+            v[j] = ok[j] ? __ldg(&G.head[x]) : 0;
+            rin[j] = ok[j] ? lcg(a[j] < 0 ? &G.r[x] : &G.rr[x]) : 0;
+            K.bfs_arcs += ok[j];
+        }
+#pragma unroll
+        for (int j = 0; j < kIlpB; ++j) disc[j] = rin[j] > 0 && v[j] != G.s;
+        if (!cas) {
+            int hv[kIlpB];
+#pragma unroll
+            for (int j = 0; j < kIlpB; ++j) hv[j] = disc[j] ? lcg(&G.h[v[j]]) : 0;
+#pragma unroll
+            for (int j = 0; j < kIlpB; ++j) disc[j] = disc[j] && hv[j] == n;
+        }
+        int old[kIlpB];
+#pragma unroll
+        for (int j = 0; j < kIlpB; ++j) old[j] = disc[j] ? atomicCAS(&G.h[v[j]], n, Ls + 1) : 0;
+        bool any = false;
+#pragma unroll
+        for (int j = 0; j < kIlpB; ++j) {
+            disc[j] = disc[j] && old[j] == n;
+            any |= disc[j];
+        }
+        if (!__any_sync(kFull, any)) return;
+#pragma unroll
+        for (int j = 0; j < kIlpB; ++j) {
+            beg[j] = disc[j] ? __ldg(&G.row[v[j]]) : 0;
+            end[j] = disc[j] ? __ldg(&G.row[v[j] + 1]) : 0;
+            K.bfs_verts += disc[j];
+        }
+        add(disc, v, beg, end, a, q, spill, true);
+    };
+    // the active ones of the vertices found so far join the global lists (a
+    // vertex of the pull side is active when deficient); every thread calls,
+    // between barriers
+    auto flush = [&]() {
+        const int k = W.nw;
+        for (int i0 = 0; i0 < k; i0 += kBlock) {
+            const int i = i0 + tid;
+            const int x = i < k ? swl[i] : 0, v = x & 0x7fffffff;
+            const long long ev = i < k ? lcg(&G.e[v]) : 0;
+            const int deg = i < k ? __ldg(&G.row[v + 1]) - __ldg(&G.row[v]) : 0;
+            const bool act = i < k && (x < 0 ? ev < 0 : ev > 0);
+            warp_append(act && deg <= kHubDeg, v, &C->wcnt, G.wl);
+            warp_append(act && deg > kHubDeg, v, &C->hcnt, G.hl);
+        }
+        __syncthreads();
+        if (tid == 0) W.nw = 0;
+    };
+
+    if (tid == 0) W = SoloWords{};
+    __syncthreads();
+    const int *F0 = (L & 1) ? G.qb1 : G.qb0;
+    for (int i0 = 0; i0 < cur; i0 += kBlock) {
+        const int i = i0 + tid;
+        bool ok[kIlpB];
+        int v[kIlpB], beg[kIlpB], end[kIlpB], a[kIlpB];
+#pragma unroll
+        for (int j = 0; j < kIlpB; ++j) {
+            v[j] = j == 0 && i < cur ? lcg(&F0[i]) : 0;
+            ok[j] = j == 0 && i < cur && v[j] >= 0 && v[j] < n;
+            beg[j] = ok[j] ? __ldg(&G.row[v[j]]) : 0;
+            end[j] = ok[j] ? __ldg(&G.row[v[j] + 1]) : 0;
+            a[j] = ok[j] && dual && G.part[v[j]] == kPartS ? (int)0x80000000u : 0;
+        }
+        add(ok, v, beg, end, a, 0, nullptr, false);   // (at most kSoloCap vertices)
+    }
+    __syncthreads();
+    int Ls = L, b = 0, cs = cur;
+    long long seen = arcs_seen, mfs = 0;
+    for (;;) {
+        int *spill = (Ls & 1) ? G.qb0 : G.qb1;   // positions >= kSoloCap of the next frontier
+        const int na = W.na[b], nbig = W.nbig[b];
+        const bool cas = na <= kSoloCas;
+        for (int k0 = 0; k0 < na; k0 += kIlpB * kBlock) {
+            int a[kIlpB];
+            bool ok[kIlpB];
+#pragma unroll
+            for (int j = 0; j < kIlpB; ++j) {
+                const int k = k0 + j * kBlock + tid;
+                ok[j] = k < na;
+                a[j] = ok[j] ? sa[b][k] : 0;
+            }
+            visit(a, ok, cas, Ls, b ^ 1, spill);
+        }
+        for (int q = tid >> 5; q < nbig; q += kBlock / 32) {
+            const int2 r = sbig[b][q];
+            const int a0 = r.x & 0x7fffffff;
+            for (int ab = a0; ab < r.y; ab += 32 * kIlpB) {
+                int a[kIlpB];
+                bool ok[kIlpB];
+#pragma unroll
+                for (int j = 0; j < kIlpB; ++j) {
+                    const int x = ab + 32 * j + lane;
+                    ok[j] = x < r.y;
+                    a[j] = x | (r.x & (int)0x80000000u);
+                }
+                visit(a, ok, false, Ls, b ^ 1, spill);
+            }
+        }
+        __syncthreads();
+        if (tid == 0 && trace) {
+            const unsigned long long now = gtimer();
+            s_stat[S_T_BFS] += (long long)(now - tprev);
+            const int k = C->trace_n++;
+            if (k < G.trace_cap) trace[k] = TraceRec{(short)S_T_BFS, 4, (int)it, Ls, cs, (long long)(now - tprev)};
+            tprev = now;
+        }
+        ++Ls;
+        b ^= 1;
+        cs = W.nv[b];
+        mfs = (long long)W.arcs[b];
+        const bool out = cs == 0 || cs > kSoloCap || mfs > kSoloArcs || (mfs * 14 > G.A - (seen + mfs) && cs * 64LL > n);
+        const int nw = W.nw + cs;   // vertices found so far
+        __syncthreads();   // everyone has read the counts
+        if (tid == 0) W.nw = nw;
+        if (out || nw > kSoloWl - (int)kSoloArcs) {
+            __syncthreads();
+            flush();
+        }
+        if (tid == 0) {
+            W.nv[b ^ 1] = W.nbig[b ^ 1] = W.na[b ^ 1] = 0;
+            W.arcs[b ^ 1] = 0;
+        }
+        if (out) break;
+        seen += mfs;
+        __syncthreads();
+    }
+    // hand the frontier of level Ls back in the global queue
+    int *Fg = (Ls & 1) ? G.qb1 : G.qb0;
+    for (int i = tid; i < min(cs, kSoloCap); i += kBlock) Fg[i] = sv[b][i];
+    if (tid == 0) {
+        C->qcnt[Ls % 3] = cs;
+        C->asum[Ls % 3] = mfs;
+        C->qcnt[(Ls + 1) % 3] = 0;
+        C->asum[(Ls + 1) % 3] = 0;
+        C->ccnt[Ls % 3] = 0;
+        C->solo_L = Ls;
+        C->solo_seen = seen;   // arcs of the levels run, without level Ls
+    }
+}
+
 // A vertex id read from a list or queue, checked when debug_checks is on.
 __device__ __forceinline__ bool vertex_ok(const Job &J, Ctl *C, int u, int n) {
     if (!J.debug || (u >= 0 && u < n)) return true;
@@ -1965,23 +2199,6 @@ __device__ __forceinline__ bool vertex_ok(const Job &J, Ctl *C, int u, int n) {
         }                                                                     \
     } while (0)
 #define MF_SYNC(bucket) MF_SYNC_T(bucket, -1, 0, -1)
-// The same record without a grid barrier (levels CTA 0 runs alone).
-#define MF_TRACE_T(bucket, step, mode, aux)                                   \
-    do {                                                                      \
-        if (gtid == 0) {                                                      \
-            const unsigned long long now_ = gtimer();                         \
-            const long long dt_ = (long long)(now_ - tprev);                  \
-            s_stat[bucket] += dt_;                                            \
-            if (TR) {                                                         \
-                const int k_ = C->trace_n++;                                  \
-                if (k_ < G.trace_cap)                                         \
-                    TR[k_] = TraceRec{(short)(bucket), (short)(mode),         \
-                                      (int)it, (int)(step), (int)(aux), dt_}; \
-            }                                                                 \
-            tprev = now_;                                                     \
-        }                                                                     \
-    } while (0)
-
 // PP: the instance that can run Dynamic Push-Pull (Alg. 8); the plain
 // instance compiles without its code paths.
 template <bool PP>
@@ -2359,105 +2576,11 @@ __global__ void __launch_bounds__(kBlock, 1) k_solve(DevGraph G, Job J) {
             if (!bottom_up) bottom_up = mf * 14 > G.A - arcs_seen && cur * (dual ? 32LL : 64LL) > n;
             else bottom_up = cur * 24LL >= n;
             if (!bottom_up && mf <= kSoloArcs && cur <= kSoloCap) {
-                // A small frontier: CTA 0 runs the levels alone, with the
-                // frontiers in shared memory and in step by __syncthreads only,
-                // until the frontier passes kSoloCap vertices or kSoloArcs arcs,
-                // the search would turn bottom-up, or the frontier empties; it
-                // then hands the frontier back in the global queue.  The rest
-                // of the grid waits at one barrier.  Every thread has read this
-                // level's counters before CTA 0 starts (the first barrier).
+                // a small frontier: CTA 0 runs the levels alone (bfs_solo).
+                // Every thread has read this level's counters before it starts
+                // (the first barrier).
                 MF_SYNC_T(S_T_BFS, L, 6, cur);
-                if (blockIdx.x == 0) {
-                    int (*s_front)[kSoloCap] = reinterpret_cast<int (*)[kSoloCap]>(s_bfs);
-                    __shared__ int s_cnt[2];
-                    __shared__ long long s_arcs[2];
-                    __shared__ int s_big;
-                    const int cw = threadIdx.x >> 5;
-                    const int *F0 = (L & 1) ? G.qb1 : G.qb0;
-                    for (int i = threadIdx.x; i < cur; i += kBlock) s_front[0][i] = lcg(&F0[i]);
-                    if (threadIdx.x == 0) {
-                        s_cnt[1] = 0;
-                        s_arcs[1] = 0;
-                        s_big = 0;
-                    }
-                    __syncthreads();
-                    int Ls = L, cs = cur, b = 0;
-                    long long seen = arcs_seen, mfs = 0;
-                    for (;;) {
-                        int *ccs = &C->ccnt[Ls % 3];
-                        int *spill = (Ls & 1) ? G.qb0 : G.qb1;   // positions >= kSoloCap of the next frontier
-                        Front SF{&s_cnt[b ^ 1], s_front[b ^ 1], &s_arcs[b ^ 1], kSoloCap, spill, nullptr, 0, 0};
-                        int gs = 32;   // frontier vertices per warp: fewer when they do not fill the warps
-                        while (gs > 1 && (gs >> 1) * (kBlock / 32) >= cs) gs >>= 1;
-                        for (int grp = cw; grp * gs < cs; grp += kBlock / 32) {
-                            const int idx = grp * gs + lane;
-                            int beg = 0, deg = 0;
-                            bool fwd = false;
-                            if (lane < gs && idx < cs) {
-                                const int u = s_front[b][idx];
-                                fwd = dual && G.part[u] == kPartS;
-                                beg = __ldg(&G.row[u]);
-                                deg = __ldg(&G.row[u + 1]) - beg;
-                                if (deg > kBigDeg) {
-                                    const int nc = (deg + kChunk - 1) / kChunk;
-                                    const int pos = atomicAdd(ccs, nc);
-                                    for (int c = 0; c < nc; ++c) G.cb[pos + c] = make_int2(u, beg + c * kChunk);
-                                    s_big = 1;
-                                    deg = 0;
-                                }
-                            }
-                            bfs_expand_warp(G, beg, deg, fwd, dual, Ls, SF, K);
-                        }
-                        __syncthreads();
-                        if (s_big) {
-                            const int nch = lcg(ccs);
-                            for (int c = cw; c < nch; c += kBlock / 32) {
-                                const int2 item = lcg(&G.cb[c]);
-                                const unsigned fw = (dual && G.part[item.x] == kPartS) ? (1u << kIlpB) - 1u : 0u;
-                                const int a1 = min(item.y + kChunk, __ldg(&G.row[item.x + 1]));
-                                for (int ab = item.y; ab < a1; ab += 32 * kIlpB) {
-                                    int a[kIlpB];
-                                    bool ok[kIlpB];
-#pragma unroll
-                                    for (int j = 0; j < kIlpB; ++j) {
-                                        a[j] = ab + 32 * j + lane;
-                                        ok[j] = a[j] < a1;
-                                    }
-                                    bfs_visit_n(G, a, ok, fw, dual, Ls, SF, K);
-                                }
-                            }
-                            __syncthreads();
-                        }
-                        MF_TRACE_T(S_T_BFS, Ls, 4, cs);
-                        ++Ls;
-                        cs = s_cnt[b ^ 1];
-                        mfs = s_arcs[b ^ 1];
-                        __syncthreads();   // everyone has read the counts
-                        b ^= 1;
-                        if (threadIdx.x == 0) {
-                            s_cnt[b ^ 1] = 0;
-                            s_arcs[b ^ 1] = 0;
-                            s_big = 0;
-                            C->ccnt[Ls % 3] = 0;
-                        }
-                        if (cs == 0 || cs > kSoloCap || mfs > kSoloArcs ||
-                            (mfs * 14 > G.A - (seen + mfs) && cs * 64LL > n))
-                            break;
-                        seen += mfs;
-                        __syncthreads();
-                    }
-                    // hand the frontier of level Ls back in the global queue
-                    int *Fg = (Ls & 1) ? G.qb1 : G.qb0;
-                    for (int i = threadIdx.x; i < min(cs, kSoloCap); i += kBlock) Fg[i] = s_front[b][i];
-                    if (threadIdx.x == 0) {
-                        C->qcnt[Ls % 3] = cs;
-                        C->asum[Ls % 3] = mfs;
-                        C->qcnt[(Ls + 1) % 3] = 0;
-                        C->asum[(Ls + 1) % 3] = 0;
-                        C->solo_L = Ls;
-                        C->solo_seen = seen;   // arcs of the levels run, without level Ls
-                    }
-                }
+                if (blockIdx.x == 0) bfs_solo(G, L, cur, arcs_seen, dual, s_dyn, s_stat, tprev, it, TR, K);
                 MF_SYNC_T(S_T_BFS, L, 5, cur);
                 L = lctl(&C->solo_L);
                 arcs_seen = lctl(&C->solo_seen);
