@@ -32,9 +32,9 @@
 // persistent kernel never relies on L1 contents across a grid barrier.
 //
 // The phases avoid atomics that the whole grid aims at one address: the
-// items of a phase are dealt to the warps by a fixed stride (no work
-// tickets), and each warp stages the BFS frontier it discovers in shared
-// memory and publishes it a stage at a time.
+// items of a phase are dealt to the CTAs by a fixed stride and taken by their
+// warps from a counter in shared memory, and each warp stages the BFS frontier
+// it discovers in shared memory and publishes it a stage at a time.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -372,6 +372,18 @@ __device__ __forceinline__ int cta_ticket(int *word) {
     int k = 0;
     if ((threadIdx.x & 31) == 0) k = atomicAdd(word, 1);
     return __shfl_sync(kFull, k, 0);
+}
+
+// The next of a phase's `count` work items, to one warp: each warp starts with
+// item gwarp (item w belongs to CTA w mod gridDim.x) and takes further ones of
+// its CTA's share as it gets free.  A fixed stride over the warps left them
+// waiting at the barrier 33-58 % of the time in the search and hub phases; the
+// slowest of 24 warps sets the CTA's time.  (RMAT-20 100k and static solve -4 %,
+// 2048^2 grid -4 %; a counter of the whole grid would be one hot word.)
+// Returns >= count when there is none.  All 32 lanes call.
+__device__ __forceinline__ int next_item(int *word, int count) {
+    const int first = (int)gridDim.x * (int)(blockDim.x >> 5);
+    return count <= first ? count : first + cta_ticket(word) * (int)gridDim.x + (int)blockIdx.x;
 }
 
 // Bounded grid barrier for a cooperative (co-resident) grid.  One word holds
@@ -1639,14 +1651,17 @@ __device__ __forceinline__ void hub_lowest(const DevGraph &G, int nitems, int pa
                                            const unsigned char *pt, Counters &K) {
     const int lane = threadIdx.x & 31;
     const HubItem *items = par ? G.hit1 : G.hit0;
-    HubItem cur = hub_item(items, gwarp, nitems), nxt = hub_item(items, gwarp + nwarps, nitems);
-    if (gwarp < nitems) hub_issue(G, cur, stg);
+    int *const tick = cta_words();
+    int w = gwarp, w1 = next_item(tick, nitems);
+    HubItem cur = hub_item(items, w, nitems), nxt = hub_item(items, w1, nitems);
+    if (w < nitems) hub_issue(G, cur, stg);
     asm volatile("cp.async.commit_group;" ::: "memory");
     int b = 0;
-    for (int w = gwarp; w < nitems; w += nwarps) {
-        if (w + nwarps < nitems) hub_issue(G, nxt, stg + (b ^ 1) * 2 * kHubBuf);
+    while (w < nitems) {
+        if (w1 < nitems) hub_issue(G, nxt, stg + (b ^ 1) * 2 * kHubBuf);
         asm volatile("cp.async.commit_group;" ::: "memory");
-        const HubItem nn = hub_item(items, w + 2 * nwarps, nitems);
+        const int w2 = next_item(tick, nitems);
+        const HubItem nn = hub_item(items, w2, nitems);
         asm volatile("cp.async.wait_group 1;" ::: "memory");
         __syncwarp();
         int hv[kHubArcs];
@@ -1660,6 +1675,8 @@ __device__ __forceinline__ void hub_lowest(const DevGraph &G, int nitems, int pa
         __syncwarp();   // every lane is done with the item's buffer
         cur = nxt;
         nxt = nn;
+        w = w1;
+        w1 = w2;
         b ^= 1;
     }
     asm volatile("cp.async.wait_all;" ::: "memory");
@@ -1726,16 +1743,19 @@ __device__ __forceinline__ void hub_push(const DevGraph &G, int nitems, int par,
         const long long rem = lcg(&G.hrem[m.x]);
         return __shfl_sync(kFull, hh < G.n - 1 && key == hh && rem > 0 ? hh : -1, 0);
     };
-    HubItem cur = hub_item(items, gwarp, nitems), nxt = hub_item(items, gwarp + nwarps, nitems);
-    int hh = push_height(cur, gwarp);
+    int *const tick = cta_words();
+    int w = gwarp, w1 = next_item(tick, nitems);
+    HubItem cur = hub_item(items, w, nitems), nxt = hub_item(items, w1, nitems);
+    int hh = push_height(cur, w);
     if (hh >= 0) hub_issue(G, cur, stg);
     asm volatile("cp.async.commit_group;" ::: "memory");
-    int hn = push_height(nxt, gwarp + nwarps);
+    int hn = push_height(nxt, w1);
     int b = 0;
-    for (int w = gwarp; w < nitems; w += nwarps) {
+    while (w < nitems) {
         if (hn >= 0) hub_issue(G, nxt, stg + (b ^ 1) * 2 * kHubBuf);
         asm volatile("cp.async.commit_group;" ::: "memory");
-        const HubItem nn = hub_item(items, w + 2 * nwarps, nitems);
+        const int w2 = next_item(tick, nitems);
+        const HubItem nn = hub_item(items, w2, nitems);
         if (hh >= 0) {
             asm volatile("cp.async.wait_group 1;" ::: "memory");
             __syncwarp();
@@ -1826,7 +1846,9 @@ __device__ __forceinline__ void hub_push(const DevGraph &G, int nitems, int par,
         cur = nxt;
         nxt = nn;
         hh = hn;
-        hn = push_height(nxt, w + 2 * nwarps);
+        hn = push_height(nxt, w2);
+        w = w1;
+        w1 = w2;
         b ^= 1;
     }
     asm volatile("cp.async.wait_all;" ::: "memory");
@@ -2599,21 +2621,26 @@ __global__ void __launch_bounds__(kBlock, 1) k_solve(DevGraph G, Job J) {
             }
             Front FR{ncnt, NF, asum, 0x7fffffff, nullptr, s_bfs + (threadIdx.x >> 5) * kWq, 0, 0};
             if (bottom_up) {
-                // groups of 32 consecutive vertex ids (warp w: groups w, w + W, ...)
+                // groups of 32 consecutive vertex ids
                 const int groups = (n + 31) / 32;
-                BuPre pre = bu_prefetch(G, gwarp * 32);
-                for (int grp = gwarp; grp < groups; grp += nwarps) {
+                int *const tick = cta_words();
+                int grp = gwarp, nxt;
+                BuPre pre = bu_prefetch(G, min(grp, groups) * 32);
+                for (; grp < groups; grp = nxt) {
                     const BuPre cur = pre;
-                    if (grp + nwarps < groups) pre = bu_prefetch(G, (grp + nwarps) * 32);
+                    nxt = next_item(tick, groups);
+                    pre = bu_prefetch(G, min(nxt, groups) * 32);
                     bfs_bottom_up_group(G, grp * 32, cur, dual, L, FR, ccnt, K);
                 }
             } else {
-                // groups of gs frontier vertices (warp w: groups w, w + W, ...):
+                // groups of gs frontier vertices:
                 // 32, or fewer when the frontier does not fill the grid's warps,
                 // so that the arcs of a small frontier still spread over them
                 int gs = 32;
                 while (gs > 1 && (long long)(gs >> 1) * nwarps >= cur) gs >>= 1;
-                for (int grp = gwarp; grp * gs < cur; grp += nwarps) {
+                int *const tick = cta_words();
+                const int groups = (cur + gs - 1) / gs;
+                for (int grp = gwarp; grp < groups; grp = next_item(tick, groups)) {
                     const int idx = grp * gs + lane;
                     int beg = 0, deg = 0;
                     bool fwd = false;
@@ -2636,21 +2663,24 @@ __global__ void __launch_bounds__(kBlock, 1) k_solve(DevGraph G, Job J) {
             MF_SYNC_T(S_T_BFS, L, bottom_up ? 2 : 0, cur);
             const int nch = lctl(ccnt);
             if (nch > 0) {
+                int *const tick = cta_words();
                 if (bottom_up) {
-                    for (int c = gwarp; c < nch; c += nwarps) bfs_bottom_up_item(G, lcg(&G.cb[c]), dual, L, FR, K);
+                    for (int c = gwarp; c < nch; c = next_item(tick, nch))
+                        bfs_bottom_up_item(G, lcg(&G.cb[c]), dual, L, FR, K);
                 } else {
                     // items staged one ahead (see item_issue)
                     int *const ibuf = s_dyn + kItemOff + (threadIdx.x >> 5) * kItemWarp;
-                    int c = gwarp, b = 0;
+                    int c = gwarp, c1 = next_item(tick, nch), b = 0;
                     ItemMeta cur = c < nch ? item_meta(G, c, dual) : ItemMeta{0, 0, 0, false};
                     if (c < nch) item_issue(G, cur, ibuf);
                     asm volatile("cp.async.commit_group;" ::: "memory");
-                    ItemMeta nxt = c + nwarps < nch ? item_meta(G, c + nwarps, dual) : ItemMeta{0, 0, 0, false};
-                    for (; c < nch; c += nwarps) {
-                        if (c + nwarps < nch) item_issue(G, nxt, ibuf + (b ^ 1) * 2 * kItemBuf);
+                    ItemMeta nxt = c1 < nch ? item_meta(G, c1, dual) : ItemMeta{0, 0, 0, false};
+                    while (c < nch) {
+                        if (c1 < nch) item_issue(G, nxt, ibuf + (b ^ 1) * 2 * kItemBuf);
                         asm volatile("cp.async.commit_group;" ::: "memory");
-                        const ItemMeta nn =
-                            c + 2 * nwarps < nch ? item_meta(G, c + 2 * nwarps, dual) : ItemMeta{0, 0, 0, false};
+                        c = c1;
+                        c1 = next_item(tick, nch);
+                        const ItemMeta nn = c1 < nch ? item_meta(G, c1, dual) : ItemMeta{0, 0, 0, false};
                         asm volatile("cp.async.wait_group 1;" ::: "memory");   // the current item's copies
                         __syncwarp();
                         const int *sv = ibuf + b * 2 * kItemBuf;
@@ -2842,8 +2872,8 @@ const int max_rounds = L > kMaxRounds ? L : kMaxRounds;
             const int qtail0 = qmode ? lctl(&AL.Q->tail) : 0;   // queued by the hub cycles
             if (qmode && cnt + qtail0 > 0) {
                 // PushRelabel from the activation queue, without rounds: the
-                // worklist entries (generation 0) are dealt to the warps by
-                // stride, then each warp takes a ticket for the next queued
+                // worklist entries (generation 0) are dealt to the warps first,
+                // then each warp takes a ticket for the next queued
                 // entry and waits for it; of the vertices that a visit turns
                 // active the warp serves one itself (visit_chain_t) and queues
                 // the others at once with the next generation, for the next
@@ -2864,7 +2894,8 @@ const int max_rounds = L > kMaxRounds ? L : kMaxRounds;
                 if (threadIdx.x == 0) s_deadline = gtimer() + (s_bfs_end - s_bfs_begin) * kQueueShareNum / kQueueShareDen;
                 __syncthreads();
                 int ndone = 0;   // entries finished and not yet counted (warp-uniform)
-                for (int i = gwarp;; i += nwarps) {
+                int *const tick = cta_words();
+                for (int i = gwarp;; i = i < n0 ? next_item(tick, n0) : i) {
                     int u = -1, gen = 0;
                     if (i < n0) {
                         u = bcast_ld(&G.wl[i]);
@@ -3004,18 +3035,11 @@ const int max_rounds = L > kMaxRounds ? L : kMaxRounds;
         // the h- form, Algorithm 7)
         const unsigned char *ptc = stage ? G.part : nullptr;
         const int nrl = lctl(&C->rlcnt);
-        for (int i = gwarp; i < nrl; i += nwarps) {
-            const int u = bcast_ld(&G.rl[i]);
-            if (!vertex_ok(J, C, u, n)) continue;   // warp-uniform
-            const unsigned char side = ptc ? ptc[u] : kPartT;
-            if (side == kPartS)
-                remove_invalid_warp_t<true>(G, u, &C->ri_moved[par], ptc, side, K);
-            else
-                remove_invalid_warp_t<false>(G, u, &C->ri_moved[par], ptc, side, K);
-        }
         const int nri = lctl(&C->rhcnt);
-        for (int w = gwarp; w < nri; w += nwarps) {
-            const int2 item = lcg(&G.hri[w]);
+        int *const tick = cta_words();
+        int ri = gwarp;   // hub items first (they cost the most), then vertices
+        for (; ri < nri; ri = next_item(tick, nri + nrl)) {
+            const int2 item = lcg(&G.hri[ri]);
             const int u = __shfl_sync(kFull, item.x, 0);
             if (!vertex_ok(J, C, u, n)) continue;   // warp-uniform
             const int hu = bcast_ld(&G.h[u]);
@@ -3034,6 +3058,15 @@ const int max_rounds = L > kMaxRounds ? L : kMaxRounds;
                     C->ri_moved[par] = 1;
                 }
             }
+        }
+        for (; ri < nri + nrl; ri = next_item(tick, nri + nrl)) {
+            const int u = bcast_ld(&G.rl[ri - nri]);
+            if (!vertex_ok(J, C, u, n)) continue;   // warp-uniform
+            const unsigned char side = ptc ? ptc[u] : kPartT;
+            if (side == kPartS)
+                remove_invalid_warp_t<true>(G, u, &C->ri_moved[par], ptc, side, K);
+            else
+                remove_invalid_warp_t<false>(G, u, &C->ri_moved[par], ptc, side, K);
         }
         MF_SYNC_T(S_T_RI, 0, 0, nrl + nri);
         if ((it & 255) == 255) flush_counters(K, ST);
