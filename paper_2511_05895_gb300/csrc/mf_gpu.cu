@@ -97,8 +97,9 @@ constexpr int kMinHubCyclesPP = 8;
 // another dual BFS (measured on RMAT-20: 1.66 -> 1.32 ms per repair).
 constexpr int kMaxPasses = 2;
 constexpr int kMaxPassesPP = 4;
-// BFS levels whose frontier has at most this many arcs and vertices run on
-// CTA 0 alone, with the frontiers in shared memory
+// BFS levels whose frontier has at most this many arcs and vertices (fewer in
+// some graphs: search_rules) run on CTA 0 alone, with the frontiers in shared
+// memory
 constexpr long long kSoloArcs = 8192;
 constexpr int kSoloCap = 4096;
 // Above this many hubs the cycles file no activations and one pass over all
@@ -222,6 +223,8 @@ struct DevGraph {
     int al16;                 // head, r and rr start on 16-byte boundaries (16-byte staging copies)
     unsigned long long *aq;   // activation queue slots (generation << 32 | vertex + 1; 0 = empty)
     int qc;                   // its capacity
+    int solo_arcs;            // most arcs of a frontier that CTA 0 searches alone (<= kSoloArcs)
+    int alpha;                // the search goes bottom-up when alpha x its frontier's arcs pass the unvisited arcs
 };
 
 // Push-pull partitions (Alg. 8): T can reach a sink, S cannot (the previous
@@ -693,30 +696,33 @@ __device__ __forceinline__ void bfs_expand_warp(const DevGraph &G, int beg, int 
 }
 
 // Bottom-up step of the backward BFS (direction-optimising search): the
-// unvisited vertices v of a group of 32 consecutive ids look for a residual
+// unvisited vertices v of kBuV groups of 32 consecutive ids look for a residual
 // arc v -> w into the current frontier (h(w) == L); the first one found gives
-// h(v) = L + 1.  The group's arcs are balanced over the lanes and the scan of
-// a vertex stops once it is found.  Vertices of degree > kBigDeg become
-// kChunk-arc items of the chunk list instead.  In the first stage of a
-// push-pull repair (dual) a vertex of the pull side looks for a residual arc
-// w -> v from the frontier instead, and only frontier vertices of the
-// vertex's own side count.  All 32 lanes call.
-// What a lane needs of its vertex base + lane before the group's scan: its
-// height and arc range, loaded one group ahead (the warp loads the next
-// group's while it scans this one).  During a bottom-up level only the
-// owning lane writes an unvisited vertex's height, so the early read is
-// exact.
+// h(v) = L + 1.  A lane scans its own vertices, kBuArcs arcs of each at a time,
+// until it has found one: in the levels that matter most vertices find a
+// parent among their first arcs.  (The group's arcs balanced over the lanes
+// read whole rows, 128 arcs a round, before any vertex could stop, and paid
+// seven shuffles a slot for the owner of each arc.  Per level: RMAT-20 27 -> 15
+// us, 2048^2 grid 84 -> 40 us, 1023 x 769 grid 28 -> 13 us.)  Vertices of
+// degree > kBigDeg become kChunk-arc items of the chunk list instead.  In the first
+// stage of a push-pull repair (dual) a vertex of the pull side looks for a
+// residual arc w -> v from the frontier instead, and only frontier vertices of
+// the vertex's own side count.  All 32 lanes call.
+constexpr int kBuV = 2, kBuArcs = 2;   // (1 x 4, 2 x 4, 1 x 8: 0-25 % slower on RMAT and grids)
+
+// The heights of a lane's vertices, loaded one piece ahead.  During a
+// bottom-up level only the owning lane writes an unvisited vertex's height, so
+// the early read is exact.
 struct BuPre {
-    int hv, beg, end;
+    int hv[kBuV];
 };
 
-__device__ __forceinline__ BuPre bu_prefetch(const DevGraph &G, int base) {
-    const int v = base + (threadIdx.x & 31);
-    BuPre p{-1, 0, 0};
-    if (v < G.n) {
-        p.hv = lcg(&G.h[v]);
-        p.beg = __ldg(&G.row[v]);
-        p.end = __ldg(&G.row[v + 1]);
+__device__ __forceinline__ BuPre bu_prefetch(const DevGraph &G, long long base) {
+    BuPre p;
+#pragma unroll
+    for (int q = 0; q < kBuV; ++q) {
+        const long long v = base + 32 * q + (threadIdx.x & 31);
+        p.hv[q] = v < G.n ? lcg(&G.h[v]) : -1;
     }
     return p;
 }
@@ -724,63 +730,72 @@ __device__ __forceinline__ BuPre bu_prefetch(const DevGraph &G, int base) {
 __device__ __forceinline__ void bfs_bottom_up_group(const DevGraph &G, int base, const BuPre &pre, bool dual, int L,
                                                     Front &F, int *ccnt, Counters &K) {
     const int lane = threadIdx.x & 31;
-    const int n = G.n;
-    const int v = base + lane;
-    int beg = 0, deg = 0;
-    const int side = (dual && v < n) ? G.part[v] : kPartT;
-    if (v < n && v != G.s && pre.hv == n) {
-        beg = pre.beg;
-        deg = pre.end - beg;
-        if (deg > kBigDeg) {
-            const int nc = (deg + kChunk - 1) / kChunk;
+    int v[kBuV], beg[kBuV], left[kBuV];   // left: arcs not yet scanned (0: found, or nothing to do)
+    bool un[kBuV], pull[kBuV], any = false;
+#pragma unroll
+    for (int q = 0; q < kBuV; ++q) {
+        v[q] = base + 32 * q + lane;
+        un[q] = pre.hv[q] == G.n && v[q] != G.s;
+        any |= un[q];
+    }
+    if (!__any_sync(kFull, any)) return;
+#pragma unroll
+    for (int q = 0; q < kBuV; ++q) {
+        beg[q] = un[q] ? __ldg(&G.row[v[q]]) : 0;
+        left[q] = un[q] ? __ldg(&G.row[v[q] + 1]) : 0;
+        pull[q] = dual && un[q] && G.part[v[q]] == kPartS;
+    }
+#pragma unroll
+    for (int q = 0; q < kBuV; ++q) {
+        left[q] -= beg[q];
+        if (left[q] > kBigDeg) {
+            const int nc = (left[q] + kChunk - 1) / kChunk;
             const int pos = atomicAdd(ccnt, nc);
-            for (int c = 0; c < nc; ++c) G.cb[pos + c] = make_int2(v, beg + c * kChunk);
-            deg = 0;
+            for (int c = 0; c < nc; ++c) G.cb[pos + c] = make_int2(v[q], beg[q] + c * kChunk);
+            left[q] = 0;
         }
     }
-    const unsigned want = __ballot_sync(kFull, deg > 0);
-    unsigned found = 0;
-    if (want) {
-        int incl = deg;
+    bool disc[kBuV];
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int y = __shfl_up_sync(kFull, incl, o);
-            if (lane >= o) incl += y;
-        }
-        const int total = __shfl_sync(kFull, incl, 31);
-        const int excl = incl - deg;
-        const unsigned pull_lanes = __ballot_sync(kFull, side == kPartS);
-        for (int k0 = 0; k0 < total && found != want; k0 += 32 * kIlpB) {
-            int a[kIlpB], own[kIlpB], ra[kIlpB], w[kIlpB];
+    for (int q = 0; q < kBuV; ++q) disc[q] = false;
+    for (;;) {
+        int ra[kBuV][kBuArcs], w[kBuV][kBuArcs];
+        any = false;
 #pragma unroll
-            for (int jj = 0; jj < kIlpB; ++jj) {
-                const int k = k0 + 32 * jj + lane;
-                int j = 0;
+        for (int q = 0; q < kBuV; ++q) any |= left[q] > 0;
+        if (!__any_sync(kFull, any)) break;
 #pragma unroll
-                for (int step = 16; step >= 1; step >>= 1) {
-                    const int cand = j + step;
-                    const int ex = __shfl_sync(kFull, excl, cand & 31);
-                    if (cand < 32 && ex <= k) j = cand;
-                }
-                own[jj] = j;
-                a[jj] = __shfl_sync(kFull, beg, j) + (k - __shfl_sync(kFull, excl, j));
-                const bool live = k < total && !((found >> j) & 1u);
-                ra[jj] = live ? lcg(((pull_lanes >> j) & 1u) ? &G.rr[a[jj]] : &G.r[a[jj]]) : 0;
-                w[jj] = live ? __ldg(&G.head[a[jj]]) : 0;
-                K.bfs_arcs += live;
+        for (int q = 0; q < kBuV; ++q)
+#pragma unroll
+            for (int j = 0; j < kBuArcs; ++j) {
+                const bool ok = j < left[q];
+                const int a = beg[q] + j;
+                // (residuals do not change during the search)
+                ra[q][j] = ok ? __ldca(pull[q] ? &G.rr[a] : &G.r[a]) : 0;
+                w[q][j] = ok ? __ldg(&G.head[a]) : 0;
+                K.bfs_arcs += ok;
             }
-            unsigned hit = 0;
+        bool hit[kBuV][kBuArcs];
 #pragma unroll
-            for (int jj = 0; jj < kIlpB; ++jj)
-                if (ra[jj] > 0 && lheight(&G.h[w[jj]]) == L &&
-                    (!dual || G.part[w[jj]] == (((pull_lanes >> own[jj]) & 1u) ? kPartS : kPartT)))
-                    hit |= 1u << own[jj];
-            found |= __reduce_or_sync(kFull, hit);
+        for (int q = 0; q < kBuV; ++q)
+#pragma unroll
+            for (int j = 0; j < kBuArcs; ++j) {
+                const int hw = ra[q][j] > 0 ? lheight(&G.h[w[q][j]]) : -1;
+                hit[q][j] = hw == L;
+                if (dual && hit[q][j]) hit[q][j] = (G.part[w[q][j]] == kPartS) == pull[q];
+            }
+#pragma unroll
+        for (int q = 0; q < kBuV; ++q) {
+#pragma unroll
+            for (int j = 0; j < kBuArcs; ++j) disc[q] |= hit[q][j];
+            beg[q] += kBuArcs;
+            left[q] = disc[q] ? 0 : left[q] - kBuArcs;
         }
     }
-    const bool disc = (found >> lane) & 1u;
-    if (disc) G.h[v] = L + 1;
-    bfs_discovered(G, disc, v, side == kPartS, dual, F, K);
+#pragma unroll
+    for (int q = 0; q < kBuV; ++q)
+        if (disc[q]) G.h[v[q]] = L + 1;
+    front_stage_n(G, disc, v, F, dual, K);
 }
 
 // Bottom-up scan of one kChunk-arc item of a high-degree unvisited vertex;
@@ -1969,7 +1984,7 @@ __device__ __forceinline__ void bfs_visit_staged(const DevGraph &G, const int *s
 // their trip.  Which of the found vertices are active is looked up afterwards,
 // for the whole run.  (Measured on grids, per level: frontier of vertices, rows
 // and excesses looked up and global lists reserved in every level 4.6-5.7 us,
-// now @@.)
+// now 2.9-4.0 us.)
 constexpr int kSoloWl = 12288;      // found vertices kept at most
 constexpr int kSoloBig = 128;       // frontier vertices of degree > kBigDeg: at most kSoloArcs / (kBigDeg + 1)
 constexpr int kSoloCas = 1024;      // arcs up to which every residual arc tries the CAS at once
@@ -2160,7 +2175,7 @@ __device__ __forceinline__ void bfs_solo(const DevGraph &G, int L, int cur, long
         b ^= 1;
         cs = W.nv[b];
         mfs = (long long)W.arcs[b];
-        const bool out = cs == 0 || cs > kSoloCap || mfs > kSoloArcs || (mfs * 14 > G.A - (seen + mfs) && cs * 64LL > n);
+        const bool out = cs == 0 || cs > kSoloCap || mfs > G.solo_arcs || (mfs * G.alpha > G.A - (seen + mfs) && cs * 64LL > n);
         const int nw = W.nw + cs;   // vertices found so far
         __syncthreads();   // everyone has read the counts
         if (tid == 0) W.nw = nw;
@@ -2530,43 +2545,73 @@ __global__ void __launch_bounds__(kBlock, 1) k_solve(DevGraph G, Job J) {
             if (gtimer() - C->t_start > J.time_limit_ns) C->abort_loop = 1;
         }
         {
+            // (the roots are staged per warp like a frontier: a push-pull repair
+            // of a grid has millions, and an append per 32 vertices queued
+            // 130,000 atomics on one word: 4M vertices 56 -> 20 us)
             long long dsum = 0, rdeg = 0;
-            constexpr int kRs = 4;   // vertices in flight per thread (their excesses loaded first)
+            constexpr int kRs = 4;   // vertices in flight per thread
+            int *const roots = s_bfs + (threadIdx.x >> 5) * kWq;
+            int nroots = 0;   // staged (warp-uniform)
+            auto publish = [&]() {
+                __syncwarp();
+                int base = 0;
+                if (lane == 0) base = atomicAdd(&C->qcnt[0], nroots);
+                base = __shfl_sync(kFull, base, 0);
+                for (int i = lane; i < nroots; i += 32) G.qb0[base + i] = roots[i];
+                __syncwarp();
+                nroots = 0;
+            };
             for (long long vb0 = (long long)gwarp * 32; vb0 < n; vb0 += kRs * gthreads) {
                 long long evs[kRs];
+                unsigned char pts[kRs];
+                bool root[kRs];
+                int r0[kRs], r1[kRs];
 #pragma unroll
                 for (int j = 0; j < kRs; ++j) {
                     const long long v = vb0 + j * gthreads + lane;
                     evs[j] = v < n ? lcg(&G.e[v]) : 0;
+                    pts[j] = stage && v < n ? G.part[v] : kPartT;
                 }
 #pragma unroll
                 for (int j = 0; j < kRs; ++j) {
                     const long long v = vb0 + j * gthreads + lane;
-                    bool root = false;
-                    if (v < n) {
-                        const long long ev = evs[j];
-                        if (stage == 0) {
-                            root = (v == t) || (v != s && ev < 0);
-                            G.h[v] = root ? 0 : n;
-                            if (root && v != t) dsum += ev;
-                        } else if (stage == 1) {
-                            // Alg. 8: h+ roots are t and the deficient vertices of T,
-                            // h- roots are s and the overflowing vertices of S (both
-                            // heights live in h: the two sides are disjoint)
-                            root = G.part[v] == kPartT ? (v == t || ev < 0) : (v == s || ev > 0);
-                            G.h[v] = root ? 0 : n;
-                        } else {
-                            // the subgraph P: its deficient vertices are the sinks;
-                            // the rest of the graph sits at n + 1, out of reach
-                            const bool inP = G.part[v] == kPartP;
-                            root = inP && ev < 0;
-                            G.h[v] = inP ? (root ? 0 : n) : n + 1;
-                        }
-                        if (root) rdeg += __ldg(&G.row[v + 1]) - __ldg(&G.row[v]);
+                    const long long ev = evs[j];
+                    root[j] = false;
+                    if (v >= n) continue;
+                    if (stage == 0) {
+                        root[j] = (v == t) || (v != s && ev < 0);
+                        G.h[v] = root[j] ? 0 : n;
+                        if (root[j] && v != t) dsum += ev;
+                    } else if (stage == 1) {
+                        // Alg. 8: h+ roots are t and the deficient vertices of T,
+                        // h- roots are s and the overflowing vertices of S (both
+                        // heights live in h: the two sides are disjoint)
+                        root[j] = pts[j] == kPartT ? (v == t || ev < 0) : (v == s || ev > 0);
+                        G.h[v] = root[j] ? 0 : n;
+                    } else {
+                        // the subgraph P: its deficient vertices are the sinks;
+                        // the rest of the graph sits at n + 1, out of reach
+                        const bool inP = pts[j] == kPartP;
+                        root[j] = inP && ev < 0;
+                        G.h[v] = inP ? (root[j] ? 0 : n) : n + 1;
                     }
-                    warp_append(root, (int)v, &C->qcnt[0], G.qb0);
+                }
+#pragma unroll
+                for (int j = 0; j < kRs; ++j) {
+                    const long long v = vb0 + j * gthreads + lane;
+                    r0[j] = root[j] ? __ldg(&G.row[v]) : 0;
+                    r1[j] = root[j] ? __ldg(&G.row[v + 1]) : 0;
+                }
+                if (nroots > kWq - 32 * kRs) publish();
+#pragma unroll
+                for (int j = 0; j < kRs; ++j) {
+                    rdeg += r1[j] - r0[j];
+                    const unsigned m = __ballot_sync(kFull, root[j]);
+                    if (root[j]) roots[nroots + __popc(m & ((1u << lane) - 1u))] = (int)(vb0 + j * gthreads + lane);
+                    nroots += __popc(m);
                 }
             }
+            if (nroots) publish();
             dsum = warp_sum(dsum);
             rdeg = warp_sum(rdeg);
             if (lane == 0 && dsum) add_ll(&C->dacc[par], dsum);
@@ -2581,7 +2626,7 @@ __global__ void __launch_bounds__(kBlock, 1) k_solve(DevGraph G, Job J) {
         // backward BFS from the sinks over residual arcs (global relabel),
         // level-synchronous and direction-optimising: top-down from the
         // frontier while it is small, bottom-up from the unvisited vertices
-        // while the frontier holds more than 1/14 of the unvisited arcs.
+        // while the frontier holds more than 1/alpha of the unvisited arcs.
         int L = 0;
         bool bottom_up = false;
         long long arcs_seen = 0;
@@ -2595,9 +2640,9 @@ __global__ void __launch_bounds__(kBlock, 1) k_solve(DevGraph G, Job J) {
             // first frontier, the overflowing and deficient vertices of both
             // sides, is a few percent of the vertices but touches few of the
             // others, which then scan all their arcs bottom-up)
-            if (!bottom_up) bottom_up = mf * 14 > G.A - arcs_seen && cur * (dual ? 32LL : 64LL) > n;
+            if (!bottom_up) bottom_up = mf * G.alpha > G.A - arcs_seen && cur * (dual ? 32LL : 64LL) > n;
             else bottom_up = cur * 24LL >= n;
-            if (!bottom_up && mf <= kSoloArcs && cur <= kSoloCap) {
+            if (!bottom_up && mf <= G.solo_arcs && cur <= kSoloCap) {
                 // a small frontier: CTA 0 runs the levels alone (bfs_solo).
                 // Every thread has read this level's counters before it starts
                 // (the first barrier).
@@ -2621,16 +2666,17 @@ __global__ void __launch_bounds__(kBlock, 1) k_solve(DevGraph G, Job J) {
             }
             Front FR{ncnt, NF, asum, 0x7fffffff, nullptr, s_bfs + (threadIdx.x >> 5) * kWq, 0, 0};
             if (bottom_up) {
-                // groups of 32 consecutive vertex ids
-                const int groups = (n + 31) / 32;
+                // pieces of 32 kBuV consecutive vertex ids
+                constexpr int kPiece = 32 * kBuV;
+                const int groups = (n + kPiece - 1) / kPiece;
                 int *const tick = cta_words();
                 int grp = gwarp, nxt;
-                BuPre pre = bu_prefetch(G, min(grp, groups) * 32);
+                BuPre pre = bu_prefetch(G, (long long)min(grp, groups) * kPiece);
                 for (; grp < groups; grp = nxt) {
                     const BuPre cur = pre;
                     nxt = next_item(tick, groups);
-                    pre = bu_prefetch(G, min(nxt, groups) * 32);
-                    bfs_bottom_up_group(G, grp * 32, cur, dual, L, FR, ccnt, K);
+                    pre = bu_prefetch(G, (long long)min(nxt, groups) * kPiece);
+                    bfs_bottom_up_group(G, grp * kPiece, cur, dual, L, FR, ccnt, K);
                 }
             } else {
                 // groups of gs frontier vertices:
@@ -3535,6 +3581,23 @@ int read_ctl(mf_graph *g, Ctl *out, size_t bytes = sizeof(Ctl)) {
     return MF_OK;
 }
 
+// Where the search changes hands (see k_solve).
+//  alpha      bottom-up pays early where a vertex finds a parent soon: in a
+//             renumbered graph, whose rows begin with the likely parents, and
+//             where rows are short.  Long rows of alike heads are mostly read
+//             whole (unit assignment graph of degree 18, alpha 14 / 8 / 4 / 2:
+//             1.33 / 1.26 / 1.19 / 1.17 ms a batch; 1023 x 769 grid, degree 8,
+//             its searches 256 us with 14, 297 with 4).
+//  solo_arcs  one CTA keeps up with a thin wave of short rows (2048^2 grid: 4
+//             us a level against 7.5 on the whole grid), less so with
+//             the tails of a power-law search, whose rows are long and mostly
+//             lead back (RMAT-20 static solve with 8192 / 4096 / 2048: 2.33 /
+//             2.28 / 2.23 ms).
+void search_rules(DevGraph &D, bool renumbered) {
+    D.alpha = renumbered || D.A <= 8LL * D.n ? 14 : 3;
+    D.solo_arcs = renumbered ? 2048 : int(kSoloArcs);
+}
+
 int launch(mf_graph *g, const Job &job, cudaStream_t st) {
     DevGraph dg = g->dg;
     Job jb = job;
@@ -3810,6 +3873,7 @@ int mf_create(int32_t n, int64_t m, const int64_t *row_ptr, const int32_t *col, 
     // an allocator callback may hand out blocks without 16-byte alignment:
     // the staging copies then fall back to plain loads
     auto al16 = [](const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; };
+    search_rules(D, !g->ord.empty());
     D.al16 = al16(D.head) && al16(D.r) && al16(D.rr);
     if (!row || !head || !rev || !aoe || !est || !D.cap || !D.r || !D.rr || !D.h || !D.e || !D.cap_edge || !D.stamp ||
         !D.qb0 || !D.qb1 || !D.wl || !D.cb || !D.ctl || !g->side_buf || !D.hl || !D.hkey ||
@@ -4413,6 +4477,7 @@ int mf_solve_bicsr_noalloc(int32_t n, int64_t arcs, const int32_t *row, const in
     D.hri = reinterpret_cast<int2 *>(b + Lo::hri);
     D.aq = reinterpret_cast<unsigned long long *>(b + Lo::aq);
     D.qc = std::min(std::max(n, 1024), kNoAllocMaxN);
+    search_rules(D, false);
     // the previous call's contents stay in the array: clear what must start at 0
     MF_CUDA(cudaMemsetAsync(D.ctl, 0, sizeof(Ctl), st));
     MF_CUDA(cudaMemsetAsync(D.aq, 0, sizeof(unsigned long long) * size_t(D.qc), st));
