@@ -99,9 +99,10 @@ typedef struct mf_graph mf_graph;
  *  max_iters      cap on loop iterations (one BFS + PushRelabel +
  *                 RemoveInvalidEdges round) of one solve or repair; reaching
  *                 it reports MF_ETIMEOUT.  0 = 4 * n + 1000.
- *  grid_blocks    CTAs of the persistent solver kernel; 0 = one full wave
- *                 (co-resident CTAs per SM x SM count).  Larger values are
- *                 clamped to one full wave.
+ *  grid_blocks    CTAs of the persistent solver kernel; 0 = chosen from the
+ *                 graph's size: one full wave (co-resident CTAs per SM x SM
+ *                 count), fewer for graphs too small to fill it.  Larger
+ *                 values are clamped to one full wave.
  *  time_limit_ms  wall-clock limit of one solve/repair kernel, checked once
  *                 per loop iteration; passing it reports MF_ETIMEOUT.
  *                 0 = 60000.
