@@ -44,6 +44,7 @@
 #include <mutex>
 #include <new>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "mf.h"
@@ -1979,29 +1980,33 @@ __device__ __forceinline__ void bfs_visit_staged(const DevGraph &G, const int *s
 // queue.  What bounds a level is its chain of round trips, so the frontier is
 // kept in shared memory as the list of its arcs (sign bit: searched forward,
 // on the pull side of a push-pull repair), written when a vertex is found: a
-// level takes four trips (heads and residuals; heights; the claiming CAS; rows
-// of what it found), three where few arcs make the height reads not worth
-// their trip.  Which of the found vertices are active is looked up afterwards,
-// for the whole run.  (Measured on grids, per level: frontier of vertices, rows
-// and excesses looked up and global lists reserved in every level 4.6-5.7 us,
-// now 2.9-4.0 us.)
+// level takes three trips (heads and residuals; heights; the claiming CAS and,
+// with it, the rows of what it claims), two where few arcs make the height
+// reads not worth their trip, and one __syncthreads.  A level of at most one
+// arc per thread runs code for one (the four slots' instructions were a third
+// of its time).  Which of the found vertices are active is looked up
+// afterwards, for the whole run.  (Measured on grids, per level: frontier of
+// vertices, rows and excesses looked up and global lists reserved in every
+// level 4.6-5.7 us; rows after the claims, two barriers, four slots always
+// 3.0-3.9 us; now 2.5-3.2 us.)
 constexpr int kSoloWl = 12288;      // found vertices kept at most
 constexpr int kSoloBig = 128;       // frontier vertices of degree > kBigDeg: at most kSoloArcs / (kBigDeg + 1)
 constexpr int kSoloCas = 1024;      // arcs up to which every residual arc tries the CAS at once
 static_assert(kSoloArcs / (kBigDeg + 1) <= kSoloBig, "big vertices of a small frontier");
 static_assert(2 * kSoloArcs + 2 * kSoloCap + kSoloWl + 4 * kSoloBig <= kDynSmem / 4, "shared lists of a small frontier");
 
-struct SoloWords {
-    int nv[2], nbig[2];     // frontier vertices and big vertices, by level parity
-    int na[2];              // arcs of the others
-    unsigned arcs[2];       // all arcs (fewer than 2^31)
-    int nw;                 // vertices found before the current level, and kept
+// A level's frontier, the next one's and the one before, rotating: with three
+// a level needs one __syncthreads.
+struct alignas(16) SoloFront {
+    int nv, nbig;      // vertices, big ones
+    int na;            // arcs of the others
+    unsigned arcs;     // all arcs (fewer than 2^31)
 };
 
 __device__ __forceinline__ void bfs_solo(const DevGraph &G, int L, int cur, long long arcs_seen, bool dual, int *smem,
                                          long long *s_stat, unsigned long long &tprev, long long it, TraceRec *trace,
                                          Counters &K) {
-    __shared__ SoloWords W;
+    __shared__ SoloFront W[3];
     Ctl *C = G.ctl;
     const int n = G.n, tid = threadIdx.x, lane = tid & 31;
     int *const sv[2] = {smem, smem + kSoloCap};
@@ -2009,15 +2014,18 @@ __device__ __forceinline__ void bfs_solo(const DevGraph &G, int L, int cur, long
     int *const swl = smem + 2 * kSoloCap + 2 * (int)kSoloArcs;
     int2 *const sbig[2] = {reinterpret_cast<int2 *>(swl + kSoloWl), reinterpret_cast<int2 *>(swl + kSoloWl) + kSoloBig};
 
-    // The lanes' flagged vertices of kIlpB slots, rows [beg, end), join frontier
-    // q (positions from kSoloCap on go to spill); a sets the sign of their
-    // arcs.  One reservation per warp and counter.  All 32 lanes call.
-    auto add = [&](const bool (&ok)[kIlpB], const int (&v)[kIlpB], const int (&beg)[kIlpB], const int (&end)[kIlpB],
-                   const int (&a)[kIlpB], int q, int *spill, bool found) {
+    int nw = 0;   // vertices found before the current level, and kept (CTA-uniform)
+
+    // The lanes' flagged vertices of J slots, rows [beg, end), join frontier w,
+    // lists q (positions from kSoloCap on go to spill); a sets the sign of
+    // their arcs.  One reservation per warp and counter.  All 32 lanes call.
+    auto add = [&](const auto &ok, const auto &v, const auto &beg, const auto &end, const auto &a, SoloFront *w, int q,
+                   int *spill, bool found) {
+        constexpr int J = sizeof(v) / sizeof(int);
         unsigned mine = 0;   // this lane's vertices (high half) and listed arcs (low half)
         unsigned all = 0;
 #pragma unroll
-        for (int j = 0; j < kIlpB; ++j)
+        for (int j = 0; j < J; ++j)
             if (ok[j]) {
                 const int deg = end[j] - beg[j];
                 all += (unsigned)deg;
@@ -2032,21 +2040,21 @@ __device__ __forceinline__ void bfs_solo(const DevGraph &G, int L, int cur, long
         }
         int pv = 0, pa = 0;
         if (lane == 31) {
-            pv = atomicAdd(&W.nv[q], (int)(incl >> 16));
-            pa = atomicAdd(&W.na[q], (int)(incl & 0xffffu));
-            atomicAdd(&W.arcs[q], all);
+            pv = atomicAdd(&w->nv, (int)(incl >> 16));
+            pa = atomicAdd(&w->na, (int)(incl & 0xffffu));
+            atomicAdd(&w->arcs, all);
         }
         pv = __shfl_sync(kFull, pv, 31) + (int)((incl - mine) >> 16);
         pa = __shfl_sync(kFull, pa, 31) + (int)((incl - mine) & 0xffffu);
 #pragma unroll
-        for (int j = 0; j < kIlpB; ++j) {
+        for (int j = 0; j < J; ++j) {
             if (!ok[j]) continue;
             const int deg = end[j] - beg[j], sign = a[j] & (int)0x80000000u;
             (pv < kSoloCap ? sv[q] : spill)[pv] = v[j];
-            if (found) swl[W.nw + pv] = v[j] | sign;
+            if (found) swl[nw + pv] = v[j] | sign;
             ++pv;
             if (deg > kBigDeg) {
-                const int k = atomicAdd(&W.nbig[q], 1);
+                const int k = atomicAdd(&w->nbig, 1);
                 if (k < kSoloBig) sbig[q][k] = make_int2(beg[j] | sign, end[j]);
             } else {
                 // (a frontier of more than kSoloArcs arcs is handed back: its
@@ -2057,63 +2065,77 @@ __device__ __forceinline__ void bfs_solo(const DevGraph &G, int L, int cur, long
             }
         }
     };
-    // kIlpB arcs per lane (ok[j]: arc a[j], sign set: searched forward)
-    auto visit = [&](const int (&a)[kIlpB], const bool (&ok)[kIlpB], bool cas, int Ls, int q, int *spill) {
-        int v[kIlpB], rin[kIlpB], beg[kIlpB], end[kIlpB];
-        bool disc[kIlpB];
+    // J arcs per lane (ok[j]: arc a[j], sign set: searched forward)
+    auto visit = [&](const auto &a, const auto &ok, bool cas, int Ls, SoloFront *w, int q, int *spill) {
+        constexpr int J = sizeof(a) / sizeof(int);
+        int v[J], rin[J], beg[J], end[J];
+        bool disc[J];
 #pragma unroll
-        for (int j = 0; j < kIlpB; ++j) {
+        for (int j = 0; j < J; ++j) {
             const int x = a[j] & 0x7fffffff;
             v[j] = ok[j] ? __ldg(&G.head[x]) : 0;
             rin[j] = ok[j] ? lcg(a[j] < 0 ? &G.r[x] : &G.rr[x]) : 0;
             K.bfs_arcs += ok[j];
         }
 #pragma unroll
-        for (int j = 0; j < kIlpB; ++j) disc[j] = rin[j] > 0 && v[j] != G.s;
+        for (int j = 0; j < J; ++j) disc[j] = rin[j] > 0 && v[j] != G.s;
         if (!cas) {
-            int hv[kIlpB];
+            int hv[J];
 #pragma unroll
-            for (int j = 0; j < kIlpB; ++j) hv[j] = disc[j] ? lcg(&G.h[v[j]]) : 0;
+            for (int j = 0; j < J; ++j) hv[j] = disc[j] ? lcg(&G.h[v[j]]) : 0;
 #pragma unroll
-            for (int j = 0; j < kIlpB; ++j) disc[j] = disc[j] && hv[j] == n;
+            for (int j = 0; j < J; ++j) disc[j] = disc[j] && hv[j] == n;
         }
-        int old[kIlpB];
+        // (the rows of all that are tried, on the same trip as the claims)
+        int old[J];
 #pragma unroll
-        for (int j = 0; j < kIlpB; ++j) old[j] = disc[j] ? atomicCAS(&G.h[v[j]], n, Ls + 1) : 0;
-        bool any = false;
-#pragma unroll
-        for (int j = 0; j < kIlpB; ++j) {
-            disc[j] = disc[j] && old[j] == n;
-            any |= disc[j];
-        }
-        if (!__any_sync(kFull, any)) return;
-#pragma unroll
-        for (int j = 0; j < kIlpB; ++j) {
+        for (int j = 0; j < J; ++j) {
+            old[j] = disc[j] ? atomicCAS(&G.h[v[j]], n, Ls + 1) : 0;
             beg[j] = disc[j] ? __ldg(&G.row[v[j]]) : 0;
             end[j] = disc[j] ? __ldg(&G.row[v[j] + 1]) : 0;
+        }
+        bool any = false;
+#pragma unroll
+        for (int j = 0; j < J; ++j) {
+            disc[j] = disc[j] && old[j] == n;
+            any |= disc[j];
             K.bfs_verts += disc[j];
         }
-        add(disc, v, beg, end, a, q, spill, true);
+        if (__any_sync(kFull, any)) add(disc, v, beg, end, a, w, q, spill, true);
+    };
+    // the level's listed arcs, J per thread at once
+    auto scan = [&](auto jc, int na, int q, bool cas, int Ls, SoloFront *w, int *spill) {
+        constexpr int J = decltype(jc)::value;
+        for (int k0 = tid & ~31; k0 < na; k0 += J * kBlock) {
+            int a[J];
+            bool ok[J];
+#pragma unroll
+            for (int j = 0; j < J; ++j) {
+                const int k = k0 + j * kBlock + lane;
+                ok[j] = k < na;
+                a[j] = ok[j] ? sa[q][k] : 0;
+            }
+            visit(a, ok, cas, Ls, w, q ^ 1, spill);
+        }
     };
     // the active ones of the vertices found so far join the global lists (a
     // vertex of the pull side is active when deficient); every thread calls,
     // between barriers
     auto flush = [&]() {
-        const int k = W.nw;
-        for (int i0 = 0; i0 < k; i0 += kBlock) {
+        for (int i0 = 0; i0 < nw; i0 += kBlock) {
             const int i = i0 + tid;
-            const int x = i < k ? swl[i] : 0, v = x & 0x7fffffff;
-            const long long ev = i < k ? lcg(&G.e[v]) : 0;
-            const int deg = i < k ? __ldg(&G.row[v + 1]) - __ldg(&G.row[v]) : 0;
-            const bool act = i < k && (x < 0 ? ev < 0 : ev > 0);
+            const int x = i < nw ? swl[i] : 0, v = x & 0x7fffffff;
+            const long long ev = i < nw ? lcg(&G.e[v]) : 0;
+            const int deg = i < nw ? __ldg(&G.row[v + 1]) - __ldg(&G.row[v]) : 0;
+            const bool act = i < nw && (x < 0 ? ev < 0 : ev > 0);
             warp_append(act && deg <= kHubDeg, v, &C->wcnt, G.wl);
             warp_append(act && deg > kHubDeg, v, &C->hcnt, G.hl);
         }
         __syncthreads();
-        if (tid == 0) W.nw = 0;
+        nw = 0;
     };
 
-    if (tid == 0) W = SoloWords{};
+    if (tid < 3) W[tid] = SoloFront{0, 0, 0, 0};
     __syncthreads();
     const int *F0 = (L & 1) ? G.qb1 : G.qb0;
     for (int i0 = 0; i0 < cur; i0 += kBlock) {
@@ -2128,27 +2150,21 @@ __device__ __forceinline__ void bfs_solo(const DevGraph &G, int L, int cur, long
             end[j] = ok[j] ? __ldg(&G.row[v[j] + 1]) : 0;
             a[j] = ok[j] && dual && G.part[v[j]] == kPartS ? (int)0x80000000u : 0;
         }
-        add(ok, v, beg, end, a, 0, nullptr, false);   // (at most kSoloCap vertices)
+        add(ok, v, beg, end, a, &W[0], 0, nullptr, false);   // (at most kSoloCap vertices)
     }
     __syncthreads();
-    int Ls = L, b = 0, cs = cur;
+    int Ls = L, b = 0, c = 0, cs = cur;   // b: the level's lists, c: its counts
     long long seen = arcs_seen, mfs = 0;
+    SoloFront f = W[0];
     for (;;) {
         int *spill = (Ls & 1) ? G.qb0 : G.qb1;   // positions >= kSoloCap of the next frontier
-        const int na = W.na[b], nbig = W.nbig[b];
-        const bool cas = na <= kSoloCas;
-        for (int k0 = 0; k0 < na; k0 += kIlpB * kBlock) {
-            int a[kIlpB];
-            bool ok[kIlpB];
-#pragma unroll
-            for (int j = 0; j < kIlpB; ++j) {
-                const int k = k0 + j * kBlock + tid;
-                ok[j] = k < na;
-                a[j] = ok[j] ? sa[b][k] : 0;
-            }
-            visit(a, ok, cas, Ls, b ^ 1, spill);
-        }
-        for (int q = tid >> 5; q < nbig; q += kBlock / 32) {
+        SoloFront *const w = &W[c == 2 ? 0 : c + 1];
+        if (tid == 0) W[c == 0 ? 2 : c - 1] = SoloFront{0, 0, 0, 0};   // (read a barrier ago)
+        if (f.na <= kBlock)
+            scan(std::integral_constant<int, 1>{}, f.na, b, f.na <= kSoloCas, Ls, w, spill);
+        else
+            scan(std::integral_constant<int, kIlpB>{}, f.na, b, f.na <= kSoloCas, Ls, w, spill);
+        for (int q = tid >> 5; q < f.nbig; q += kBlock / 32) {
             const int2 r = sbig[b][q];
             const int a0 = r.x & 0x7fffffff;
             for (int ab = a0; ab < r.y; ab += 32 * kIlpB) {
@@ -2160,7 +2176,7 @@ __device__ __forceinline__ void bfs_solo(const DevGraph &G, int L, int cur, long
                     ok[j] = x < r.y;
                     a[j] = x | (r.x & (int)0x80000000u);
                 }
-                visit(a, ok, false, Ls, b ^ 1, spill);
+                visit(a, ok, false, Ls, w, b ^ 1, spill);
             }
         }
         __syncthreads();
@@ -2173,23 +2189,15 @@ __device__ __forceinline__ void bfs_solo(const DevGraph &G, int L, int cur, long
         }
         ++Ls;
         b ^= 1;
-        cs = W.nv[b];
-        mfs = (long long)W.arcs[b];
+        c = c == 2 ? 0 : c + 1;
+        f = *w;
+        cs = f.nv;
+        mfs = (long long)f.arcs;
         const bool out = cs == 0 || cs > kSoloCap || mfs > G.solo_arcs || (mfs * G.alpha > G.A - (seen + mfs) && cs * 64LL > n);
-        const int nw = W.nw + cs;   // vertices found so far
-        __syncthreads();   // everyone has read the counts
-        if (tid == 0) W.nw = nw;
-        if (out || nw > kSoloWl - (int)kSoloArcs) {
-            __syncthreads();
-            flush();
-        }
-        if (tid == 0) {
-            W.nv[b ^ 1] = W.nbig[b ^ 1] = W.na[b ^ 1] = 0;
-            W.arcs[b ^ 1] = 0;
-        }
+        nw += cs;
+        if (out || nw > kSoloWl - (int)kSoloArcs) flush();
         if (out) break;
         seen += mfs;
-        __syncthreads();
     }
     // hand the frontier of level Ls back in the global queue
     int *Fg = (Ls & 1) ? G.qb1 : G.qb0;
