@@ -508,9 +508,9 @@ struct Front {
 __device__ __forceinline__ void front_flush_entries(const DevGraph &G, Front &F, bool dual, Counters &K) {
     const int lane = threadIdx.x & 31;
     __syncwarp();
+    // (the reservation is on its way while the vertices are looked up)
     int base = 0;
     if (lane == 0) base = atomicAdd(F.cnt, F.sn);
-    base = __shfl_sync(kFull, base, 0);
     long long ds = 0;
     for (int i0 = 0; i0 < F.sn; i0 += 32 * kFl) {
         int v[kFl], deg[kFl];
@@ -521,13 +521,16 @@ __device__ __forceinline__ void front_flush_entries(const DevGraph &G, Front &F,
             const int i = i0 + 32 * j + lane;
             ok[j] = i < F.sn;
             v[j] = ok[j] ? F.stage[i] : 0;
-            if (ok[j]) F.buf[base + i] = v[j];
         }
 #pragma unroll
         for (int j = 0; j < kFl; ++j) {
             deg[j] = ok[j] ? __ldg(&G.row[v[j] + 1]) - __ldg(&G.row[v[j]]) : 0;
             ev[j] = ok[j] ? lcg(&G.e[v[j]]) : 0;
         }
+        if (i0 == 0) base = __shfl_sync(kFull, base, 0);
+#pragma unroll
+        for (int j = 0; j < kFl; ++j)
+            if (ok[j]) F.buf[base + i0 + 32 * j + lane] = v[j];
 #pragma unroll
         for (int j = 0; j < kFl; ++j) {
             // a vertex of the pull side (forward search) is active when deficient
