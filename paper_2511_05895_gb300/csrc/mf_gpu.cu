@@ -224,6 +224,7 @@ struct DevGraph {
     int al16;                 // head, r and rr start on 16-byte boundaries (16-byte staging copies)
     unsigned long long *aq;   // activation queue slots (generation << 32 | vertex + 1; 0 = empty)
     int qc;                   // its capacity
+    int bu_long;              // bottom-up levels mostly read whole rows (search_rules)
     int solo_arcs;            // most arcs of a frontier that CTA 0 searches alone (<= kSoloArcs)
     int alpha;                // the search goes bottom-up when alpha x its frontier's arcs pass the unvisited arcs
 };
@@ -700,9 +701,9 @@ __device__ __forceinline__ void bfs_expand_warp(const DevGraph &G, int beg, int 
 }
 
 // Bottom-up step of the backward BFS (direction-optimising search): the
-// unvisited vertices v of kBuV groups of 32 consecutive ids look for a residual
+// unvisited vertices v of V groups of 32 consecutive ids look for a residual
 // arc v -> w into the current frontier (h(w) == L); the first one found gives
-// h(v) = L + 1.  A lane scans its own vertices, kBuArcs arcs of each at a time,
+// h(v) = L + 1.  A lane scans its own vertices, kArcs arcs of each at a time,
 // until it has found one: in the levels that matter most vertices find a
 // parent among their first arcs.  (The group's arcs balanced over the lanes
 // read whole rows, 128 arcs a round, before any vertex could stop, and paid
@@ -712,45 +713,58 @@ __device__ __forceinline__ void bfs_expand_warp(const DevGraph &G, int beg, int 
 // stage of a push-pull repair (dual) a vertex of the pull side looks for a
 // residual arc w -> v from the frontier instead, and only frontier vertices of
 // the vertex's own side count.  All 32 lanes call.
-constexpr int kBuV = 2, kBuArcs = 2;   // (1 x 4, 2 x 4, 1 x 8: 0-25 % slower on RMAT and grids)
+// The many-vertex shape (2 vertices, 2 arcs of each) is for levels with pieces
+// for every warp and parents among the first arcs (1 x 4, 2 x 4, 1 x 8: 0-25 %
+// slower on RMAT-20 and grids).  The long-row shape (1 vertex, 4 arcs) is for
+// graphs too small to give every warp a 64-vertex piece, where the rounds of
+// one lane are the level's time, and for rows that are mostly read whole
+// (search_rules): per level, many-vertex / long-row, 16,384 x 2 assignment
+// graph 21.0 / 14.6 us, 262,144 x 2 one 37.7 / 34.5 (its 9.4M random height
+// reads take 38 at the rate measured for L2), RMAT-16 8.2 / 7.3, 1,000-vertex
+// graph 6.7 / 5.4 (1 x 6, 1 x 8, 2 x 4: 2-60 % above 1 x 4).
+constexpr int kBuV = 2, kBuArcs = 2;
+constexpr int kBuVLong = 1, kBuArcsLong = 4;
 
 // The heights of a lane's vertices, loaded one piece ahead.  During a
 // bottom-up level only the owning lane writes an unvisited vertex's height, so
 // the early read is exact.
+template <int V>
 struct BuPre {
-    int hv[kBuV];
+    int hv[V];
 };
 
-__device__ __forceinline__ BuPre bu_prefetch(const DevGraph &G, long long base) {
-    BuPre p;
+template <int V>
+__device__ __forceinline__ BuPre<V> bu_prefetch(const DevGraph &G, long long base) {
+    BuPre<V> p;
 #pragma unroll
-    for (int q = 0; q < kBuV; ++q) {
+    for (int q = 0; q < V; ++q) {
         const long long v = base + 32 * q + (threadIdx.x & 31);
         p.hv[q] = v < G.n ? lcg(&G.h[v]) : -1;
     }
     return p;
 }
 
-__device__ __forceinline__ void bfs_bottom_up_group(const DevGraph &G, int base, const BuPre &pre, bool dual, int L,
+template <int V, int kArcs>
+__device__ __forceinline__ void bfs_bottom_up_group(const DevGraph &G, int base, const BuPre<V> &pre, bool dual, int L,
                                                     Front &F, int *ccnt, Counters &K) {
     const int lane = threadIdx.x & 31;
-    int v[kBuV], beg[kBuV], left[kBuV];   // left: arcs not yet scanned (0: found, or nothing to do)
-    bool un[kBuV], pull[kBuV], any = false;
+    int v[V], beg[V], left[V];   // left: arcs not yet scanned (0: found, or nothing to do)
+    bool un[V], pull[V], any = false;
 #pragma unroll
-    for (int q = 0; q < kBuV; ++q) {
+    for (int q = 0; q < V; ++q) {
         v[q] = base + 32 * q + lane;
         un[q] = pre.hv[q] == G.n && v[q] != G.s;
         any |= un[q];
     }
     if (!__any_sync(kFull, any)) return;
 #pragma unroll
-    for (int q = 0; q < kBuV; ++q) {
+    for (int q = 0; q < V; ++q) {
         beg[q] = un[q] ? __ldg(&G.row[v[q]]) : 0;
         left[q] = un[q] ? __ldg(&G.row[v[q] + 1]) : 0;
         pull[q] = dual && un[q] && G.part[v[q]] == kPartS;
     }
 #pragma unroll
-    for (int q = 0; q < kBuV; ++q) {
+    for (int q = 0; q < V; ++q) {
         left[q] -= beg[q];
         if (left[q] > kBigDeg) {
             const int nc = (left[q] + kChunk - 1) / kChunk;
@@ -759,19 +773,19 @@ __device__ __forceinline__ void bfs_bottom_up_group(const DevGraph &G, int base,
             left[q] = 0;
         }
     }
-    bool disc[kBuV];
+    bool disc[V];
 #pragma unroll
-    for (int q = 0; q < kBuV; ++q) disc[q] = false;
+    for (int q = 0; q < V; ++q) disc[q] = false;
     for (;;) {
-        int ra[kBuV][kBuArcs], w[kBuV][kBuArcs];
+        int ra[V][kArcs], w[V][kArcs];
         any = false;
 #pragma unroll
-        for (int q = 0; q < kBuV; ++q) any |= left[q] > 0;
+        for (int q = 0; q < V; ++q) any |= left[q] > 0;
         if (!__any_sync(kFull, any)) break;
 #pragma unroll
-        for (int q = 0; q < kBuV; ++q)
+        for (int q = 0; q < V; ++q)
 #pragma unroll
-            for (int j = 0; j < kBuArcs; ++j) {
+            for (int j = 0; j < kArcs; ++j) {
                 const bool ok = j < left[q];
                 const int a = beg[q] + j;
                 // (residuals do not change during the search)
@@ -779,25 +793,25 @@ __device__ __forceinline__ void bfs_bottom_up_group(const DevGraph &G, int base,
                 w[q][j] = ok ? __ldg(&G.head[a]) : 0;
                 K.bfs_arcs += ok;
             }
-        bool hit[kBuV][kBuArcs];
+        bool hit[V][kArcs];
 #pragma unroll
-        for (int q = 0; q < kBuV; ++q)
+        for (int q = 0; q < V; ++q)
 #pragma unroll
-            for (int j = 0; j < kBuArcs; ++j) {
+            for (int j = 0; j < kArcs; ++j) {
                 const int hw = ra[q][j] > 0 ? lheight(&G.h[w[q][j]]) : -1;
                 hit[q][j] = hw == L;
                 if (dual && hit[q][j]) hit[q][j] = (G.part[w[q][j]] == kPartS) == pull[q];
             }
 #pragma unroll
-        for (int q = 0; q < kBuV; ++q) {
+        for (int q = 0; q < V; ++q) {
 #pragma unroll
-            for (int j = 0; j < kBuArcs; ++j) disc[q] |= hit[q][j];
-            beg[q] += kBuArcs;
-            left[q] = disc[q] ? 0 : left[q] - kBuArcs;
+            for (int j = 0; j < kArcs; ++j) disc[q] |= hit[q][j];
+            beg[q] += kArcs;
+            left[q] = disc[q] ? 0 : left[q] - kArcs;
         }
     }
 #pragma unroll
-    for (int q = 0; q < kBuV; ++q)
+    for (int q = 0; q < V; ++q)
         if (disc[q]) G.h[v[q]] = L + 1;
     front_stage_n(G, disc, v, F, dual, K);
 }
@@ -2717,18 +2731,24 @@ __global__ void __launch_bounds__(kBlock, 1) k_solve(DevGraph G, Job J) {
             }
             Front FR{ncnt, NF, asum, 0x7fffffff, nullptr, s_bfs + (threadIdx.x >> 5) * kWq, 0, 0};
             if (bottom_up) {
-                // pieces of 32 kBuV consecutive vertex ids
-                constexpr int kPiece = 32 * kBuV;
-                const int groups = (n + kPiece - 1) / kPiece;
+                // pieces of 32 V consecutive vertex ids
                 int *const tick = cta_words();
-                int grp = gwarp, nxt;
-                BuPre pre = bu_prefetch(G, (long long)min(grp, groups) * kPiece);
-                for (; grp < groups; grp = nxt) {
-                    const BuPre cur = pre;
-                    nxt = next_item(tick, groups);
-                    pre = bu_prefetch(G, (long long)min(nxt, groups) * kPiece);
-                    bfs_bottom_up_group(G, grp * kPiece, cur, dual, L, FR, ccnt, K);
-                }
+                auto pieces = [&](auto vc, auto ac) {
+                    constexpr int V = decltype(vc)::value, kPiece = 32 * V;
+                    const int groups = (n + kPiece - 1) / kPiece;
+                    int grp = gwarp, nxt;
+                    BuPre<V> pre = bu_prefetch<V>(G, (long long)min(grp, groups) * kPiece);
+                    for (; grp < groups; grp = nxt) {
+                        const BuPre<V> cur = pre;
+                        nxt = next_item(tick, groups);
+                        pre = bu_prefetch<V>(G, (long long)min(nxt, groups) * kPiece);
+                        bfs_bottom_up_group<V, decltype(ac)::value>(G, grp * kPiece, cur, dual, L, FR, ccnt, K);
+                    }
+                };
+                if (G.bu_long || n <= 32LL * kBuV * nwarps)
+                    pieces(std::integral_constant<int, kBuVLong>{}, std::integral_constant<int, kBuArcsLong>{});
+                else
+                    pieces(std::integral_constant<int, kBuV>{}, std::integral_constant<int, kBuArcs>{});
             } else {
                 // groups of gs frontier vertices:
                 // 32, or fewer when the frontier does not fill the grid's warps,
@@ -3645,7 +3665,9 @@ int read_ctl(mf_graph *g, Ctl *out, size_t bytes = sizeof(Ctl)) {
 //             lead back (RMAT-20 static solve with 8192 / 4096 / 2048: 2.33 /
 //             2.28 / 2.23 ms).
 void search_rules(DevGraph &D, bool renumbered) {
-    D.alpha = renumbered || D.A <= 8LL * D.n ? 14 : 3;
+    const bool soon = renumbered || D.A <= 8LL * D.n;   // a parent is found soon
+    D.alpha = soon ? 14 : 3;
+    D.bu_long = !soon;
     D.solo_arcs = renumbered ? 2048 : int(kSoloArcs);
 }
 
