@@ -151,8 +151,9 @@ typedef struct mf_options {
  *               mode the rounds (a vertex made active by a push is served in
  *               the next round of the same iteration); in the data-driven and
  *               push-pull modes the highest generation of the activation
- *               queue (a vertex made active is queued at once with the
- *               pusher's generation + 1) plus one, summed over the phases
+ *               queue (a vertex made active is queued, or served next by the
+ *               same warp, with the pusher's generation + 1) plus one, summed
+ *               over the phases
  *  policy_*     last policy decision: kind 0 = repair, 1 = recompute; the
  *               KERNELCYCLES chosen; 1 if the learned policy fell back
  *  exit_kind    how the loop ended: 0 = a BFS found no active vertex; 1 = the
@@ -278,7 +279,7 @@ int mf_set_stream(mf_graph *g, void *stream);
 /* Device memory the graph holds (bytes). */
 int mf_device_bytes(const mf_graph *g, int64_t *bytes);
 
-/* CTAs of the graph's persistent kernel (options.grid_blocks after clamping). */
+/* CTAs of the graph's persistent kernel (options.grid_blocks after clamping, or as chosen). */
 int mf_grid_blocks(const mf_graph *g, int32_t *blocks);
 
 /* CTAs of the graph's following solve/repair launches (clamped to one full
@@ -339,7 +340,7 @@ void mf_destroy(mf_graph *g);
  * another framework which owns all device memory through its own pool, or a
  * service path where allocations are forbidden after start-up -- and so
  * cannot use mf_create.  Instead of allocating, it works in one static
- * device array of 14,371,072 bytes (about 13.6 MiB) that every GPU which
+ * device array of 14,371,072 bytes (about 13.7 MiB) that every GPU which
  * loads this library holds until the process exits.
  *   n, arcs        vertices (2 .. 131072) and Bi-CSR arcs (0 .. 2097152);
  *                  larger graphs are rejected with MF_EINVAL
@@ -490,10 +491,11 @@ void mf_server_destroy(mf_server *s);
  *          high-degree vertices, 2 bottom-up groups, 3 bottom-up items,
  *          4 a level of a small frontier run by CTA 0 alone (not a barrier),
  *          6 / 5 the barriers before and after such a run; hub
- *          cycles 0 set-up, 1 lowest-neighbour scan, 3 pushes;
+ *          cycles 0 the list of live hubs, 1 lowest-neighbour scan, 3
+ *          pushes, 2 what the cycles' pushes turned active collected;
  *          RemoveInvalidEdges: why the loop went on to another BFS, bits
- *          1 the activation rounds or generations reached their cap (or
- *          the activation queue was full), 2 the hub cycles
+ *          1 the activation rounds reached their cap, or the activation
+ *          queue ran out of its time or was full, 2 the hub cycles
  *          reached theirs, 4 an arc was saturated, 8 a push re-activated a
  *          high-degree vertex (0: it stopped; a height-init record of step 1,
  *          the recount of the deficits, follows)

@@ -1,8 +1,8 @@
 // GB300 (sm_103a) dynamic max-flow: device kernels and the C ABI of mf.h.
 //
 // The whole solve / repair of one graph is ONE persistent cooperative kernel
-// (k_solve): every CTA of one full wave runs the phases below in lock-step,
-// separated by a bounded grid barrier, so the data-dependent loops (BFS
+// (k_solve): its CTAs, one full wave or fewer for a small graph, run the phases
+// below in lock-step, separated by a bounded grid barrier, so the loops (BFS
 // levels, the push/relabel rounds) never return to the host (the paper also
 // decides termination on the device, Sec. 3):
 //
@@ -28,8 +28,10 @@
 // vertex from a contiguous array instead of gathering r[rev[a]].  Every write
 // to r[x] has a matching write to rr[rev[x]].
 //
-// Mutable arrays are read with ld.global.cg (L2, coherent across SMs): the
-// persistent kernel never relies on L1 contents across a grid barrier.
+// Mutable arrays are read with ld.global.cg (L2, coherent across SMs), or
+// through L1 (ld.ca) in phases during which they do not change or an early read
+// is exact; the barrier's acquire drops what L1 holds, so nothing is relied on
+// across one.
 //
 // The phases avoid atomics that the whole grid aims at one address: the
 // items of a phase are dealt to the CTAs by a fixed stride and taken by their
@@ -263,15 +265,6 @@ __device__ __forceinline__ void add_ll(long long *p, long long v) {
     atomicAdd(reinterpret_cast<unsigned long long *>(p), static_cast<unsigned long long>(v));
 }
 
-// Arrival on a counter with acquire-release order at GPU scope: this
-// thread's earlier writes are visible to whoever sees the new count, and the
-// last arrival sees everyone's.
-__device__ __forceinline__ int arrive_acq_rel(int *p) {
-    int old;
-    asm volatile("atom.acq_rel.gpu.global.add.s32 %0, [%1], 1;" : "=r"(old) : "l"(p) : "memory");
-    return old;
-}
-
 __device__ __forceinline__ unsigned ld_acquire(const unsigned *p) {
     unsigned v;
     asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
@@ -315,15 +308,6 @@ __device__ __forceinline__ long long bcast_ld(const long long *p) {
 __device__ __forceinline__ long long warp_sum(long long v) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
-    return v;
-}
-
-__device__ __forceinline__ unsigned long long warp_min(unsigned long long v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        unsigned long long w = __shfl_xor_sync(kFull, v, o);
-        v = w < v ? w : v;
-    }
     return v;
 }
 
@@ -449,11 +433,9 @@ struct ArcRoundBfs {
 };
 
 // Warp-aggregated append of the lanes' flagged values of N slots: one
-// atomicAdd for the whole warp and all slots; positions from cap on go to
-// spill (same positions) instead of buf.  All 32 lanes call.
+// atomicAdd for the whole warp and all slots.  All 32 lanes call.
 template <int N>
-__device__ __forceinline__ void warp_append_n(const bool (&pred)[N], const int (&val)[N], int *cnt, int *buf,
-                                              int cap = 0x7fffffff, int *spill = nullptr) {
+__device__ __forceinline__ void warp_append_n(const bool (&pred)[N], const int (&val)[N], int *cnt, int *buf) {
     const int lane = threadIdx.x & 31;
     const unsigned below = (1u << lane) - 1u;
     unsigned m[N];
@@ -469,10 +451,7 @@ __device__ __forceinline__ void warp_append_n(const bool (&pred)[N], const int (
     base = __shfl_sync(kFull, base, 0);
 #pragma unroll
     for (int j = 0; j < N; ++j) {
-        if (pred[j]) {
-            const int pos = base + __popc(m[j] & below);
-            (pos < cap ? buf : spill)[pos] = val[j];
-        }
+        if (pred[j]) buf[base + __popc(m[j] & below)] = val[j];
         base += __popc(m[j]);
     }
 }
@@ -480,23 +459,18 @@ __device__ __forceinline__ void warp_append_n(const bool (&pred)[N], const int (
 constexpr int kWq = 320;   // staged frontier entries per warp (24 warps: 7680 ints)
 constexpr int kFl = 4;     // staged entries per lane in flight when a stage is published
 
-// The next BFS frontier as one warp writes it.  In grid-wide levels the
-// entries are staged in the warp's kWq ints of shared memory and reach the
-// global queue buf a whole stage at a time (one reservation on cnt); the
-// bookkeeping of the staged vertices (their degrees for the frontier's arc
-// total, their excess for the active lists) is done when the stage is
-// published, for up to 32 kFl vertices at once, instead of inside the arc
-// scan that discovered them: the scan's chain of dependent accesses ends at
-// the height CAS.  front_flush must run before the level's grid barrier.  In
-// CTA 0's small-frontier levels (stage == nullptr) entries go straight to the
-// shared frontier (positions >= cap to spill) with their bookkeeping done at
-// once, and the arc total goes to its counter.
+// The next BFS frontier as one warp writes it.  The entries are staged in the
+// warp's kWq ints of shared memory and reach the global queue buf a whole stage
+// at a time (one reservation on cnt); the bookkeeping of the staged vertices
+// (their degrees for the frontier's arc total, their excess for the active
+// lists) is done when the stage is published, for up to 32 kFl vertices at
+// once, instead of inside the arc scan that discovered them: the scan's chain
+// of dependent accesses ends at the height CAS.  front_flush must run before
+// the level's grid barrier.
 struct Front {
     int *cnt, *buf;
     long long *asum;
-    int cap;
-    int *spill;
-    int *stage;     // this warp's kWq shared ints, or nullptr
+    int *stage;     // this warp's kWq shared ints
     int sn;         // staged entries (warp-uniform)
     long long ds;   // arc total not yet added (warp-uniform)
 };
@@ -552,13 +526,13 @@ __device__ __forceinline__ void front_flush_entries(const DevGraph &G, Front &F,
 
 // Publish what the warp has staged.  All 32 lanes call.
 __device__ __forceinline__ void front_flush(const DevGraph &G, Front &F, bool dual, Counters &K) {
-    if (F.stage && F.sn) front_flush_entries(G, F, dual, K);
+    if (F.sn) front_flush_entries(G, F, dual, K);
     if (F.ds && (threadIdx.x & 31) == 0) add_ll(F.asum, F.ds);
     F.ds = 0;
 }
 
 // Stage the lanes' flagged values of N slots (at most 32 N <= kWq entries).
-// Only for grid-wide levels (F.stage set).  All 32 lanes call.
+// All 32 lanes call.
 template <int N>
 __device__ __forceinline__ void front_stage_n(const DevGraph &G, const bool (&pred)[N], const int (&val)[N],
                                               Front &F, bool dual, Counters &K) {
@@ -579,59 +553,6 @@ __device__ __forceinline__ void front_stage_n(const DevGraph &G, const bool (&pr
         base += __popc(m[j]);
     }
     F.sn = base;
-}
-
-// bfs_discovered for kIlpB slots per lane at once.  Grid-wide levels stage
-// the vertices (bookkeeping when the stage is published); CTA 0's levels do
-// the bookkeeping here, the loads of all slots issued together and each list
-// getting one reservation per warp.
-__device__ __forceinline__ void bfs_discovered_n(const DevGraph &G, const bool (&disc)[kIlpB], const int (&v)[kIlpB],
-                                                 unsigned fwd, bool dual, Front &F, Counters &K) {
-    bool any = false;
-#pragma unroll
-    for (int j = 0; j < kIlpB; ++j) any |= disc[j];
-    if (!__any_sync(kFull, any)) return;
-    if (F.stage) {
-        front_stage_n(G, disc, v, F, dual, K);
-        return;
-    }
-    warp_append_n(disc, v, F.cnt, F.buf, F.cap, F.spill);
-    int deg[kIlpB];
-    long long ev[kIlpB];
-#pragma unroll
-    for (int j = 0; j < kIlpB; ++j) {
-        deg[j] = disc[j] ? __ldg(&G.row[v[j] + 1]) - __ldg(&G.row[v[j]]) : 0;
-        ev[j] = disc[j] ? lcg(&G.e[v[j]]) : 0;
-    }
-    long long ds = 0;
-    bool small[kIlpB], hub[kIlpB];
-#pragma unroll
-    for (int j = 0; j < kIlpB; ++j) {
-        ds += deg[j];
-        K.bfs_verts += disc[j];
-        // a vertex of the pull side (forward search) is active when deficient
-        const bool act = disc[j] && (((fwd >> j) & 1u) ? ev[j] < 0 : ev[j] > 0);
-        hub[j] = act && deg[j] > kHubDeg;
-        small[j] = act && !hub[j];
-    }
-    ds = warp_sum(ds);
-    if ((threadIdx.x & 31) == 0 && ds) add_ll(F.asum, ds);
-    warp_append_n(small, v, &G.ctl->wcnt, G.wl);
-    warp_append_n(hub, v, &G.ctl->hcnt, G.hl);
-}
-
-// Bookkeeping of a vertex v reached at the next level (disc), one slot per
-// lane: as bfs_discovered_n.  All 32 lanes call.
-__device__ __forceinline__ void bfs_discovered(const DevGraph &G, bool disc, int v, bool fwd, bool dual,
-                                               Front &F, Counters &K) {
-    bool d1[kIlpB];
-    int v1[kIlpB];
-#pragma unroll
-    for (int j = 0; j < kIlpB; ++j) {
-        d1[j] = j == 0 && disc;
-        v1[j] = j == 0 ? v : 0;
-    }
-    bfs_discovered_n(G, d1, v1, fwd ? 1u : 0u, dual, F, K);
 }
 
 // Backward BFS step over kIlpB arcs per lane (a[j] of frontier vertex u, head
@@ -657,7 +578,7 @@ __device__ __forceinline__ void bfs_visit_n(const DevGraph &G, const int (&a)[kI
     for (int j = 0; j < kIlpB; ++j) hv[j] = (rin[j] > 0 && v[j] != G.s) ? lheight(&G.h[v[j]]) : -1;
 #pragma unroll
     for (int j = 0; j < kIlpB; ++j) disc[j] = hv[j] == n && atomicCAS(&G.h[v[j]], n, L + 1) == n;
-    bfs_discovered_n(G, disc, v, fwd, dual, F, K);
+    front_stage_n(G, disc, v, F, dual, K);
 }
 
 // Expand up to 32 frontier vertices (one per lane, degree deg starting at
@@ -846,7 +767,9 @@ __device__ __forceinline__ void bfs_bottom_up_item(const DevGraph &G, int2 item,
         if (hit && lane == 0) disc = atomicCAS(&G.h[v], G.n, L + 1) == G.n;
     }
     disc = __shfl_sync(kFull, disc, 0);
-    bfs_discovered(G, disc && lane == 0, v, side == kPartS, dual, F, K);
+    const bool one[1] = {disc && lane == 0};
+    const int val[1] = {v};
+    front_stage_n(G, one, val, F, dual, K);
 }
 
 // ------------------------------------------------------ push / relabel --
@@ -1986,7 +1909,7 @@ __device__ __forceinline__ void bfs_visit_staged(const DevGraph &G, const int *s
     for (int j = 0; j < kIlpB; ++j) hv[j] = (rin[j] > 0 && v[j] != G.s) ? lheight(&G.h[v[j]]) : -1;
 #pragma unroll
     for (int j = 0; j < kIlpB; ++j) disc[j] = hv[j] == n && atomicCAS(&G.h[v[j]], n, L + 1) == n;
-    bfs_discovered_n(G, disc, v, fwd, dual, F, K);
+    front_stage_n(G, disc, v, F, dual, K);
 }
 
 // --------------------------------------- BFS levels of a small frontier --
@@ -2729,7 +2652,7 @@ __global__ void __launch_bounds__(kBlock, 1) k_solve(DevGraph G, Job J) {
                 C->asum[(L + 2) % 3] = 0;
                 if (bottom_up) s_stat[S_BU_LEVELS] += 1;
             }
-            Front FR{ncnt, NF, asum, 0x7fffffff, nullptr, s_bfs + (threadIdx.x >> 5) * kWq, 0, 0};
+            Front FR{ncnt, NF, asum, s_bfs + (threadIdx.x >> 5) * kWq, 0, 0};
             if (bottom_up) {
                 // pieces of 32 V consecutive vertex ids
                 int *const tick = cta_words();
