@@ -79,13 +79,15 @@ enum ExitKind { EXIT_BFS = 0, EXIT_CLEAN = 1, EXIT_NO_CUT_CHANGE = 2, EXIT_PUSH_
 // (more on deep graphs), and the fewest
 // cooperative cycles the high-degree vertices get per iteration (see k_solve).
 constexpr int kMaxRounds = 16;
-// Share of the last BFS's time that the activation queue gets (see k_solve).
-// Measured per batch for 1/2, 1, 2 and for the earlier bound of max(16, BFS
-// levels) generations: 1000-vertex graph 109, 126, 156, 127 us; unit
-// assignment graph of 2^18 + 2^18 vertices 1.43, 1.26, 1.40, 1.60 ms; 1023 x
-// 769 grid 1.37, 1.38, 1.75, 1.52 ms; 2048^2 grid (push-pull) 3.04, 2.69,
-// 2.76, 3.16 ms; RMAT-20 static solve 3.18, 3.20, 3.40, 3.18 ms.
-constexpr unsigned kQueueShareNum = 3, kQueueShareDen = 4;
+// The activation queue gets as long as the last BFS took (see k_solve), and
+// serves at least kMinGen generations.  Measured per batch with a share of 1/2,
+// 3/4, 1, 11/8 of it and 8 generations: unit assignment graph of 2^18 + 2^18
+// vertices 1.28, 1.20, 1.15, 1.17 ms; 1023 x 769 grid 1.05, 0.96, 0.98, 0.95 ms;
+// 2048^2 grid (push-pull) 2.17, 2.07, 1.95, 1.95 ms; RMAT-20 static solve 2.22,
+// 2.18, 2.18, 2.23 ms; 1000-vertex graph 113, 116, 119, 128 us (134 with 12
+// generations; with 6, short chains no longer end inside one phase).  A bound
+// of max(16, BFS levels) generations instead, measured before the search got
+// faster, cost the assignment graph 27 % and the grids 11-17 %.
 constexpr int kMinGen = 8;         // activation generations served whatever the time
 constexpr int kMaxGen = 1 << 30;   // generations fit the queue's 32-bit field
 constexpr int kMinHubCycles = 4;
@@ -1349,6 +1351,13 @@ __device__ __forceinline__ void visit_chain_t(const DevGraph &G, int u, int kc, 
                 left -= min(__shfl_sync(kFull, incl, 31), left);
             }
             rem -= most - left;
+            // a step that moves is the visit's last: moves decided at one height
+            // and issued after more steps found the heads relabelled, and the
+            // steep arcs and deficits that this left cost further iterations
+            // (unit assignment graph 15,386 + 3,000: 3-70 iterations a repair,
+            // 23 ms, now 1, 0.29 ms; 10,187 + 2,673 recompute 3.8 -> 0.33 ms;
+            // 2048^2 grid push-pull +5 %, the rest even)
+            if (left < most) break;
         }
         if (h != hu) {
             if (lane == 0) G.h[u] = h;
@@ -2924,14 +2933,14 @@ const int max_rounds = L > kMaxRounds ? L : kMaxRounds;
                 // the others in shared memory.  One grid barrier at the end.
                 //
                 // How long it goes on: what another global relabel costs is
-                // known, the BFS has just been timed, so the queue gets
-                // kQueueShare of that time and then leaves what is still active
-                // to the next iteration (neither side can then cost much more
+                // known, the BFS has just been timed, so the queue gets as
+                // long and then leaves what is still active to the next
+                // iteration (neither side can then cost much more
                 // than the better choice would have).  Generations below
                 // kMinGen are served in any case, so every iteration makes
                 // progress.
                 const int n0 = cnt;
-                if (threadIdx.x == 0) s_deadline = gtimer() + (s_bfs_end - s_bfs_begin) * kQueueShareNum / kQueueShareDen;
+                if (threadIdx.x == 0) s_deadline = gtimer() + (s_bfs_end - s_bfs_begin);
                 __syncthreads();
                 int ndone = 0;   // entries finished and not yet counted (warp-uniform)
                 int *const tick = cta_words();
@@ -3594,14 +3603,15 @@ void search_rules(DevGraph &D, bool renumbered) {
     D.solo_arcs = renumbered ? 2048 : int(kSoloArcs);
 }
 
-// CTAs of a graph whose options leave the choice: one per 6,144 arcs, at least
+// CTAs of a graph whose options leave the choice: one per 1,536 arcs, at least
 // four, at most one full wave.  A small graph does not fill the chip's warps,
-// and far more warps than it has active vertices serve neighbours at the same
-// time on each other's old heights (measured per batch, full wave / this: 100 x
-// 96 grid 389 / 199 us, 256^2 grid 378 / 359, RMAT-14 push-pull 219 / 197,
-// 1,000-vertex graph 89 / 76, RMAT-12 269 / 262, 8,000-vertex graph 137 / 133;
-// half as many CTAs cost RMAT-14 5 % and a 65,000-vertex graph 20 %).
-int auto_grid(int full, int64_t arcs) { return int(std::max<int64_t>(std::min(full, 4), std::min<int64_t>(full, arcs / 6144))); }
+// and every barrier waits for all CTAs; a solve or a recompute, in which every
+// vertex may be active, sets the line.  Measured per batch with one CTA per
+// 6,144 / 1,536 arcs / full wave: recompute of a 1,507-vertex graph 217 / 210 /
+// 227 us, RMAT-13 push-pull 608 / 477 / 562, unit assignment 6,869 + 4,497 737 /
+// 305 / 332, solve of a 113 x 160 grid 932 / 646 / 632; repairs of the same
+// kinds 79 / 81 / 81, 549 / 393 / 396, 314 / 296 / 319.
+int auto_grid(int full, int64_t arcs) { return int(std::max<int64_t>(std::min(full, 4), std::min<int64_t>(full, arcs / 1536))); }
 
 int launch(mf_graph *g, const Job &job, cudaStream_t st) {
     DevGraph dg = g->dg;
