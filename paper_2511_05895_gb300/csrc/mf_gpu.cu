@@ -3592,15 +3592,17 @@ int read_ctl(mf_graph *g, Ctl *out, size_t bytes = sizeof(Ctl)) {
 //             1.33 / 1.26 / 1.19 / 1.17 ms a batch; 1023 x 769 grid, degree 8,
 //             its searches 256 us with 14, 297 with 4).
 //  solo_arcs  one CTA keeps up with a thin wave of short rows (2048^2 grid: 4
-//             us a level against 7.5 on the whole grid), less so with
-//             the tails of a power-law search, whose rows are long and mostly
-//             lead back (RMAT-20 static solve with 8192 / 4096 / 2048: 2.33 /
-//             2.28 / 2.23 ms).
+//             us a level against 7.5 on the whole grid), less so with long
+//             rows: the tails of a power-law search mostly lead back (RMAT-20
+//             static solve with 8192 / 4096 / 2048: 2.33 / 2.28 / 2.23 ms), and
+//             an assignment graph's levels are written out arc by arc (8192 /
+//             2048: 4,777 + 3,483 vertices 267 / 197 us, 6,551 + 2,539 263 /
+//             215, 2^18 + 2^18 1.14 / 1.13 ms).
 void search_rules(DevGraph &D, bool renumbered) {
     const bool soon = renumbered || D.A <= 8LL * D.n;   // a parent is found soon
     D.alpha = soon ? 14 : 3;
     D.bu_long = !soon;
-    D.solo_arcs = renumbered ? 2048 : int(kSoloArcs);
+    D.solo_arcs = !renumbered && D.A <= 8LL * D.n ? int(kSoloArcs) : 2048;
 }
 
 // CTAs of a graph whose options leave the choice: one per 1,536 arcs, at least
