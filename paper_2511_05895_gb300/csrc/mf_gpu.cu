@@ -885,7 +885,7 @@ __device__ __forceinline__ void aq_push_n(const ActList &AL, const bool (&pred)[
     if (lane == 0) atomicMax(&AL.Q->maxgen, AL.gen);
 }
 
-// Single-thread enqueue of v (as aq_push_n).
+// Single-thread enqueue of v (as aq_push_n; the caller has fenced).
 __device__ __forceinline__ void aq_push_one(const ActList &AL, int v) {
     const int pos = atomicAdd(&AL.Q->tail, 1);
     if (pos < AL.qc) {
@@ -1251,6 +1251,21 @@ __device__ __forceinline__ void visit_chain_t(const DevGraph &G, int u, int kc, 
     const int gen0 = AL.gen;
     int pu = -1;            // the vertex served before, if it may still be active:
     long long pleft = 0;    // its excess after the visit (lane 0)
+    // u goes back to the queue.  A visit that only relabelled has passed no
+    // fence yet, and the next server must read this h(u) and write its own
+    // after it.
+    auto requeue = [&]() {
+        if (!AL.aq) {
+            ++AL.count;
+        } else if (lane == 0) {
+            if (AL.gen >= AL.gen_cap) {
+                atomicExch(&AL.Q->over, 1);
+            } else {
+                fence_acq_rel();
+                aq_push_one(AL, u);
+            }
+        }
+    };
     for (;;) {
         if (lane == 0) ++K.visits;
         const int deg = end - beg;
@@ -1262,14 +1277,7 @@ __device__ __forceinline__ void visit_chain_t(const DevGraph &G, int u, int kc, 
             }
             pu = -1;
             __syncwarp();
-            const bool active = visit_staged_t<PULL>(G, u, beg, end, kc, AL, pt, side, stg, RL, K);
-            if (!active) break;
-            if (!AL.aq) {
-                ++AL.count;
-            } else if (lane == 0) {
-                if (AL.gen >= AL.gen_cap) atomicExch(&AL.Q->over, 1);
-                else aq_push_one(AL, u);
-            }
+            if (visit_staged_t<PULL>(G, u, beg, end, kc, AL, pt, side, stg, RL, K)) requeue();
             break;
         }
         int ra[kIlp], v[kIlp], hv[kIlp], rb[kIlp], d[kIlp];
@@ -1364,13 +1372,7 @@ __device__ __forceinline__ void visit_chain_t(const DevGraph &G, int u, int kc, 
             note_relabel(G, u, RL);
         }
         if (rem == want) {   // nothing moved: u keeps its excess
-            if (h >= G.n || rem <= 0) break;
-            if (!AL.aq) {
-                ++AL.count;
-            } else if (lane == 0) {
-                if (AL.gen >= AL.gen_cap) atomicExch(&AL.Q->over, 1);
-                else aq_push_one(AL, u);
-            }
+            if (h < G.n && rem > 0) requeue();
             break;
         }
         long long old[kIlp];
