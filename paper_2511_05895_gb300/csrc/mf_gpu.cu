@@ -3686,6 +3686,16 @@ int gather_blocks(const mf_graph *g, long long count) {
     return int(std::max<long long>(1, std::min<long long>(g->sms * 8, (count + 255) / 256)));
 }
 
+// Copy host memory to the device before anything that follows on the graph's
+// stream.  (A plain cudaMemcpy runs on the legacy stream and may return with
+// the transfer from pageable memory still under way; a non-blocking stream
+// does not wait for it.)
+int upload(mf_graph *g, void *dst, const void *src, size_t bytes) {
+    MF_CUDA(cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, g->last));
+    MF_CUDA(cudaStreamSynchronize(g->last));
+    return MF_OK;
+}
+
 // Fill ext_row / arc_at of a renumbered graph (and d_arc_at if device memory
 // allows; a caller that finds it null permutes on the host).
 int need_external_arcs(mf_graph *g) {
@@ -3700,10 +3710,11 @@ int need_external_arcs(mf_graph *g) {
     } catch (const std::bad_alloc &) {
         return set_err(MF_ENOMEM, "host allocation");
     }
-    g->d_arc_at = dnew<int>(g, size_t(std::max<int64_t>(g->A, 1)));
-    if (g->d_arc_at && g->A)
-        MF_CUDA(cudaMemcpy(g->d_arc_at, g->arc_at.data(), size_t(g->A) * 4, cudaMemcpyHostToDevice));
-    return MF_OK;
+    int *at = dnew<int>(g, size_t(std::max<int64_t>(g->A, 1)));
+    if (!at) return MF_OK;
+    const int rc = upload(g, at, g->arc_at.data(), size_t(g->A) * 4);
+    if (rc == MF_OK) g->d_arc_at = at;   // (never an index that is not there)
+    return rc;
 }
 
 // Make h the exact BFS heights of the current state (a no-op on the device
@@ -4244,8 +4255,7 @@ int mf_export_state(mf_graph *g, int32_t *r, int64_t *excess, int32_t *height, i
                 }
                 b.resize(at.size());
                 gather_i32(a.data(), at.data(), count, false, b.data());
-                MF_CUDA(cudaMemcpy(dst, b.data(), at.size() * 4, cudaMemcpyHostToDevice));
-                return MF_OK;
+                return upload(g, dst, b.data(), at.size() * 4);
             };
             cudaGetLastError();   // an earlier, unrelated failure of this thread is not these launches'
             int rc = out32(r, g->dg.r, g->arc_at, g->d_arc_at);
