@@ -4366,8 +4366,8 @@ int mf_set_policy(mf_graph *g, int32_t mode, const float *params) {
     if (params) {
         if (!g->params) g->params = dnew<float>(g, mlp::kTotal);
         if (!g->params) return set_err(MF_ENOMEM, "policy parameter allocation failed");
-        MF_CUDA(cudaStreamSynchronize(g->last));
-        MF_CUDA(cudaMemcpy(g->params, params, sizeof(float) * mlp::kTotal, cudaMemcpyHostToDevice));
+        const int rc = upload(g, g->params, params, sizeof(float) * mlp::kTotal);
+        if (rc) return rc;
     }
     g->policy = mode;
     return MF_OK;

@@ -326,7 +326,9 @@ int mf_server_add_graph(mf_server *S, mf_graph *g, int64_t max_batch, int32_t *i
         cudaGetLastError();
         return MF_ECUDA;
     }
-    cudaMemset(sl.d_stage, 0, 16);
+    // (on the slot's stream, which does not wait for the legacy one: the first
+    // word is the batch size that the kernel below reads)
+    cudaMemsetAsync(sl.d_stage, 0, 16, sl.stream);
     // size the graph's batch staging outside any capture with an empty batch
     // (a repair that finds nothing to do), then capture
     int rc = mf_apply_updates_dev(g, sl.d_stage, max_batch, sl.d_stage + 4, sl.d_stage + 4 + max_batch, 0,
