@@ -42,6 +42,8 @@ class Team {
             for (int i = 1; i < n_; ++i) pool_.emplace_back([this] { loop(); });
         } catch (const std::system_error &) {   // fewer threads then
             n_ = int(pool_.size()) + 1;
+        } catch (const std::bad_alloc &) {      // likewise
+            n_ = int(pool_.size()) + 1;
         }
     }
     ~Team() {
@@ -152,14 +154,24 @@ void by_tail(const int64_t *row, int32_t n, int64_t b, int64_t e, F &&fn) {
     }
 }
 
+// A bitmap of n ids, all clear; false without memory for it.
+bool clear_marks(std::vector<uint64_t> &marks, int32_t n) noexcept {
+    try {
+        marks.assign(size_t(n) / 64 + 1, 0);
+        return true;
+    } catch (const std::bad_alloc &) {
+        return false;
+    }
+}
+
 // Sort p[0, d) (values below n) and keep each value once; returns how many.  A
 // row that holds a good part of all ids is sorted by marking them in a bitmap.
-int32_t sort_unique(int32_t *p, int64_t d, int32_t n, std::vector<uint64_t> &marks) {
-    if (std::is_sorted(p, p + d) || d < 4096 || d < n / 32) {
+// (Runs in the team's steps, which must not throw.)
+int32_t sort_unique(int32_t *p, int64_t d, int32_t n, std::vector<uint64_t> &marks) noexcept {
+    if (std::is_sorted(p, p + d) || d < 4096 || d < n / 32 || !clear_marks(marks, n)) {
         if (!std::is_sorted(p, p + d)) std::sort(p, p + d);
         return int32_t(std::unique(p, p + d) - p);
     }
-    marks.assign(size_t(n) / 64 + 1, 0);
     for (int64_t i = 0; i < d; ++i) marks[size_t(p[i]) >> 6] |= uint64_t(1) << (p[i] & 63);
     int32_t *q = p;
     for (size_t w = 0; w < marks.size(); ++w)
