@@ -2520,6 +2520,7 @@ __global__ void __launch_bounds__(kBlock, 1) k_solve(DevGraph G, Job J) {
 
     // ---- device loop (Algorithm 4 while-loop) ----------------------------
     bool early = false;   // stopped when PushRelabel left no active vertex
+    bool limited = false; // stopped by max_iters or the wall-clock limit
     unsigned snext = stamp_base;   // next unused activation stamp
     for (it = 0; !fast; ++it) {
         const int par = (int)(it & 1);
@@ -2777,12 +2778,9 @@ __global__ void __launch_bounds__(kBlock, 1) k_solve(DevGraph G, Job J) {
             }
             break;
         }
-        if (it >= J.max_iters) {
-            if (gtid == 0) atomicOr(&C->status, ST_ITERS);
-            break;
-        }
-        if (lctl(&C->abort_loop)) {   // written before the height-init barrier
-            if (gtid == 0) atomicOr(&C->status, ST_TIME);
+        if (it >= J.max_iters || lctl(&C->abort_loop)) {   // (abort_loop: written before the height-init barrier)
+            if (gtid == 0) atomicOr(&C->status, it >= J.max_iters ? ST_ITERS : ST_TIME);
+            limited = true;
             break;
         }
 
@@ -3205,6 +3203,14 @@ const int max_rounds = L > kMaxRounds ? L : kMaxRounds;
         C->heights_exact = !fast && !early && !pp_ran;
         if (kind == JOB_SOLVE) C->pairs_ok = 1;   // (cleared with the whole block by mf_import_state)
         C->cut_exact = !early;   // the fast path keeps the exact cut it started from
+        C->stamp_base = snext;
+        if (batch_job) C->bseq = seq;
+    }
+    // After a limit the words that decided it stay: no barrier lies between
+    // here and that decision, which other CTAs may yet have to take (one that
+    // read abort_loop cleared would go on and wait for the rest in vain).  The
+    // status is sticky, and mf_solve starts from a cleared block.
+    if (gtid == 0 && !limited) {
         C->ri_moved[0] = C->ri_moved[1] = 0;
         C->phc[0] = C->phc[1] = 0;
         C->rhcnt = 0;
@@ -3215,10 +3221,8 @@ const int max_rounds = L > kMaxRounds ? L : kMaxRounds;
         }
         C->wcnt = C->hcnt = C->rlcnt = 0;
         C->acnt[0] = C->acnt[1] = C->acnt[2] = 0;
-        C->stamp_base = snext;
-        if (batch_job) C->bseq = seq;
         C->hub_live[0] = C->hub_live[1] = C->hub_items[0] = C->hub_items[1] = 0;
-            C->hub_act[0] = C->hub_act[1] = 0;
+        C->hub_act[0] = C->hub_act[1] = 0;
         C->dacc[0] = C->dacc[1] = 0;
         C->batch_err = 0;
         C->abort_loop = 0;
