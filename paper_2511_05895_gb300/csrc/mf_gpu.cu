@@ -3611,15 +3611,24 @@ void search_rules(DevGraph &D, bool renumbered) {
     D.solo_arcs = !renumbered && D.A <= 8LL * D.n ? int(kSoloArcs) : 2048;
 }
 
-// CTAs of a graph whose options leave the choice: one per 1,536 arcs, at least
-// four, at most one full wave.  A small graph does not fill the chip's warps,
-// and every barrier waits for all CTAs; a solve or a recompute, in which every
-// vertex may be active, sets the line.  Measured per batch with one CTA per
-// 6,144 / 1,536 arcs / full wave: recompute of a 1,507-vertex graph 217 / 210 /
-// 227 us, RMAT-13 push-pull 608 / 477 / 562, unit assignment 6,869 + 4,497 737 /
-// 305 / 332, solve of a 113 x 160 grid 932 / 646 / 632; repairs of the same
-// kinds 79 / 81 / 81, 549 / 393 / 396, 314 / 296 / 319.
-int auto_grid(int full, int64_t arcs) { return int(std::max<int64_t>(std::min(full, 4), std::min<int64_t>(full, arcs / 1536))); }
+// CTAs of a graph whose options leave the choice: one per 1,536 arcs or per
+// 4,096 vertices, whichever are more, at least four, at most one full wave.  A
+// small graph does not fill the chip's warps, and every barrier waits for all
+// CTAs.  For the arcs, a solve or a recompute, in which every vertex may be
+// active, sets the line.  Measured per batch with one CTA per 6,144 / 1,536 arcs /
+// full wave: recompute of a 1,507-vertex graph 217 / 210 / 227 us, RMAT-13
+// push-pull 608 / 477 / 562, unit assignment 6,869 + 4,497 737 / 305 / 332, solve
+// of a 113 x 160 grid 932 / 646 / 632; repairs of the same kinds 79 / 81 / 81,
+// 549 / 393 / 396, 314 / 296 / 319.  The vertices count where arcs are few: the
+// sweeps over all vertices (heights, cut sides, final sums) then set the time.
+// Per batch, data-driven / push-pull, of 2^20 vertices and 5,000 edges with 5,
+// 38, 76, 152 CTAs: 182 / 469, 105 / 167, 95 / 146, 91 / 137 us; of 200,000 and
+// 20,000 with 4, 25, 38, 152: 93 / 172, 88 / 115, 83 / 109, 80 / 105; of 50,000
+// and 10,000 the same from 10 on.
+int auto_grid(int full, int64_t arcs, int32_t n) {
+    const int64_t want = std::max(arcs / 1536, int64_t(n) / 4096);
+    return int(std::max<int64_t>(std::min(full, 4), std::min<int64_t>(full, want)));
+}
 
 int launch(mf_graph *g, const Job &job, cudaStream_t st) {
     DevGraph dg = g->dg;
@@ -3851,7 +3860,7 @@ int mf_create(int32_t n, int64_t m, const int64_t *row_ptr, const int32_t *col, 
     if (per_sm < 1)
         return fail(MF_ECUDA, "occupancy query failed");
     g->max_grid = per_sm * g->sms;
-    g->grid = g->opt.grid_blocks > 0 ? std::min(g->max_grid, int(g->opt.grid_blocks)) : auto_grid(g->max_grid, H.arcs);
+    g->grid = g->opt.grid_blocks > 0 ? std::min(g->max_grid, int(g->opt.grid_blocks)) : auto_grid(g->max_grid, H.arcs, n);
 
     g->n = n; g->m = m; g->A = H.arcs; g->s = s; g->t = t;
     g->cap_limit = H.cap_limit;
@@ -4525,7 +4534,7 @@ int mf_solve_bicsr_noalloc(int32_t n, int64_t arcs, const int32_t *row, const in
     j.time_limit_ns = 60ull * 1000ull * 1000ull * 1000ull;
     void *args[] = {&D, &j};
     cudaError_t e =
-        cudaLaunchCooperativeKernel((const void *)k_solve<false>, dim3(auto_grid(ND.grid, arcs)), dim3(kBlock), args,
+        cudaLaunchCooperativeKernel((const void *)k_solve<false>, dim3(auto_grid(ND.grid, arcs, n)), dim3(kBlock), args,
                                     kDynSmem, st);
     if (e != cudaSuccess) {
         cudaGetLastError();
