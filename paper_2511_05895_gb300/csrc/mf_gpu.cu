@@ -3748,10 +3748,15 @@ int status_to_code(mf_graph *g, const Ctl &c) {
         g->solved = false;
         static const char *kinds[] = {"?", "list entry out of range", "excess differs from the net inflow",
                                       "residual pair or mirror inconsistent"};
-        const long long kind = c.chk_where >> 40, where = c.chk_where & 0xffffffffffll;
-        const bool vertex = (kind == 1 || kind == 2) && where >= 0 && where < g->n && !g->ord.empty();
+        const long long kind = c.chk_where >> 40;
+        long long where = c.chk_where & 0xffffffffffll;
+        // a renumbered graph's vertex or arc by the caller's numbers
+        if (!g->ord.empty() && kind == 3 && where < g->A && need_external_arcs(g) == MF_OK)
+            where = std::find(g->arc_at.begin(), g->arc_at.end(), int32_t(where)) - g->arc_at.begin();
+        else if (!g->ord.empty() && (kind == 1 || kind == 2) && where < g->n)
+            where = g->ord[size_t(where)];
         return set_err(MF_ECHECK, std::string("debug check failed: ") + kinds[kind >= 1 && kind <= 3 ? kind : 0] +
-                                      " (index " + std::to_string(vertex ? (long long)g->ord[size_t(where)] : where) + ")");
+                                      " (index " + std::to_string(where) + ")");
     }
     if (c.status & ST_STICKY) {
         g->solved = false;
