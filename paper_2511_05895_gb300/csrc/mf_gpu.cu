@@ -3472,7 +3472,7 @@ struct mf_graph {
     std::vector<int32_t> ord, inv;   // input id of each vertex, and the inverse (empty: not renumbered)
     int *d_inv = nullptr;            // inv on the device
     std::vector<int32_t> ext_row, arc_at;   // the arcs in the input's order, made when first asked for
-    int *d_arc_at = nullptr;                // and on the device, where it fits
+    int *d_arc_at = nullptr;                // and on the device, for exports to device buffers, where it fits
 };
 
 namespace {
@@ -3709,8 +3709,7 @@ int upload(mf_graph *g, void *dst, const void *src, size_t bytes) {
     return MF_OK;
 }
 
-// Fill ext_row / arc_at of a renumbered graph (and d_arc_at if device memory
-// allows; a caller that finds it null permutes on the host).
+// Fill ext_row / arc_at of a renumbered graph.
 int need_external_arcs(mf_graph *g) {
     if (g->ord.empty() || !g->ext_row.empty()) return MF_OK;
     try {
@@ -3723,10 +3722,22 @@ int need_external_arcs(mf_graph *g) {
     } catch (const std::bad_alloc &) {
         return set_err(MF_ENOMEM, "host allocation");
     }
-    int *at = dnew<int>(g, size_t(std::max<int64_t>(g->A, 1)));
+    return MF_OK;
+}
+
+// arc_at on the device too, where it fits (a caller that finds d_arc_at null
+// permutes on the host).
+int need_arc_index(mf_graph *g) {
+    if (g->d_arc_at || g->A == 0) return MF_OK;
+    int *at = dnew<int>(g, size_t(g->A));
     if (!at) return MF_OK;
     const int rc = upload(g, at, g->arc_at.data(), size_t(g->A) * 4);
-    if (rc == MF_OK) g->d_arc_at = at;   // (never an index that is not there)
+    if (rc == MF_OK) {
+        g->d_arc_at = at;   // (never an index that is not there)
+    } else {
+        dforget(g, at);
+        dfree(g, at);
+    }
     return rc;
 }
 
@@ -4252,6 +4263,7 @@ int mf_export_state(mf_graph *g, int32_t *r, int64_t *excess, int32_t *height, i
         // buffers, else (host buffers, or no room for arc_at) on the host
         if (r) {
             int rc = need_external_arcs(g);
+            if (rc == MF_OK && (flags & MF_DEVICE_PTRS)) rc = need_arc_index(g);
             if (rc) return rc;
         }
         try {
