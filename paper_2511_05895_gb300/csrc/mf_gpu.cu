@@ -89,7 +89,6 @@ constexpr int kMaxRounds = 16;
 // of max(16, BFS levels) generations instead, measured before the search got
 // faster, cost the assignment graph 27 % and the grids 11-17 %.
 constexpr int kMinGen = 8;         // activation generations served whatever the time
-constexpr int kMaxGen = 1 << 30;   // generations fit the queue's 32-bit field
 constexpr int kMinHubCycles = 4;
 // The push-pull instance gives its hubs more cycles per pass: there a hub
 // left active costs another dual search of the whole graph (measured on
@@ -837,7 +836,8 @@ struct ActList {
     int *hcnt, *hlist;          // the next pass's hub list, its size and its stamp
     unsigned hstamp;
     unsigned long long *aq;     // activation queue, or nullptr: count only
-    int qc, gen, gen_cap;       // its capacity; generation of what is filed, and the first one not queued
+    int qc, gen;                // its capacity; generation of what is filed (a phase has time for
+                                // some millions at most: they fit the slot's upper half)
     const volatile unsigned long long *deadline;   // shared: when the phase ends (globaltimer)
     Ctl::Queue *Q;
     int count;                  // filed without a queue (warp-uniform)
@@ -912,8 +912,7 @@ __device__ __forceinline__ void file_hubs(const DevGraph &G, bool (&add_hub)[N],
 }
 
 // File the vertices that moves turned active (add: worklist vertices; add_hub:
-// hubs; neither s nor t).  Past the generation cap a worklist vertex is left
-// active, unqueued, and the phase is flagged.  All 32 lanes call.
+// hubs; neither s nor t).  All 32 lanes call.
 template <int N>
 __device__ __forceinline__ void file_activations(const DevGraph &G, bool (&add)[N], bool (&add_hub)[N],
                                                  const int (&v)[N], ActList &AL) {
@@ -925,10 +924,6 @@ __device__ __forceinline__ void file_activations(const DevGraph &G, bool (&add)[
     if (!AL.aq) {
 #pragma unroll
         for (int j = 0; j < N; ++j) AL.count += __popc(__ballot_sync(kFull, add[j]));
-        return;
-    }
-    if (AL.gen >= AL.gen_cap) {
-        if ((threadIdx.x & 31) == 0) atomicExch(&AL.Q->over, 1);
         return;
     }
     __syncwarp();
@@ -959,18 +954,16 @@ __device__ __forceinline__ void note_relabel(const DevGraph &G, int u, Relabelle
 }
 
 // One round of a warp's arc scan: lane i holds arcs a0 + 32 j + i (j < kIlp)
-// with their residual (0 past `end`), head and the head's height, and, when
-// the round is one to push along (REV), the reverse arcs of its residual
-// arcs.  All loads of the round are issued before any is used; the reverse
-// arcs load beside the heights.
+// with their residual (0 past `end`), head and the head's height.  All loads of
+// one kind are issued before any is used.
 struct ArcRound {
-    int ra[kIlp], v[kIlp], hv[kIlp], rb[kIlp];
+    int ra[kIlp], v[kIlp], hv[kIlp];
 };
 
 // The residual is that of the arc u -> head (push) or head -> u (pull, the
 // mirror rr).  With a partition array pt, an arc to a vertex of another part
 // counts as absent (push-pull: each side works on its own vertices only).
-template <bool PULL, bool REV>
+template <bool PULL>
 __device__ __forceinline__ void load_round_t(const DevGraph &G, int a0, int end, ArcRound &R,
                                              const unsigned char *pt, unsigned char side) {
     const int lane = threadIdx.x & 31;
@@ -987,10 +980,7 @@ __device__ __forceinline__ void load_round_t(const DevGraph &G, int a0, int end,
             if (R.ra[j] > 0 && pt[R.v[j]] != side) R.ra[j] = 0;
     }
 #pragma unroll
-    for (int j = 0; j < kIlp; ++j) {
-        R.hv[j] = R.ra[j] > 0 ? lheight(&G.h[R.v[j]]) : 0;
-        R.rb[j] = (REV && R.ra[j] > 0) ? __ldg(&G.rev[a0 + 32 * j + lane]) : 0;
-    }
+    for (int j = 0; j < kIlp; ++j) R.hv[j] = R.ra[j] > 0 ? lheight(&G.h[R.v[j]]) : 0;
 }
 
 __device__ __forceinline__ int round_arcs(int a0, int end) {
@@ -1092,8 +1082,10 @@ __device__ __forceinline__ unsigned stage_heights(const DevGraph &G, const int *
 }
 
 // The moves of N slots per lane (d[j] > 0: d[j] units along arc a[j] of u,
-// reverse b[j], head v[j]) and the filing of the vertices they turn active,
-// as move_round.  Returns this lane's total moved.  All 32 lanes call.
+// reverse b[j], head v[j]) and the filing of the vertices they turn active: a
+// push that raised e(v) above 0 (a pull that lowered it below 0) makes v active.
+// The heads' degrees load beside the move atomics.  Returns this lane's total
+// moved.  All 32 lanes call.
 constexpr int kMv = 4;   // moves in flight per lane
 template <bool PULL, int N>
 __device__ __forceinline__ long long move_batch(const DevGraph &G, const int (&a)[N], const int (&b)[N],
@@ -1225,13 +1217,15 @@ __device__ __forceinline__ bool visit_staged_t(const DevGraph &G, int u, int beg
     return active && h < G.n;
 }
 
-// Serve the active vertex u of generation AL.gen - 1 by one warp: up to kc
-// steps of Algorithm 2 (as visit_staged_t) on the residuals and heights of
-// one load of its arcs (<= 32 kIlp; larger vertices: visit_staged_t), which
-// the steps share -- heights only rise and residuals out of u only grow
-// meanwhile, so the moves stay within the residuals, and an arc that a stale
-// height made steep is RemoveInvalidEdges' to saturate, as with Alg. 2's own
-// unlocked reads.  All moves are issued together at the end.
+// Serve the active vertex u of generation AL.gen - 1 by one warp (its arcs in
+// registers, <= 32 kIlp; larger vertices: visit_staged_t): steps of Algorithm 2
+// (as visit_staged_t), each on the residuals and heights as they are then, until
+// one has moved something, kc at most.  So KERNELCYCLES bounds the relabels of a
+// visit here, and the pushes that further steps would make are left to u's next
+// visit.  Heights only rise and residuals out of u only grow meanwhile, so the
+// moves stay within the residuals, and an arc that a stale height made steep is
+// RemoveInvalidEdges' to saturate, as with Alg. 2's own unlocked reads.  All moves
+// are issued together at the end.
 //
 // Then the warp goes on with one of the vertices its moves turned active,
 // whose arc range has come back beside the move atomics, and only the others
@@ -1258,12 +1252,8 @@ __device__ __forceinline__ void visit_chain_t(const DevGraph &G, int u, int kc, 
         if (!AL.aq) {
             ++AL.count;
         } else if (lane == 0) {
-            if (AL.gen >= AL.gen_cap) {
-                atomicExch(&AL.Q->over, 1);
-            } else {
-                fence_acq_rel();
-                aq_push_one(AL, u);
-            }
+            fence_acq_rel();
+            aq_push_one(AL, u);
         }
     };
     for (;;) {
@@ -1414,7 +1404,7 @@ __device__ __forceinline__ void visit_chain_t(const DevGraph &G, int u, int kc, 
             AL.count += __shfl_sync(kFull, maybe && (PULL ? pleft < 0 : pleft > 0), 0);
             break;
         }
-        if (AL.gen >= kMinGen && (AL.gen >= AL.gen_cap || __any_sync(kFull, gtimer() > *AL.deadline))) {
+        if (AL.gen >= kMinGen && __any_sync(kFull, gtimer() > *AL.deadline)) {
             const bool self = __shfl_sync(kFull, maybe && (PULL ? pleft < 0 : pleft > 0), 0);
             if ((tot || self) && lane == 0) atomicExch(&AL.Q->over, 1);
             break;
@@ -1469,7 +1459,7 @@ __device__ __forceinline__ long long remove_invalid_range_t(const DevGraph &G, i
     long long moved = 0;
     for (int b0 = a0; b0 < a1; b0 += 32 * kIlp) {
         ArcRound R;
-        load_round_t<PULL, false>(G, b0, a1, R, pt, side);
+        load_round_t<PULL>(G, b0, a1, R, pt, side);
         K.ri_arcs += round_arcs(b0, a1);
 #pragma unroll
         for (int j = 0; j < kIlp; ++j) {
@@ -2209,11 +2199,10 @@ __global__ void __launch_bounds__(kBlock, 1) k_solve(DevGraph G, Job J) {
     const int nwarps = (int)(gthreads >> 5);
     const int n = G.n, s = G.s, t = G.t;
     Counters K;
-    // BFS frontiers in shared memory: CTA 0's small-frontier levels, and the
-    // warps' staged entries in grid-wide levels (barriers keep them apart)
     // dynamic shared memory (kDynSmem bytes), used by one kind of phase at a
-    // time (grid barriers keep them apart): the BFS frontiers at its start,
-    // the warps' arc stages of PushRelabel
+    // time (grid barriers keep them apart): the BFS frontiers (CTA 0's small
+    // ones, or the warps' staged entries) at its start, the warps' arc stages of
+    // PushRelabel
     extern __shared__ __align__(16) int s_dyn[];
     int *const s_bfs = s_dyn;
     int *const stg = s_dyn + (threadIdx.x >> 5) * kStgWarp;
@@ -2786,12 +2775,13 @@ __global__ void __launch_bounds__(kBlock, 1) k_solve(DevGraph G, Job J) {
 
         // PushRelabel (Alg. 2), in passes.  A pass serves the high-degree
         // vertices of its hub list together, in kPrChunk-arc items over the
-        // whole grid (cooperative cycles), and then the worklist, one warp per
-        // vertex, in activation rounds: a vertex that a push turns active joins
-        // the list of the next round instead of waiting for the next BFS.
-        // Cycles and rounds are separated by grid barriers, so no vertex is
-        // ever processed by two warps at once.  High-degree vertices that a
-        // pass turns active again form the hub list of the next pass.
+        // whole grid (cooperative cycles separated by grid barriers), and then
+        // the worklist, one warp per vertex: from the activation queue in one
+        // phase, where the sign of the excess says who holds a vertex (ActList),
+        // or, topology-driven, in rounds separated by grid barriers, each of
+        // which serves an active vertex once.  So no vertex is ever processed by
+        // two warps at once.  High-degree vertices that a pass turns active
+        // again form the hub list of the next pass.
         const unsigned rstamp_it = snext++;   // relabel-list stamp of this iteration
         Relabelled RL;
         RL.stamp = rstamp_it;
@@ -2802,12 +2792,12 @@ __global__ void __launch_bounds__(kBlock, 1) k_solve(DevGraph G, Job J) {
         bool rounds_clean = true;   // the last activation round left no active vertex
         bool hubs_clean = true;     // the last hub cycle left no hub active
         int pend = 0;               // hubs that the last pass turned active
-        // Rounds per pass (topology-driven mode): kMaxRounds, and past that, while the list holds at
-        // most one vertex per warp, as many as the BFS just run had levels --
-        // such a round costs about what a BFS level costs, so on deep graphs
-        // (grids) finishing a few active vertices by rounds is cheaper than
-        // another global relabel.
-const int max_rounds = L > kMaxRounds ? L : kMaxRounds;
+        // Rounds per pass (topology-driven mode): kMaxRounds, and past that,
+        // while at most one vertex per warp is active, as many as the BFS just
+        // run had levels -- such a round costs about what a BFS level costs, so
+        // on deep graphs (grids) finishing a few active vertices by rounds is
+        // cheaper than another global relabel.
+        const int max_rounds = L > kMaxRounds ? L : kMaxRounds;
         int hub_no = 0;             // hub cycles' lists built in this iteration
         for (int pass = 0; pass < (PP ? kMaxPassesPP : kMaxPasses); ++pass) {
             const int *HL = (pass & 1) ? G.hl2 : G.hl;
@@ -2829,7 +2819,7 @@ const int max_rounds = L > kMaxRounds ? L : kMaxRounds;
             // the data-driven and push-pull modes run PushRelabel from the
             // activation queue; the topology-driven mode in rounds
             const bool qmode = jmode != MF_MODE_TOPOLOGY && G.aq != nullptr;
-            ActList AL{pcnt, (pass & 1) ? G.hl : G.hl2, hstamp, qmode ? G.aq : nullptr, G.qc, 0, kMaxGen, &s_deadline,
+            ActList AL{pcnt, (pass & 1) ? G.hl : G.hl2, hstamp, qmode ? G.aq : nullptr, G.qc, 0, &s_deadline,
                        &C->q[pass & 1], 0, nhp > kDeferHubs};
             bool pass_hubs_clean = true;
             if (nhp > 0) {
@@ -2929,7 +2919,7 @@ const int max_rounds = L > kMaxRounds ? L : kMaxRounds;
                 // free warps.  The phase ends when every queued entry has been
                 // processed: a warp counts what it has finished when it finds
                 // no entry ready, and the one that makes the counts equal
-                // raises aq_fin.  One warp per CTA polls that word and tells
+                // raises fin.  One warp per CTA polls that word and tells
                 // the others in shared memory.  One grid barrier at the end.
                 //
                 // How long it goes on: what another global relabel costs is
