@@ -91,9 +91,13 @@ extern "C" {
 typedef struct mf_graph mf_graph;
 
 /* Options.  Initialise with mf_options_default() and override fields.
- *  kernel_cycles  KERNELCYCLES of Algorithm 2: push/relabel steps per active
- *                 vertex between two global relabels.  0 = max(1, round(m/n)),
- *                 the average degree used in Sec. 6.1.
+ *  kernel_cycles  KERNELCYCLES of Algorithm 2: the most push/relabel steps of
+ *                 one visit to an active vertex; a vertex still active after
+ *                 them is visited again.  (A vertex of up to 128 arcs also
+ *                 ends its visit with the first step that pushes, so there
+ *                 only relabels count towards it; one of more than 512 gets
+ *                 at least 4 cycles a pass, 8 in push-pull.)
+ *                 0 = max(1, round(m/n)), the average degree used in Sec. 6.1.
  *  mode           MF_MODE_DATA_DRIVEN (default), MF_MODE_TOPOLOGY or
  *                 MF_MODE_PUSH_PULL.
  *  max_iters      cap on loop iterations (one BFS + PushRelabel +
@@ -276,7 +280,10 @@ int mf_flow_value_async(mf_graph *g, int64_t *result, void *stream);
  * destroying a stream the graph last ran on. */
 int mf_set_stream(mf_graph *g, void *stream);
 
-/* Device memory the graph holds (bytes). */
+/* Device memory the graph holds now (bytes).  Besides what mf_create took:
+ * batch staging as large as the largest batch so far, a trace buffer, policy
+ * parameters, and, from the first mf_export_state of residuals to device
+ * buffers on, 4 bytes per arc if the graph is renumbered (see there). */
 int mf_device_bytes(const mf_graph *g, int64_t *bytes);
 
 /* CTAs of the graph's persistent kernel (options.grid_blocks after clamping, or as chosen). */
@@ -317,7 +324,11 @@ int mf_export_graph(mf_graph *g, int64_t *arc_row, int32_t *head, int32_t *rev, 
 /* Checkpoint: copy residuals r [arcs] int32, excess [n] int64 and heights
  * [n] int32 out (host or device buffers per flags; any may be NULL).  The
  * heights are the exact BFS heights (recomputed first when needed, as for
- * mf_min_cut).  Synchronises. */
+ * mf_min_cut).  Synchronises.
+ * A graph whose degrees are very uneven is kept in vertex ids of the library's
+ * own; what is exported is in the caller's.  The first export or import of
+ * such a graph works out the arcs' order on the host (8 bytes of host memory
+ * per arc while it does, 4 from then on), and later ones permute by it. */
 int mf_export_state(mf_graph *g, int32_t *r, int64_t *excess, int32_t *height, int32_t flags);
 
 /* Resume: load residuals, excess and heights previously exported from a

@@ -3583,10 +3583,15 @@ int read_ctl(mf_graph *g, Ctl *out, size_t bytes = sizeof(Ctl)) {
 // Where the search changes hands (see k_solve).
 //  alpha      bottom-up pays early where a vertex finds a parent soon: in a
 //             renumbered graph, whose rows begin with the likely parents, and
-//             where rows are short.  Long rows of alike heads are mostly read
-//             whole (unit assignment graph of degree 18, alpha 14 / 8 / 4 / 2:
-//             1.33 / 1.26 / 1.19 / 1.17 ms a batch; 1023 x 769 grid, degree 8,
-//             its searches 256 us with 14, 297 with 4).
+//             where rows are short (1023 x 769 grid, degree 8, its searches 256
+//             us with 14, 297 with 4).  Long rows of alike heads are mostly read
+//             whole, and anything below 14 does (unit assignment graph of degree
+//             18, alpha 14 / 8 / 4 / 3 / 2: 1.33 / 1.10 / 1.21 / 1.14 / 1.17 ms a
+//             batch, runs of one value 5 % apart).  On grids of longer rows it
+//             does not matter: 6-connected 128^3 (10 arcs a vertex, push-pull)
+//             2.45 / 2.30 / 2.53 / 2.40 / 2.35, 8-connected 512^2 (12) 2.92 / 3.04 /
+//             3.11 / 2.94 / 2.95, 26-connected 64^3 (30, push-pull) 2.45 / 2.32 /
+//             2.45 / 2.68 / 2.49.
 //  solo_arcs  one CTA keeps up with a thin wave of short rows (2048^2 grid: 4
 //             us a level against 7.5 on the whole grid), less so with long
 //             rows: the tails of a power-law search mostly lead back (RMAT-20
@@ -3604,14 +3609,14 @@ void search_rules(DevGraph &D, bool renumbered) {
 // CTAs of a graph whose options leave the choice: one per 1,536 arcs or per
 // 4,096 vertices, whichever are more, at least four, at most one full wave.  A
 // small graph does not fill the chip's warps, and every barrier waits for all
-// CTAs.  For the arcs, a solve or a recompute, in which every vertex may be
-// active, sets the line.  Measured per batch with one CTA per 6,144 / 1,536 arcs /
-// full wave: recompute of a 1,507-vertex graph 217 / 210 / 227 us, RMAT-13
-// push-pull 608 / 477 / 562, unit assignment 6,869 + 4,497 737 / 305 / 332, solve
-// of a 113 x 160 grid 932 / 646 / 632; repairs of the same kinds 79 / 81 / 81,
-// 549 / 393 / 396, 314 / 296 / 319.  The vertices count where arcs are few: the
-// sweeps over all vertices (heights, cut sides, final sums) then set the time.
-// Per batch, data-driven / push-pull, of 2^20 vertices and 5,000 edges with 5,
+// CTAs.  (A server's grids for small batches are shares of this, down to one.)
+// For the arcs, a solve or a recompute, in which every vertex may be active, sets
+// the line.  Measured per batch with one CTA per 6,144 / 1,536 arcs / full wave:
+// recompute of a 1,507-vertex graph 217 / 210 / 227 us, RMAT-13 push-pull 608 /
+// 477 / 562, unit assignment 6,869 + 4,497 737 / 305 / 332, solve of a 113 x 160
+// grid 932 / 646 / 632; repairs of the same kinds 79 / 81 / 81, 549 / 393 / 396,
+// 314 / 296 / 319.  The vertices count where arcs are few: the sweeps over all
+// vertices (heights, cut sides, final sums) then set the time.  Per batch, data-driven / push-pull, of 2^20 vertices and 5,000 edges with 5,
 // 38, 76, 152 CTAs: 182 / 469, 105 / 167, 95 / 146, 91 / 137 us; of 200,000 and
 // 20,000 with 4, 25, 38, 152: 93 / 172, 88 / 115, 83 / 109, 80 / 105; of 50,000
 // and 10,000 the same from 10 on.

@@ -65,7 +65,10 @@ constexpr int kGridClasses = 3;
 // a small graph is latency bound: a smaller grid costs it little and frees
 // SMs), but never smaller than the graph's size allows (max_class): every
 // repair runs at least one BFS over the whole graph, so on a graph of 2^21
-// vertices or more a smaller grid only makes it slower.
+// vertices or more a smaller grid only makes it slower.  The shares hold for the
+// few CTAs of a small graph too: with 10 / 5 / 2 CTAs 24 graphs of 1,000 vertices
+// take 18 us a request of 1,500 entries (20 of 5,000), with 10 for every class 24
+// (26), and a request alone takes the same (317-322 us).
 int grid_class(int64_t k, int32_t flags, int max_class) {
     if ((flags & MF_RECOMPUTE) || k > 20000) return 0;
     const int c = k > 2000 ? 1 : 2;
