@@ -427,7 +427,7 @@ void gather_i32(const int32_t *src, const int32_t *at, int64_t count, bool scatt
     Team team(count);
     team.each(count, [&](int64_t b, int64_t e) {
         if (scatter)
-            for (int64_t i = b; i < e; ++i) dst[at[i]] = src[i];
+            for (int64_t i = b; i < e; ++i) dst[at[i]] = src ? src[i] : int32_t(i);
         else
             for (int64_t i = b; i < e; ++i) dst[i] = src[at[i]];
     });

@@ -3461,7 +3461,7 @@ struct mf_graph {
     // input's (s, t above too)
     std::vector<int32_t> ord, inv;   // input id of each vertex, and the inverse (empty: not renumbered)
     int *d_inv = nullptr;            // inv on the device
-    std::vector<int32_t> ext_row, arc_at;   // the arcs in the input's order, made when first asked for
+    HostArray<int32_t> ext_row, arc_at;   // the arcs in the input's order, made when first asked for
     int *d_arc_at = nullptr;                // and on the device, for exports to device buffers, where it fits
 };
 
@@ -3708,12 +3708,12 @@ int upload(mf_graph *g, void *dst, const void *src, size_t bytes) {
 int need_external_arcs(mf_graph *g) {
     if (g->ord.empty() || !g->ext_row.empty()) return MF_OK;
     try {
-        std::vector<int32_t> row(size_t(g->n) + 1), head(size_t(g->A)), ext_row(size_t(g->n) + 1), at(size_t(g->A));
+        HostArray<int32_t> row(size_t(g->n) + 1), head(size_t(g->A)), ext_row(size_t(g->n) + 1), at(size_t(g->A));
         MF_CUDA(cudaMemcpy(row.data(), g->dg.row, row.size() * 4, cudaMemcpyDeviceToHost));
         if (g->A) MF_CUDA(cudaMemcpy(head.data(), g->dg.head, head.size() * 4, cudaMemcpyDeviceToHost));
         external_arcs(g->n, row.data(), head.data(), g->ord.data(), g->inv.data(), ext_row.data(), at.data());
-        g->ext_row.swap(ext_row);
-        g->arc_at.swap(at);
+        g->ext_row = std::move(ext_row);
+        g->arc_at = std::move(at);
     } catch (const std::bad_alloc &) {
         return set_err(MF_ENOMEM, "host allocation");
     }
@@ -4209,7 +4209,7 @@ int mf_export_graph(mf_graph *g, int64_t *arc_row, int32_t *head, int32_t *rev, 
         if (rc) return rc;
         if (arc_row) for (size_t i = 0; i < g->ext_row.size(); ++i) arc_row[i] = g->ext_row[i];
         try {
-            std::vector<int32_t> tmp(size_t(g->A));
+            HostArray<int32_t> tmp(static_cast<size_t>(g->A));
             if (cap && g->A) {
                 MF_CUDA(cudaMemcpy(tmp.data(), g->dg.cap, tmp.size() * 4, cudaMemcpyDeviceToHost));
                 gather_i32(tmp.data(), g->arc_at.data(), g->A, false, cap);
@@ -4217,17 +4217,15 @@ int mf_export_graph(mf_graph *g, int64_t *arc_row, int32_t *head, int32_t *rev, 
             if (head && g->A) {
                 MF_CUDA(cudaMemcpy(tmp.data(), g->dg.head, tmp.size() * 4, cudaMemcpyDeviceToHost));
                 gather_i32(tmp.data(), g->arc_at.data(), g->A, false, head);
-                gather_i32(g->ord.data(), head, g->A, false, tmp.data());
-                std::copy(tmp.begin(), tmp.end(), head);
+                gather_i32(g->ord.data(), head, g->A, false, head);
             }
             if (rev && g->A) {
                 // the reverse arc's place in the input's order
-                std::vector<int32_t> place(size_t(g->A)), iota(size_t(g->A));
-                for (size_t i = 0; i < iota.size(); ++i) iota[i] = int32_t(i);
-                gather_i32(iota.data(), g->arc_at.data(), g->A, true, place.data());
+                HostArray<int32_t> place(static_cast<size_t>(g->A));
+                gather_i32(nullptr, g->arc_at.data(), g->A, true, place.data());
                 MF_CUDA(cudaMemcpy(tmp.data(), g->dg.rev, tmp.size() * 4, cudaMemcpyDeviceToHost));
-                gather_i32(tmp.data(), g->arc_at.data(), g->A, false, iota.data());
-                gather_i32(place.data(), iota.data(), g->A, false, rev);
+                gather_i32(tmp.data(), g->arc_at.data(), g->A, false, rev);
+                gather_i32(place.data(), rev, g->A, false, rev);
             }
         } catch (const std::bad_alloc &) {
             return set_err(MF_ENOMEM, "host allocation");
@@ -4262,8 +4260,8 @@ int mf_export_state(mf_graph *g, int32_t *r, int64_t *excess, int32_t *height, i
             if (rc) return rc;
         }
         try {
-            std::vector<int32_t> a, b;
-            auto out32 = [&](int32_t *dst, const int *src, const std::vector<int32_t> &at, const int *d_at) -> int {
+            HostArray<int32_t> a, b;
+            auto out32 = [&](int32_t *dst, const int *src, const auto &at, const int *d_at) -> int {
                 const long long count = (long long)at.size();
                 if (!dst || count == 0) return MF_OK;
                 if ((flags & MF_DEVICE_PTRS) && d_at) {
@@ -4291,7 +4289,7 @@ int mf_export_state(mf_graph *g, int32_t *r, int64_t *excess, int32_t *height, i
                                                                       g->d_inv, (long long)g->n);
                 MF_CUDA(cudaGetLastError());
             } else if (excess) {
-                std::vector<int64_t> e(size_t(g->n));
+                HostArray<int64_t> e(static_cast<size_t>(g->n));
                 MF_CUDA(cudaMemcpyAsync(e.data(), g->dg.e, e.size() * 8, cudaMemcpyDeviceToHost, g->last));
                 MF_CUDA(cudaStreamSynchronize(g->last));
                 for (int32_t v = 0; v < g->n; ++v) excess[v] = e[size_t(g->inv[size_t(v)])];
@@ -4320,8 +4318,8 @@ int mf_import_state(mf_graph *g, const int32_t *r, const int64_t *excess, const 
         if (rc) return rc;
         const cudaMemcpyKind in = (flags & MF_DEVICE_PTRS) ? cudaMemcpyDeviceToHost : cudaMemcpyHostToHost;
         try {
-            std::vector<int32_t> a(size_t(std::max<int64_t>(g->A, g->n))), b(a.size());
-            std::vector<int64_t> x(size_t(g->n)), y(size_t(g->n));
+            HostArray<int32_t> a(size_t(std::max<int64_t>(g->A, g->n))), b(a.size());
+            HostArray<int64_t> x(static_cast<size_t>(g->n)), y(static_cast<size_t>(g->n));
             if (g->A) {
                 MF_CUDA(cudaMemcpy(a.data(), r, size_t(g->A) * 4, in));
                 gather_i32(a.data(), g->arc_at.data(), g->A, true, b.data());
@@ -4341,21 +4339,26 @@ int mf_import_state(mf_graph *g, const int32_t *r, const int64_t *excess, const 
         MF_CUDA(cudaMemcpy(g->dg.e, excess, size_t(g->n) * 8, kind));
         MF_CUDA(cudaMemcpy(g->dg.h, height, size_t(g->n) * 4, kind));
     }
-    // rebuild the mirror rr[a] = r[rev[a]] on the host side of the copy
-    std::vector<int32_t> hr(size_t(g->A)), hrev(size_t(g->A)), hrr(size_t(g->A));
-    if (g->A) {
-        MF_CUDA(cudaMemcpy(hr.data(), g->dg.r, size_t(g->A) * 4, cudaMemcpyDeviceToHost));
-        MF_CUDA(cudaMemcpy(hrev.data(), g->dg.rev, size_t(g->A) * 4, cudaMemcpyDeviceToHost));
-        for (size_t a = 0; a < hr.size(); ++a) hrr[a] = hr[size_t(hrev[a])];
-        MF_CUDA(cudaMemcpy(g->dg.rr, hrr.data(), size_t(g->A) * 4, cudaMemcpyHostToDevice));
+    long long flow = 0;
+    try {
+        // rebuild the mirror rr[a] = r[rev[a]] on the host side of the copy
+        if (g->A) {
+            HostArray<int32_t> hr(static_cast<size_t>(g->A)), hrev(hr.size()), hrr(hr.size());
+            MF_CUDA(cudaMemcpy(hr.data(), g->dg.r, hr.size() * 4, cudaMemcpyDeviceToHost));
+            MF_CUDA(cudaMemcpy(hrev.data(), g->dg.rev, hrev.size() * 4, cudaMemcpyDeviceToHost));
+            gather_i32(hr.data(), hrev.data(), g->A, false, hrr.data());
+            MF_CUDA(cudaMemcpy(g->dg.rr, hrr.data(), hrr.size() * 4, cudaMemcpyHostToDevice));
+        }
+        // value of the imported state: e(t) plus the deficits (Alg. 4, final sum)
+        HostArray<int64_t> he(static_cast<size_t>(g->n));
+        MF_CUDA(cudaMemcpy(he.data(), g->dg.e, he.size() * 8, cudaMemcpyDeviceToHost));
+        const int32_t ds = g->dg.s, dt = g->dg.t;
+        flow = he[size_t(dt)];
+        for (int32_t v = 0; v < g->n; ++v)
+            if (v != ds && v != dt && he[size_t(v)] < 0) flow += he[size_t(v)];
+    } catch (const std::bad_alloc &) {
+        return set_err(MF_ENOMEM, "host allocation");
     }
-    // value of the imported state: e(t) plus the deficits (Alg. 4, final sum)
-    std::vector<int64_t> he(size_t(g->n));
-    MF_CUDA(cudaMemcpy(he.data(), g->dg.e, size_t(g->n) * 8, cudaMemcpyDeviceToHost));
-    const int32_t ds = g->dg.s, dt = g->dg.t;
-    long long flow = he[size_t(dt)];
-    for (int32_t v = 0; v < g->n; ++v)
-        if (v != ds && v != dt && he[size_t(v)] < 0) flow += he[size_t(v)];
     MF_CUDA(cudaMemset(g->dg.ctl, 0, sizeof(Ctl)));
     MF_CUDA(cudaMemset(g->dg.stamp, 0, size_t(std::max<int64_t>(g->m, 1)) * 4));
     MF_CUDA(cudaMemset(g->dg.astamp, 0, size_t(g->n) * 4));

@@ -85,7 +85,8 @@ int build_bicsr(int32_t n, int64_t m, const int64_t *row_ptr, const int32_t *col
 void external_arcs(int32_t n, const int32_t *row, const int32_t *head, const int32_t *ord, const int32_t *inv,
                    int32_t *ext_row, int32_t *arc_at);
 
-// dst[i] = src[at[i]], or with scatter dst[at[i]] = src[i], on several threads.
+// dst[i] = src[at[i]] (dst may be at itself), or with scatter dst[at[i]] = src[i]
+// (src null: i), on several threads.
 void gather_i32(const int32_t *src, const int32_t *at, int64_t count, bool scatter, int32_t *dst);
 
 }  // namespace mf
